@@ -21,6 +21,7 @@
 #include "bf_internal.cuh"
 #include "bf_window_fast.cuh"
 #include "bf_strip.cuh"
+#include "bf_run.cuh"
 
 int bf_apply_f32(const bf_graph* g, int op, const float* X, int64_t ldx, int k, float* Y,
                  int64_t ldy, double* dots, cudaStream_t s);
@@ -142,6 +143,37 @@ __device__ __forceinline__ void stage1(const Geom<T>& g, const Tile& t, Vec<T, 1
   }
 }
 
+// Last block of the start: the sums s^T r, s^T s, r^T r, x0^T x0 into the state.
+template <typename T>
+__device__ void cg_init_tail(const CgArgs<T>& a, const double* tot) {
+  CgState* st = a.st;
+  st->sr = tot[0];
+  st->ss = tot[1];
+  st->rr = tot[2];
+  const double b2 = (double)a.shift * (double)a.shift * tot[3];
+  st->ref2 = b2 > 0.0 ? b2 : tot[2];
+  st->beta = 0.0;
+  st->alpha = 0.0;
+  st->iter = 0;
+  st->status = (isfinite(tot[0]) && isfinite(tot[1]) && isfinite(tot[2])) ? CG_RUN : CG_NONFINITE;
+}
+
+// Last block of a direction: p^T q, the breakdown tests and alpha.
+template <typename T>
+__device__ void cg_dir_tail(const CgArgs<T>& a, double pq) {
+  CgState* st = a.st;
+  st->pq = pq;
+  if (st->sr == 0.0) {
+    st->status = CG_CONV;
+  } else if (!isfinite(pq)) {
+    st->status = CG_NONFINITE;
+  } else if (!(pq > 0.0)) {
+    st->status = CG_BREAK;
+  } else {
+    st->alpha = st->sr / pq;
+  }
+}
+
 // r = -L x0 (= b - A x0 for either system), x = x0, s = T r; sums s^T r, s^T s, r^T r, x0^T x0.
 template <typename T>
 __global__ void __launch_bounds__(BF_THREADS) k_cg_init(const Geom<T> g, const CgArgs<T> a) {
@@ -171,18 +203,7 @@ __global__ void __launch_bounds__(BF_THREADS) k_cg_init(const Geom<T> g, const C
   }
   double blk[4], tot[4];
   block_sum<4, T>(v, red, blk);
-  if (grid_sum_last<4>(blk, a.partials, &a.st->counter, tot, &last)) {
-    CgState* st = a.st;
-    st->sr = tot[0];
-    st->ss = tot[1];
-    st->rr = tot[2];
-    const double b2 = (double)a.shift * (double)a.shift * tot[3];
-    st->ref2 = b2 > 0.0 ? b2 : tot[2];
-    st->beta = 0.0;
-    st->alpha = 0.0;
-    st->iter = 0;
-    st->status = (isfinite(tot[0]) && isfinite(tot[1]) && isfinite(tot[2])) ? CG_RUN : CG_NONFINITE;
-  }
+  if (grid_sum_last<4>(blk, a.partials, &a.st->counter, tot, &last)) cg_init_tail(a, tot);
 }
 
 // p = s + beta p_old (first: p = s) on tile + halo, q = (L + shift I) p, p^T q, alpha.
@@ -214,19 +235,7 @@ __global__ void __launch_bounds__(BF_THREADS) k_cg_dir(const Geom<T> g, const Cg
   }
   double blk[1], tot[1];
   block_sum<1, T>(v, red, blk);
-  if (grid_sum_last<1>(blk, a.partials, &a.st->counter, tot, &last)) {
-    CgState* st = a.st;
-    st->pq = tot[0];
-    if (st->sr == 0.0) {
-      st->status = CG_CONV;
-    } else if (!isfinite(tot[0])) {
-      st->status = CG_NONFINITE;
-    } else if (!(tot[0] > 0.0)) {
-      st->status = CG_BREAK;
-    } else {
-      st->alpha = st->sr / tot[0];
-    }
-  }
+  if (grid_sum_last<1>(blk, a.partials, &a.st->counter, tot, &last)) cg_dir_tail(a, tot[0]);
 }
 
 // Last block of an update: record alpha/beta, beta for the next direction from
@@ -341,18 +350,7 @@ __global__ void __launch_bounds__(BF_THREADS) k_cg_init_lx(const CgArgs<T> a) {
   }
   double blk[4], tot[4];
   block_sum<4, T>(v, red, blk);
-  if (grid_sum_last<4>(blk, a.partials, &a.st->counter, tot, &last)) {
-    CgState* st = a.st;
-    st->sr = tot[0];
-    st->ss = tot[1];
-    st->rr = tot[2];
-    const double b2 = (double)a.shift * (double)a.shift * tot[3];
-    st->ref2 = b2 > 0.0 ? b2 : tot[2];
-    st->beta = 0.0;
-    st->alpha = 0.0;
-    st->iter = 0;
-    st->status = (isfinite(tot[0]) && isfinite(tot[1]) && isfinite(tot[2])) ? CG_RUN : CG_NONFINITE;
-  }
+  if (grid_sum_last<4>(blk, a.partials, &a.st->counter, tot, &last)) cg_init_tail(a, tot);
 }
 
 // p = s + beta p_old (first: p = s).
@@ -381,19 +379,7 @@ __global__ void __launch_bounds__(BF_THREADS) k_cg_pq(const CgArgs<T> a) {
   }
   double blk[1], tot[1];
   block_sum<1, T>(v, red, blk);
-  if (grid_sum_last<1>(blk, a.partials, &a.st->counter, tot, &last)) {
-    CgState* st = a.st;
-    st->pq = tot[0];
-    if (st->sr == 0.0) {
-      st->status = CG_CONV;
-    } else if (!isfinite(tot[0])) {
-      st->status = CG_NONFINITE;
-    } else if (!(tot[0] > 0.0)) {
-      st->status = CG_BREAK;
-    } else {
-      st->alpha = st->sr / tot[0];
-    }
-  }
+  if (grid_sum_last<1>(blk, a.partials, &a.st->counter, tot, &last)) cg_dir_tail(a, tot[0]);
 }
 
 // ---- specialised-window versions of k_cg_init / k_cg_dir (float graphs, common windows)
@@ -455,18 +441,7 @@ __global__ void __launch_bounds__(BF_THREADS) k_cg_init_fast(const Geom<float> g
   }
   double blk[4], tot[4];
   block_sum<4, float>(v, red, blk);
-  if (grid_sum_last<4>(blk, a.partials, &a.st->counter, tot, &last)) {
-    CgState* st = a.st;
-    st->sr = tot[0];
-    st->ss = tot[1];
-    st->rr = tot[2];
-    const double b2 = (double)a.shift * (double)a.shift * tot[3];
-    st->ref2 = b2 > 0.0 ? b2 : tot[2];
-    st->beta = 0.0;
-    st->alpha = 0.0;
-    st->iter = 0;
-    st->status = (isfinite(tot[0]) && isfinite(tot[1]) && isfinite(tot[2])) ? CG_RUN : CG_NONFINITE;
-  }
+  if (grid_sum_last<4>(blk, a.partials, &a.st->counter, tot, &last)) cg_init_tail(a, tot);
 }
 
 template <class SH, bool STORED>
@@ -510,19 +485,7 @@ __global__ void __launch_bounds__(BF_THREADS) k_cg_dir_fast(const Geom<float> g,
   }
   double blk[1], tot[1];
   block_sum<1, float>(v, red, blk);
-  if (grid_sum_last<1>(blk, a.partials, &a.st->counter, tot, &last)) {
-    CgState* st = a.st;
-    st->pq = tot[0];
-    if (st->sr == 0.0) {
-      st->status = CG_CONV;
-    } else if (!isfinite(tot[0])) {
-      st->status = CG_NONFINITE;
-    } else if (!(tot[0] > 0.0)) {
-      st->status = CG_BREAK;
-    } else {
-      st->alpha = st->sr / tot[0];
-    }
-  }
+  if (grid_sum_last<1>(blk, a.partials, &a.st->counter, tot, &last)) cg_dir_tail(a, tot[0]);
 }
 
 // ---- strip path: FP32 graphs with the 7 x 7 window, T = Jacobi or identity -----------
@@ -543,8 +506,8 @@ __global__ void __launch_bounds__(STRIP_THREADS, 2) k_cgs_init(const Geom<float>
   __shared__ int last;
   const int nx = g.nx, ny = g.ny;
   float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-  const float* src[2] = {a.x0, WM == BF_W_ONTHEFLY ? a.guide : nullptr};
-  const int64_t ld[2] = {1, 1};
+  const float* src[1] = {a.x0};
+  const int64_t ld[1] = {1};
   auto epi = [&](int bx, int by, int lx, int ly0, const float (&xi)[STRIP_P], const float (&acc)[STRIP_P]) {
     const int x = bx + lx;
 #pragma unroll
@@ -563,21 +526,10 @@ __global__ void __launch_bounds__(STRIP_THREADS, 2) k_cgs_init(const Geom<float>
       }
     }
   };
-  strip_run<WM, 2, false>(g, a.wf, a.n, src, ld, 1, [](float*) {}, epi);
+  strip_run<WM, 1, false>(g, a.wf, a.n, src, ld, [](float*) {}, epi);
   double blk[4], tot[4];
   block_sum<4, float>(v, red, blk);
-  if (grid_sum_last<4>(blk, a.partials, &a.st->counter, tot, &last)) {
-    CgState* st = a.st;
-    st->sr = tot[0];
-    st->ss = tot[1];
-    st->rr = tot[2];
-    const double b2 = (double)a.shift * (double)a.shift * tot[3];
-    st->ref2 = b2 > 0.0 ? b2 : tot[2];
-    st->beta = 0.0;
-    st->alpha = 0.0;
-    st->iter = 0;
-    st->status = (isfinite(tot[0]) && isfinite(tot[1]) && isfinite(tot[2])) ? CG_RUN : CG_NONFINITE;
-  }
+  if (grid_sum_last<4>(blk, a.partials, &a.st->counter, tot, &last)) cg_init_tail(a, tot);
 }
 
 // p = s + beta p_old (first: p = s), q = (L + shift I) p, p^T q, alpha.
@@ -590,8 +542,8 @@ __global__ void __launch_bounds__(STRIP_THREADS, 2) k_cgs_dir(const Geom<float> 
   const int nx = g.nx, ny = g.ny;
   float v[1] = {0.0f};
   const bool first = a.first != 0;
-  const float* src[3] = {a.s, first ? nullptr : a.p_old, WM == BF_W_ONTHEFLY ? a.guide : nullptr};
-  const int64_t ld[3] = {1, 1, 1};
+  const float* src[2] = {a.s, first ? nullptr : a.p_old};
+  const int64_t ld[2] = {1, 1};
   auto combine = [&](float* st) {
     if (first) return;
     for (int hp = threadIdx.x; hp < STRIP_HP; hp += STRIP_THREADS) st[hp] = fmaf(beta, st[STRIP_HP + hp], st[hp]);
@@ -610,22 +562,83 @@ __global__ void __launch_bounds__(STRIP_THREADS, 2) k_cgs_dir(const Geom<float> 
       }
     }
   };
-  strip_run<WM, 3, true>(g, a.wf, a.n, src, ld, 2, combine, epi);
+  strip_run<WM, 2, true>(g, a.wf, a.n, src, ld, combine, epi);
   double blk[1], tot[1];
   block_sum<1, float>(v, red, blk);
-  if (grid_sum_last<1>(blk, a.partials, &a.st->counter, tot, &last)) {
-    CgState* st = a.st;
-    st->pq = tot[0];
-    if (st->sr == 0.0) {
-      st->status = CG_CONV;
-    } else if (!isfinite(tot[0])) {
-      st->status = CG_NONFINITE;
-    } else if (!(tot[0] > 0.0)) {
-      st->status = CG_BREAK;
-    } else {
-      st->alpha = st->sr / tot[0];
+  if (grid_sum_last<1>(blk, a.partials, &a.st->counter, tot, &last)) cg_dir_tail(a, tot[0]);
+}
+
+// k_cgs_init and k_cgs_dir with weights on the fly, by horizontal runs (bf_run.cuh).
+static_assert(RUN_THREADS == BF_THREADS, "the block reductions assume BF_THREADS threads");
+__global__ void __launch_bounds__(RUN_THREADS, 3)
+k_cgr_init(const __grid_constant__ RunConst c, int nx, int ny, const __grid_constant__ RunSrc<2> src, int vec,
+           const CgArgs<float> a) {
+  __shared__ double red[4 * (RUN_THREADS / 32)];
+  __shared__ int last;
+  float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+  auto epi = [&](int x0, int y, const float (&xi)[RUN_P], const float (&acc)[RUN_P], const float (&)[RUN_P]) {
+    const int cnt = run_count(x0, y, nx, ny);
+    if (!cnt) return;
+    const int64_t i0 = (int64_t)y * nx + x0;
+    float sj[RUN_P], d[RUN_P];
+    if (a.dinv) run_load(a.d, i0, cnt, vec, d);
+#pragma unroll
+    for (int j = 0; j < RUN_P; ++j) {
+      if (j >= cnt) continue;
+      const float r = -acc[j];
+      sj[j] = a.dinv ? __fdiv_rn(r, d[j]) : r;
+      v[0] = fmaf(sj[j], r, v[0]);
+      v[1] = fmaf(sj[j], sj[j], v[1]);
+      v[2] = fmaf(r, r, v[2]);
+      v[3] = fmaf(xi[j], xi[j], v[3]);
     }
-  }
+    run_store(a.x, i0, cnt, vec, xi);
+    run_store(a.s, i0, cnt, vec, sj);
+  };
+  run_tiles<2, true, false, false>(c, nx, ny, src, [](float*) {}, epi);
+  double blk[4], tot[4];
+  block_sum<4, float>(v, red, blk);
+  if (grid_sum_last<4>(blk, a.partials, &a.st->counter, tot, &last)) cg_init_tail(a, tot);
+}
+
+// Bound by the FP32 pipe and the SFU (see bf_run.cuh) with 20 B per pixel beside them.
+template <bool FIRST>
+__global__ void __launch_bounds__(RUN_THREADS, 3)
+k_cgr_dir(const __grid_constant__ RunConst c, int nx, int ny, const __grid_constant__ RunSrc<FIRST ? 2 : 3> src, int vec,
+          const CgArgs<float> a) {
+  if (a.st->status != CG_RUN) return;
+  __shared__ double red[RUN_THREADS / 32];
+  __shared__ int last;
+  const float beta = (float)a.st->beta;
+  float v[1] = {0.0f};
+  auto combine = [&](float* st) {
+    for (int q = threadIdx.x; q < RUN_HP / 4; q += RUN_THREADS) {
+      float4 sv = reinterpret_cast<float4*>(st)[q];
+      const float4 po = reinterpret_cast<const float4*>(st + RUN_HP)[q];
+      sv.x = fmaf(beta, po.x, sv.x);
+      sv.y = fmaf(beta, po.y, sv.y);
+      sv.z = fmaf(beta, po.z, sv.z);
+      sv.w = fmaf(beta, po.w, sv.w);
+      reinterpret_cast<float4*>(st)[q] = sv;
+    }
+  };
+  auto epi = [&](int x0, int y, const float (&pi)[RUN_P], const float (&acc)[RUN_P], const float (&)[RUN_P]) {
+    const int cnt = run_count(x0, y, nx, ny);
+    if (!cnt) return;
+    const int64_t i0 = (int64_t)y * nx + x0;
+    float q[RUN_P];
+#pragma unroll
+    for (int j = 0; j < RUN_P; ++j) {
+      q[j] = fmaf(a.shift, pi[j], acc[j]);
+      if (j < cnt) v[0] = fmaf(pi[j], q[j], v[0]);
+    }
+    run_store(a.p_new, i0, cnt, vec, pi);
+    run_store(a.q, i0, cnt, vec, q);
+  };
+  run_tiles<FIRST ? 2 : 3, true, false, !FIRST>(c, nx, ny, src, combine, epi);
+  double blk[1], tot[1];
+  block_sum<1, float>(v, red, blk);
+  if (grid_sum_last<1>(blk, a.partials, &a.st->counter, tot, &last)) cg_dir_tail(a, tot[0]);
 }
 
 // One pixel of the update: x += alpha p, s -= alpha T q, and the four sums.
@@ -800,13 +813,68 @@ int cg_strip_loop_w(const bf_graph* g, CgArgs<float>& a, int kmax, double tol, c
   return BF_OK;
 }
 
+template <class F>
+int run_grid(const bf_graph* g, F fn, int na, int& per_sm) {
+  if (per_sm == 0) {
+    int v = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, fn, RUN_THREADS, run_smem(na)) != cudaSuccess || v < 1) v = 1;
+    per_sm = v;
+  }
+  const int64_t ntiles = (int64_t)run_tiles_x(g->nx) * run_tiles_y(g->ny);
+  return (int)std::min<int64_t>(ntiles, (int64_t)per_sm * cg_num_sms());
+}
+
+// The same loop with weights on the fly (bf_run.cuh).
+int cg_run_loop(const bf_graph* g, CgArgs<float>& a, int kmax, double tol, cudaStream_t s, float* const* pbuf) {
+  static int occ[3] = {0, 0, 0};
+  const unsigned nb_vec =
+      (unsigned)std::max<int64_t>(1, std::min<int64_t>((a.n / 4 + BF_THREADS - 1) / BF_THREADS, 8 * cg_num_sms()));
+  a.d = (const float*)g->d;
+  const RunConst c = run_const(g->gf);
+  const int nx = g->nx, ny = g->ny, vec = nx % 4 == 0;       // x, d, s, p, q are 16-byte aligned
+  RunSrc<2> s2;
+  s2.p[0] = a.x0;
+  s2.p[1] = a.guide;
+  s2.ld[0] = s2.ld[1] = 1;
+  run_src_vec(s2, nx);
+  BF_LAUNCH(k_cgr_init<<<run_grid(g, k_cgr_init, 2, occ[0]), RUN_THREADS, run_smem(2), s>>>(c, nx, ny, s2, vec, a));
+  for (int it = 0; it < kmax; ++it) {
+    a.first = (it == 0);
+    a.p_old = pbuf[it & 1];
+    a.p_new = pbuf[(it + 1) & 1];
+    if (it == 0) {
+      s2.p[0] = a.s;
+      run_src_vec(s2, nx);
+      BF_LAUNCH(k_cgr_dir<true><<<run_grid(g, k_cgr_dir<true>, 2, occ[1]), RUN_THREADS, run_smem(2), s>>>(
+          c, nx, ny, s2, vec, a));
+    } else {
+      RunSrc<3> s3;
+      s3.p[0] = a.s;
+      s3.p[1] = a.p_old;
+      s3.p[2] = a.guide;
+      s3.ld[0] = s3.ld[1] = s3.ld[2] = 1;
+      run_src_vec(s3, nx);
+      BF_LAUNCH(k_cgr_dir<false><<<run_grid(g, k_cgr_dir<false>, 3, occ[2]), RUN_THREADS, run_smem(3), s>>>(
+          c, nx, ny, s3, vec, a));
+    }
+    BF_LAUNCH(k_cgs_update<<<nb_vec, BF_THREADS, 0, s>>>(a));
+    if (tol > 0.0 && (it + 1) % CG_POLL == 0 && it + 1 < kmax) {
+      int stv = 0;
+      BF_CUDA(cudaMemcpyAsync(&stv, &a.st->status, sizeof(int), cudaMemcpyDeviceToHost, s));
+      BF_CUDA(cudaStreamSynchronize(s));
+      if (stv != CG_RUN) break;
+    }
+  }
+  return BF_OK;
+}
+
 int cg_strip_loop(const bf_graph* g, CgArgs<float>& a, int kmax, double tol, cudaStream_t s,
                   float* const* pbuf) {
   switch (g->p.weight_mode) {
     case BF_W_STORED_F32: return cg_strip_loop_w<BF_W_STORED_F32>(g, a, kmax, tol, s, pbuf);
     case BF_W_STORED_BF16: return cg_strip_loop_w<BF_W_STORED_BF16>(g, a, kmax, tol, s, pbuf);
   }
-  return cg_strip_loop_w<BF_W_ONTHEFLY>(g, a, kmax, tol, s, pbuf);
+  return cg_run_loop(g, a, kmax, tol, s, pbuf);
 }
 
 // Device buffers of one CG run: residual r, preconditioned residual s, q = A p, the two

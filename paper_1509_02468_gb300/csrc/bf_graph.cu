@@ -17,6 +17,7 @@
 #include "bf_window_fast.cuh"
 #include "bf_strip.cuh"
 #include "bf_hrun.cuh"
+#include "bf_run.cuh"
 
 // ================================================================== errors
 static thread_local std::string g_last_error;
@@ -112,6 +113,41 @@ k_weights(const Geom<T> g, const T* __restrict__ guide, int64_t n, T* d, T* dinv
   dinv[i] = T(1) / dd;
   dis[i] = T(1) / sqrt(dd);
   dls[i] = (wsum > T(1e-30)) ? T(1) / sqrt(wsum) : T(0);
+}
+
+// The degree and scalings of a float graph with the 7 x 7 window and weights on the fly, by
+// horizontal runs (bf_run.cuh); also copies the guide into the graph.  Bound by the SFU and
+// the FP32 pipe (48 exponentials and 4 x 48 lane operations per pixel) with 4 B read and
+// 20 B written per pixel beside them.
+__global__ void __launch_bounds__(RUN_THREADS, 3)
+k_weights_run(const __grid_constant__ RunConst c, int nx, int ny, const __grid_constant__ RunSrc<1> src, int vec,
+              float* guide, float* d, float* dinv, float* dis, float* dls, int* flag) {
+  auto epi = [&](int x0, int y, const float (&)[RUN_P], const float (&)[RUN_P], const float (&ws)[RUN_P]) {
+    const int cnt = run_count(x0, y, nx, ny);
+    if (!cnt) return;
+    const int64_t i0 = (int64_t)y * nx + x0;
+    float gi[RUN_P], dd[RUN_P], o[RUN_P];
+    run_load(src.p[0], i0, cnt, src.vec, gi);
+    bool bad = false;
+#pragma unroll
+    for (int j = 0; j < RUN_P; ++j) {
+      bad = bad || !isfinite(gi[j]);
+      dd[j] = 1.0f + ws[j];
+    }
+    if (bad) atomicOr(flag, 1);
+    run_store(guide, i0, cnt, vec, gi);
+    run_store(d, i0, cnt, vec, dd);
+#pragma unroll
+    for (int j = 0; j < RUN_P; ++j) o[j] = 1.0f / dd[j];
+    run_store(dinv, i0, cnt, vec, o);
+#pragma unroll
+    for (int j = 0; j < RUN_P; ++j) o[j] = 1.0f / sqrtf(dd[j]);
+    run_store(dis, i0, cnt, vec, o);
+#pragma unroll
+    for (int j = 0; j < RUN_P; ++j) o[j] = ws[j] > 1e-30f ? 1.0f / sqrtf(ws[j]) : 0.0f;
+    run_store(dls, i0, cnt, vec, o);
+  };
+  run_tiles<1, false, true, false>(c, nx, ny, src, [](float*) {}, epi);
 }
 
 // Export every window weight in canonical tap order (centre = 1, 0 off the image).
@@ -311,15 +347,55 @@ __global__ void __launch_bounds__(BF_THREADS) k_apply_fast(const Geom<float> g, 
   }
 }
 
-// One column (k = 1) through the 7 x 7 window, L-type operators (L, D^-1/2 L D^-1/2,
-// (diag L)^-1/2 L (diag L)^-1/2): strip-blocked window sums (bf_strip.cuh), persistent over
-// 32 x 32 tiles, optional fused dot x^T y.
+// One column (k = 1) through the 7 x 7 window with weights on the fly, by horizontal runs
+// (bf_run.cuh), persistent over 64 x 16 tiles: the L-type operators (SCALED: D^-1/2 L D^-1/2
+// and (diag L)^-1/2 L (diag L)^-1/2), or STEP: the BF step D^-1 W in difference form,
+// y_i = x_i - sum_j w_ij (x_i - x_j) / d_i; optional fused dot x^T y.
+template <bool SCALED, bool STEP>
+__global__ void __launch_bounds__(RUN_THREADS, 3)
+k_apply1_run(const __grid_constant__ RunConst c, int nx, int ny, const __grid_constant__ RunSrc<SCALED ? 3 : 2> src,
+             int vec_y, float* Y, int64_t ldy, double* dots) {
+  constexpr int NA = SCALED ? 3 : 2;
+  float dsum = 0.0f;
+  auto combine = [&](float* st) {           // operand of the scaled operators: x * scale
+    for (int q = threadIdx.x; q < RUN_HP; q += RUN_THREADS) st[q] *= st[RUN_HP + q];
+  };
+  auto epi = [&](int x0, int y, const float (&vi)[RUN_P], const float (&acc)[RUN_P], const float (&ws)[RUN_P]) {
+    const int cnt = run_count(x0, y, nx, ny);
+    if (!cnt) return;
+    const int64_t i0 = (int64_t)y * nx + x0;
+    float yv[RUN_P];
+#pragma unroll
+    for (int j = 0; j < RUN_P; ++j) {
+      yv[j] = acc[j];
+      if (SCALED) yv[j] *= j < cnt ? src.p[1][i0 + j] : 0.0f;
+      if (STEP) yv[j] = fmaf(-acc[j], 1.0f / (1.0f + ws[j]), vi[j]);
+      if (dots && j < cnt) dsum = fmaf(SCALED ? src.p[0][(i0 + j) * src.ld[0]] : vi[j], yv[j], dsum);
+    }
+    if (ldy == 1) {
+      run_store(Y, i0, cnt, vec_y, yv);
+    } else {
+#pragma unroll
+      for (int j = 0; j < RUN_P; ++j)
+        if (j < cnt) Y[(i0 + j) * ldy] = yv[j];
+    }
+  };
+  run_tiles<NA, true, STEP, SCALED>(c, nx, ny, src, combine, epi);
+  if (dots) {
+    const float w = warp_sum(dsum);
+    if ((threadIdx.x & 31) == 0) atomicAdd(dots, (double)w);
+  }
+}
+
+// One column (k = 1) with stored weights through the 7 x 7 window, L-type operators (L,
+// D^-1/2 L D^-1/2, (diag L)^-1/2 L (diag L)^-1/2): strip-blocked window sums (bf_strip.cuh),
+// persistent over 32 x 32 tiles, optional fused dot x^T y.
 template <int WM>
 __global__ void __launch_bounds__(STRIP_THREADS, 2) k_apply1_strip(const Geom<float> g, const ApplyArgs<float> a) {
   const int nx = g.nx, ny = g.ny;
   float dsum = 0.0f;
-  const float* src[3] = {a.X, a.scale, WM == BF_W_ONTHEFLY ? a.guide : nullptr};
-  const int64_t ld[3] = {a.ldx, 1, 1};
+  const float* src[2] = {a.X, a.scale};
+  const int64_t ld[2] = {a.ldx, 1};
   const bool scaled = a.scale != nullptr;
   auto combine = [&](float* st) {           // operand of the scaled operators: x * scale
     if (!scaled) return;
@@ -338,7 +414,7 @@ __global__ void __launch_bounds__(STRIP_THREADS, 2) k_apply1_strip(const Geom<fl
       }
     }
   };
-  strip_run<WM, 3, true>(g, a.wf, a.n, src, ld, 2, combine, epi);
+  strip_run<WM, 2, true>(g, a.wf, a.n, src, ld, combine, epi);
   if (a.dots) {
     const float w = warp_sum(dsum);
     if ((threadIdx.x & 31) == 0) atomicAdd(a.dots, (double)w);
@@ -740,7 +816,38 @@ static int launch_apply1_hrun(const bf_graph* g, const ApplyArgs<float>& a, cuda
   return BF_OK;
 }
 
-static int launch_apply1_strip_w(const bf_graph* g, const ApplyArgs<float>& a, cudaStream_t s) {
+template <bool SCALED, bool STEP>
+static int launch_apply1_run(const bf_graph* g, const ApplyArgs<float>& a, cudaStream_t s) {
+  constexpr int NA = SCALED ? 3 : 2;
+  static int per_sm = 0;
+  if (per_sm == 0) {
+    int v = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k_apply1_run<SCALED, STEP>, RUN_THREADS, run_smem(NA)) !=
+            cudaSuccess ||
+        v < 1)
+      v = 1;
+    per_sm = v;
+  }
+  RunSrc<NA> src;
+  src.p[0] = a.X;
+  src.ld[0] = a.ldx;
+  if (SCALED) {
+    src.p[1] = a.scale;
+    src.ld[1] = 1;
+  }
+  src.p[NA - 1] = a.guide;
+  src.ld[NA - 1] = 1;
+  run_src_vec(src, g->nx);
+  const int vec_y = g->nx % 4 == 0 && ((uintptr_t)a.Y & 15) == 0;
+  const int64_t ntiles = (int64_t)run_tiles_x(g->nx) * run_tiles_y(g->ny);
+  const int grid = (int)std::min<int64_t>(ntiles, (int64_t)per_sm * num_sms());
+  BF_LAUNCH(k_apply1_run<SCALED, STEP><<<grid, RUN_THREADS, run_smem(NA), s>>>(run_const(g->gf), g->nx, g->ny, src,
+                                                                             vec_y, a.Y, a.ldy, a.dots));
+  BF_CUDA(cudaGetLastError());
+  return BF_OK;
+}
+
+static int launch_apply1_w(const bf_graph* g, const ApplyArgs<float>& a, cudaStream_t s) {
   // stored weights by horizontal runs when the rows are whole 16-byte vectors of the planes
   if (g->p.weight_mode != BF_W_ONTHEFLY && g->nx % 4 == 0 && a.ldx == 1 && ((uintptr_t)g->wf & 15) == 0) {
     if (g->p.weight_mode == BF_W_STORED_BF16) return launch_apply1_hrun<BF_W_STORED_BF16>(g, a, s);
@@ -750,7 +857,7 @@ static int launch_apply1_strip_w(const bf_graph* g, const ApplyArgs<float>& a, c
     case BF_W_STORED_F32: return launch_apply1_strip<BF_W_STORED_F32>(g, a, s);
     case BF_W_STORED_BF16: return launch_apply1_strip<BF_W_STORED_BF16>(g, a, s);
   }
-  return launch_apply1_strip<BF_W_ONTHEFLY>(g, a, s);
+  return a.scale ? launch_apply1_run<true, false>(g, a, s) : launch_apply1_run<false, false>(g, a, s);
 }
 
 // Returns 1 when it launched the specialised kernel for this chunk width.
@@ -769,7 +876,11 @@ static int apply_fast_shape(const bf_graph* g, int K, const ApplyArgs<float>& a,
 static int try_apply_fast(const bf_graph* g, int K, const ApplyArgs<float>& a, cudaStream_t s, int* rc) {
   if (!(a.op == BF_OP_L || a.op == BF_OP_NSYM || a.op == BF_OP_NDIAGL || a.op == BF_OP_DINV_W)) return 0;
   if (fast_shape(g) == FAST_R3_2D && K == 1 && a.op != BF_OP_DINV_W) {
-    *rc = launch_apply1_strip_w(g, a, s);
+    *rc = launch_apply1_w(g, a, s);
+    return 1;
+  }
+  if (fast_shape(g) == FAST_R3_2D && K == 1 && g->p.weight_mode == BF_W_ONTHEFLY) {
+    *rc = launch_apply1_run<false, true>(g, a, s);
     return 1;
   }
   if (fast_shape(g) == FAST_R3_2D && !a.dots && a.op != BF_OP_DINV_W) {
@@ -997,8 +1108,29 @@ extern "C" int bf_weights(const bf_params* p, const void* guide, bf_graph** out,
 // guide value sets g->flag (which the caller clears and reads).
 static int launch_weights(bf_graph* g, const void* guide, cudaStream_t s) {
   if (g->kind == BF_KIND_GUIDED) return bf_guided_prep(g, guide, s);
-  const size_t nb = (size_t)g->n * g->esize;
   cudaError_t e;
+  if (fast_shape(g) == FAST_R3_2D && g->p.weight_mode == BF_W_ONTHEFLY) {
+    static int per_sm = 0;
+    if (per_sm == 0) {
+      int v = 0;
+      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k_weights_run, RUN_THREADS, run_smem(1)) != cudaSuccess ||
+          v < 1)
+        v = 1;
+      per_sm = v;
+    }
+    RunSrc<1> src;
+    src.p[0] = (const float*)guide;
+    src.ld[0] = 1;
+    run_src_vec(src, g->nx);
+    const int64_t ntiles = (int64_t)run_tiles_x(g->nx) * run_tiles_y(g->ny);
+    const int grid = (int)std::min<int64_t>(ntiles, (int64_t)per_sm * num_sms());
+    BF_LAUNCH(k_weights_run<<<grid, RUN_THREADS, run_smem(1), s>>>(
+        run_const(g->gf), g->nx, g->ny, src, g->nx % 4 == 0, (float*)g->guide, (float*)g->d, (float*)g->dinv,
+        (float*)g->dis, (float*)g->dls, g->flag));
+    if ((e = cudaGetLastError()) != cudaSuccess) return bf_cuda_fail(e, "k_weights_run launch");
+    return BF_OK;
+  }
+  const size_t nb = (size_t)g->n * g->esize;
   if ((e = cudaMemcpyAsync(g->guide, guide, nb, cudaMemcpyDeviceToDevice, s)) != cudaSuccess)
     return bf_cuda_fail(e, "cudaMemcpyAsync(guide)");
   const unsigned blocks = (unsigned)((g->n + BF_THREADS - 1) / BF_THREADS);
