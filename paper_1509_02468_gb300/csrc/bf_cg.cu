@@ -1,7 +1,8 @@
 // Algorithm 2 (Section 5): preconditioned CG for L x = 0 -- or the shifted system
 // (L + sigma I) x = sigma x0 -- as a polynomial filter, with the flexible beta.
 //
-// Per iteration two kernels, all scalars kept on the device in FP64:
+// Problems whose vectors fit on the chip run in one cooperative launch (bf_cgp.cu).  The
+// others take two kernels per iteration, all scalars kept on the device in FP64:
 //   k_cg_dir:    p = s + beta p on the tile and its halo, q = (L + sigma I) p (matrix-free,
 //                weights from the guide or the stored ones), block sums of p^T q, and in the
 //                last block alpha = s^T r / p^T q with the breakdown tests;
@@ -19,6 +20,7 @@
 #include <mutex>
 
 #include "bf_internal.cuh"
+#include "bf_cg.cuh"
 #include "bf_window_fast.cuh"
 #include "bf_strip.cuh"
 #include "bf_run.cuh"
@@ -44,7 +46,6 @@ int cg_num_sms() {
   return nsm;
 }
 
-enum { CG_RUN = 0, CG_CONV = 1, CG_BREAK = 2, CG_NONFINITE = 3 };
 #define CG_POLL 64
 
 // s = T r with the learned preconditioner (FP32 graphs; cg_filter checks the dtype)
@@ -68,50 +69,13 @@ inline int own_precond(const bf_cg_opts& o, const bf_graph* g, const double* r, 
   return net_precond(o.net, g, r, s, st, stop);
 }
 
-struct CgState {
-  double sr;        // s^T r of the current residual
-  double ss;        // s^T s
-  double rr;        // r^T r
-  double pq;        // p^T q
-  double alpha;
-  double beta;      // beta to use in the next direction update
-  double ref2;      // ||b||^2 (or ||r_0||^2 when b = 0)
-  double tol2;
-  int status;
-  int iter;         // completed iterations
-  int beta_mode;
-  int pad;
-  unsigned int counter;
-  unsigned int pad2;
-};
-
-template <typename T>
-struct CgArgs {
-  const T* x0;
-  T* x;
-  T* r;
-  T* s;
-  T* q;
-  const T* p_old;
-  T* p_new;
-  const T* guide;
-  const T* dinv;       // Jacobi preconditioner (NULL: identity)
-  const T* d;          // degree (the strip path divides by it)
-  const void* wf;
-  int wmode;
-  int64_t n;
-  T shift;
-  int first;           // first iteration: p = s
-  double* partials;
-  CgState* st;
-  double* hist;        // [2 kmax] or NULL
-};
-
 // The scalar state of a run, written on the device (so that a fixed-count run enqueues
 // no host-to-device copy and can be captured in a CUDA graph).  The block counter of the
-// grid reductions must start at zero.
-__global__ void k_cg_state_init(CgState* st, double tol2, int beta_mode) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// grid reductions and the exchange words of a one-launch run must start at zero.
+__global__ void __launch_bounds__(BF_THREADS) k_cg_state_init(CgState* st, double tol2, int beta_mode,
+                                                              unsigned long long* words, int nwords) {
+  for (int i = threadIdx.x; i < nwords; i += BF_THREADS) words[i] = 0ull;
+  if (threadIdx.x != 0) return;
   CgState z;
   z.sr = z.ss = z.rr = z.pq = z.alpha = z.beta = z.ref2 = 0.0;
   z.tol2 = tol2;
@@ -916,14 +880,19 @@ int cg_exec(const bf_graph* g, const T* x0, int kmax, const bf_cg_opts& o, T* x_
   a.first = 1;
   a.p_old = b.p[0];
   a.p_new = b.p[1];
-  BF_LAUNCH(k_cg_state_init<<<1, 32, 0, s>>>(a.st, o.tol > 0 ? o.tol * o.tol : 0.0, o.beta));
+  const bool net = (o.precond == BF_PRECOND_NET || o.precond == BF_PRECOND_SPD);
+  const size_t words = net ? 0 : cgp_words(g);
+  BF_LAUNCH(k_cg_state_init<<<1, BF_THREADS, 0, s>>>(a.st, o.tol > 0 ? o.tol * o.tol : 0.0, o.beta,
+                                                     (unsigned long long*)a.partials, (int)words));
   const bool one_d = (g->ny == 1 && g->ry == 0);
   const size_t hp = (size_t)((one_d ? BF_TW1 : BF_TW2) + 2 * g->rx) * ((one_d ? 1 : BF_TH2) + 2 * g->ry);
   const size_t sm = hp * 2 * sizeof(T);
-  const bool net = (o.precond == BF_PRECOND_NET || o.precond == BF_PRECOND_SPD);
   const bool guided = (g->kind == BF_KIND_GUIDED);
   int rc = BF_OK;
-  if (!guided && !net && sizeof(T) == 4 && fast_shape(g) == FAST_R3_2D && ((uintptr_t)x_out & 15) == 0) {
+  if (words) {                                     // the vectors fit on the chip: one launch
+    rc = cgp_launch<T>(g, a, kmax, s);
+    if (rc) return rc;
+  } else if (!guided && !net && sizeof(T) == 4 && fast_shape(g) == FAST_R3_2D && ((uintptr_t)x_out & 15) == 0) {
     rc = cg_strip_loop(g, reinterpret_cast<CgArgs<float>&>(a), kmax, o.tol, s,
                        reinterpret_cast<float* const*>(b.p));
     if (rc) return rc;
@@ -944,6 +913,7 @@ int cg_exec(const bf_graph* g, const T* x0, int kmax, const bf_cg_opts& o, T* x_
     info->ref = sqrt(h.ref2);
     if (h.status == CG_BREAK) return bf_fail(BF_EBREAKDOWN, std::string(who) + ": p^T q <= 0 (breakdown)");
     if (h.status == CG_NONFINITE) return bf_fail(BF_ENONFINITE, std::string(who) + ": non-finite scalar");
+    if (h.status == CG_TIMEOUT) return bf_fail(BF_ETIMEOUT, std::string(who) + ": a bounded device wait gave up");
   }
   return BF_OK;
 }
@@ -961,7 +931,8 @@ int cg_run(const bf_graph* g, const T* x0, int kmax, const bf_cg_opts& o, T* x_o
            bf_info* info, cudaStream_t s) {
   bf_graph* gm = const_cast<bf_graph*>(g);
   const size_t vb = ((size_t)g->n * sizeof(T) + 255) & ~(size_t)255;
-  const size_t pb = ((size_t)cg_partial_slots(g) * 4 * sizeof(double) + 255) & ~(size_t)255;
+  const size_t pb =
+      (std::max((size_t)cg_partial_slots(g) * 4 * sizeof(double), 8 * cgp_words(g)) + 255) & ~(size_t)255;
   int rc = bf_ws_reserve(gm, BF_WS_CG, 5 * vb + pb + 256);
   if (rc) return rc;
   char* w = (char*)gm->ws[BF_WS_CG];

@@ -239,20 +239,25 @@ __device__ __forceinline__ void run_issue(const RunConst& c, int bx, int by, int
       }
     }
   } else {
-    for (int q = threadIdx.x; q < RUN_HP; q += RUN_THREADS) {
-      const int hy = q / RUN_XS, hx = q - hy * RUN_XS;
-      const int gy = by - RUN_R + hy, gx = bx - 4 + hx;
-      const bool in = (unsigned)gx < (unsigned)nx && (unsigned)gy < (unsigned)ny;
-      const int64_t gp = in ? (int64_t)gy * nx + gx : 0;
+    for (int hy = threadIdx.x >> 5; hy < RUN_HH; hy += RUN_THREADS / 32) {
 #pragma unroll
-      for (int a = 0; a < NA; ++a) {
-        if (!src.p[a]) continue;
-        if (a == NA - 1 && !in) {
-          stage[a * RUN_HP + q] = inf;
-        } else {
-          const bool rd = in && (a < NA - 1 || c.use_guide);
-          asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(base + 4u * (unsigned)(a * RUN_HP + q)),
-                       "l"(src.p[a] + gp * src.ld[a]), "r"(rd ? 4 : 0) : "memory");
+      for (int h0 = 0; h0 < RUN_XS; h0 += 32) {
+        const int hx = h0 + (threadIdx.x & 31);
+        if (hx >= RUN_XS) continue;
+        const int q = hy * RUN_XS + hx;
+        const int gy = by - RUN_R + hy, gx = bx - 4 + hx;
+        const bool in = (unsigned)gx < (unsigned)nx && (unsigned)gy < (unsigned)ny;
+        const int64_t gp = in ? (int64_t)gy * nx + gx : 0;
+#pragma unroll
+        for (int a = 0; a < NA; ++a) {
+          if (!src.p[a]) continue;
+          if (a == NA - 1 && !in) {
+            stage[a * RUN_HP + q] = inf;
+          } else {
+            const bool rd = in && (a < NA - 1 || c.use_guide);
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(base + 4u * (unsigned)(a * RUN_HP + q)),
+                         "l"(src.p[a] + gp * src.ld[a]), "r"(rd ? 4 : 0) : "memory");
+          }
         }
       }
     }
