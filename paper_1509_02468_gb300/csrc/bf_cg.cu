@@ -71,11 +71,14 @@ inline int own_precond(const bf_cg_opts& o, const bf_graph* g, const double* r, 
 
 // The scalar state of a run, written on the device (so that a fixed-count run enqueues
 // no host-to-device copy and can be captured in a CUDA graph).  The block counter of the
-// grid reductions and the exchange words of a one-launch run must start at zero.
+// grid reductions and the exchange areas of a one-launch run must start at zero.
 __global__ void __launch_bounds__(BF_THREADS) k_cg_state_init(CgState* st, double tol2, int beta_mode,
-                                                              unsigned long long* words, int nwords) {
-  for (int i = threadIdx.x; i < nwords; i += BF_THREADS) words[i] = 0ull;
-  if (threadIdx.x != 0) return;
+                                                              unsigned long long* words, int nwords,
+                                                              ulonglong2* frames, int64_t nframes2) {
+  const int64_t t = (int64_t)blockIdx.x * BF_THREADS + threadIdx.x, nt = (int64_t)gridDim.x * BF_THREADS;
+  for (int64_t i = t; i < nwords; i += nt) words[i] = 0ull;
+  for (int64_t i = t; i < nframes2; i += nt) frames[i] = make_ulonglong2(0ull, 0ull);
+  if (t != 0) return;
   CgState z;
   z.sr = z.ss = z.rr = z.pq = z.alpha = z.beta = z.ref2 = 0.0;
   z.tol2 = tol2;
@@ -882,8 +885,12 @@ int cg_exec(const bf_graph* g, const T* x0, int kmax, const bf_cg_opts& o, T* x_
   a.p_new = b.p[1];
   const bool net = (o.precond == BF_PRECOND_NET || o.precond == BF_PRECOND_SPD);
   const size_t words = net ? 0 : cgp_words(g);
-  BF_LAUNCH(k_cg_state_init<<<1, BF_THREADS, 0, s>>>(a.st, o.tol > 0 ? o.tol * o.tol : 0.0, o.beta,
-                                                     (unsigned long long*)a.partials, (int)words));
+  // one-launch runs: 2 sizeof(T) bytes per sample from b.p[0] on (b.p[1] follows it)
+  const int64_t nframes2 = words ? ((int64_t)n * 2 * sizeof(T) + 15) / 16 : 0;
+  const unsigned nb_init = (unsigned)std::max<int64_t>(1, std::min<int64_t>(nframes2 / (4 * BF_THREADS), 4 * cg_num_sms()));
+  BF_LAUNCH(k_cg_state_init<<<nb_init, BF_THREADS, 0, s>>>(a.st, o.tol > 0 ? o.tol * o.tol : 0.0, o.beta,
+                                                           (unsigned long long*)a.partials, (int)words,
+                                                           (ulonglong2*)b.p[0], nframes2));
   const bool one_d = (g->ny == 1 && g->ry == 0);
   const size_t hp = (size_t)((one_d ? BF_TW1 : BF_TW2) + 2 * g->rx) * ((one_d ? 1 : BF_TH2) + 2 * g->ry);
   const size_t sm = hp * 2 * sizeof(T);

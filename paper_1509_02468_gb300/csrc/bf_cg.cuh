@@ -46,9 +46,10 @@ struct CgArgs {
 };
 
 // The whole run in one cooperative launch with its vectors on the chip (bf_cgp.cu).
-// cgp_words: 64-bit words of exchange area a run needs at a.partials (zeroed before the
-// launch by k_cg_state_init), 0 when the graph does not fit.  cgp_launch: BF_OK after
-// enqueuing it.
+// cgp_words: 64-bit words of exchange area a run needs at a.partials, 0 when the graph does
+// not fit; it also exchanges vector frames in a.p_old (8 bytes per sample, 16 in FP64: both
+// direction buffers, which must be contiguous).  Both areas hold zeros before the launch
+// (k_cg_state_init).  cgp_launch: BF_OK after enqueuing it.
 size_t cgp_words(const bf_graph* g);
 template <typename T>
 int cgp_launch(const bf_graph* g, const CgArgs<T>& a, int kmax, cudaStream_t s);

@@ -7,15 +7,17 @@
 // iteration: two kernels, each with a launch, a cold staging of its tiles and a last-block
 // reduction (14 + 12 us per iteration at 512 x 512 against 1.6 us of arithmetic).  Here an
 // iteration is
-//   p = s + beta p on the rectangle and its halo (the neighbours' s is read from L2),
+//   p = s + beta p on the rectangle and its halo (the neighbours' s comes through L2),
 //   q = (L + sigma I) p, p^T q  ->  all-reduce, alpha,
-//   x += alpha p, s -= alpha T q, the four sums, the frame of s to L2  ->  all-reduce, beta,
-// and the all-reduces are the only grid-wide synchronisation: every CTA writes its partial
-// sums to a slot of its own and reads all slots, so the sums come with the barrier (one
-// write and one polled read of L2 instead of an atomic, a poll and a read).  A double is
-// sent as two 64-bit words {epoch, half}, each of which is written and read whole, so a word
-// with the awaited epoch carries its data.  All CTAs add the partials in the same order and
-// take the same decisions.
+//   x += alpha p, s -= alpha T q, the four sums, the frame of s to L2  ->  all-reduce, beta.
+// Nothing else synchronises the grid, and nothing needs a fence: what a CTA sends (partial
+// sums, frame values) goes out as 64-bit words {epoch, 32 data bits}, each written and read
+// whole, and the receiver polls the word until it carries the awaited epoch.  So an
+// all-reduce is one write and one polled read of L2, and the halo words, written before it,
+// are there when it is done.  (With plain stores, a fence on either side and FP64 additions
+// the two all-reduces of an iteration took 17 of its 27 thousand cycles at 512 x 512.)
+// All CTAs add the partials alike and take the same decisions; the scalar recurrences are
+// in FP64.
 //
 // Every wait is bounded (1 s by %globaltimer): a CTA that gives up sets the status to
 // CG_TIMEOUT; the others see it and leave too.
@@ -30,20 +32,11 @@ namespace {
 
 #define CGP_T 512                          // threads of an image CTA
 #define CGP_TL 256                         // threads of a signal CTA
-#define CGP_SLOT 8                         // words of a CTA's slot (four doubles)
+#define CGP_SLOT 16                        // words of a CTA's slot: a line of L2 of its own
 #define CGP_MAXC 256                       // most CTAs of a launch
 #define CGP_WAIT_NS 1000000000ull
 #define CGP_HALO_REGS 4                    // halo pixels a thread can own
 typedef unsigned long long u64;
-
-// Words {epoch, payload} of the all-reduce and the scalars every CTA computes for itself.
-struct CgpShared {
-  double red[4][CGP_T / 32];
-  double tot[4];
-  double alpha, beta;
-  double sr, ss, rr, ref2;
-  int status;
-};
 
 __device__ __forceinline__ u64 cgp_now() {
   u64 t;
@@ -51,21 +44,149 @@ __device__ __forceinline__ u64 cgp_now() {
   return t;
 }
 
-// a / b by an FP32 seed and Newton steps in FP64 (a divide is twice as long a chain); the
-// last step corrects the quotient, so it is right to the last bit or two.  Values the seed
-// cannot hold take the divide.
-__device__ __forceinline__ double cgp_div(double a, double b) {
-  const double ab = fabs(b);
-  if (!(ab > 1e-30 && ab < 1e30)) return a / b;
-  double r = (double)__frcp_rn((float)b);
-  r = fma(r, fma(-b, r, 1.0), r);
-  r = fma(r, fma(-b, r, 1.0), r);
-  const double q = a * r;
-  return fma(r, fma(-b, q, a), q);
+// ---- words in flight
+__device__ __forceinline__ u64 cgp_word(unsigned epoch, unsigned data) { return ((u64)epoch << 32) | data; }
+__device__ __forceinline__ void cgp_put(u64* p, u64 w) {
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(w) : "memory");
+}
+__device__ __forceinline__ u64 cgp_get(const u64* p) {
+  u64 w;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(p) : "memory");
+  return w;
+}
+__device__ __forceinline__ void cgp_get2(const u64* p, u64& a, u64& b) {
+  asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+}
+// One more look at the clock and at the others: whether to give up waiting.
+__device__ bool cgp_give_up(u64 t0, CgState* st) {
+  if (*(volatile int*)&st->status == CG_TIMEOUT) return true;
+  if (cgp_now() - t0 <= CGP_WAIT_NS) return false;
+  atomicExch(&st->status, CG_TIMEOUT);
+  return true;
+}
+// Poll a word (a pair of words) until it carries `epoch`; false: gave up.
+__device__ bool cgp_wait(const u64* p, u64& w, unsigned epoch, CgState* st) {
+  const u64 t0 = cgp_now();
+  for (unsigned n = 1;; ++n) {
+    w = cgp_get(p);
+    if ((unsigned)(w >> 32) == epoch) return true;
+    if (n % 64 == 0 && cgp_give_up(t0, st)) return false;
+  }
+}
+__device__ bool cgp_wait2(const u64* p, u64& a, u64& b, unsigned epoch, CgState* st) {
+  const u64 t0 = cgp_now();
+  for (unsigned n = 1;; ++n) {
+    cgp_get2(p, a, b);
+    if ((unsigned)(a >> 32) == epoch && (unsigned)(b >> 32) == epoch) return true;
+    if (n % 64 == 0 && cgp_give_up(t0, st)) return false;
+  }
 }
 
-// Warp sums of four values at once: 6 additions instead of 20 (an FP64 instruction holds
-// the scheduler's FP64 pipe for 64 cycles); value ((lane >> 3) & 3) is returned in a lane.
+// ---- sums and scalars
+// A dependent FP64 addition takes about 115 cycles here and holds its scheduler's pipe for
+// 64, so FP32 runs carry their sums and scalars as unevaluated pairs of floats h + l (48 bits;
+// the terms are FP32 warp sums): an addition is a chain of six 4-cycle operations.  The pairs
+// are scaled by a power of two taken from the start's sums (which are FP64), so they do not
+// leave the FP32 range where the FP64 sums would not.  FP64 runs use FP64.
+struct CgpPair {
+  float h, l;
+};
+__device__ __forceinline__ CgpPair cgp_add(CgpPair a, CgpPair b) {
+  const float s = a.h + b.h, t = s - a.h;
+  return {s, ((a.h - (s - t)) + (b.h - t)) + (a.l + b.l)};
+}
+__device__ __forceinline__ double cgp_add(double a, double b) { return a + b; }
+__device__ __forceinline__ CgpPair cgp_shfl(CgpPair a, int o) {
+  return {__shfl_xor_sync(0xffffffffu, a.h, o), __shfl_xor_sync(0xffffffffu, a.l, o)};
+}
+__device__ __forceinline__ double cgp_shfl(double a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
+__device__ __forceinline__ void cgp_from(float x, CgpPair& r) { r = {x, 0.0f}; }
+__device__ __forceinline__ void cgp_from(double x, double& r) { r = x; }
+__device__ __forceinline__ void cgp_from(float x, double& r) { r = (double)x; }
+__device__ __forceinline__ CgpPair cgp_norm(CgpPair a) {
+  const float s = a.h + a.l;
+  return {s, a.l - (s - a.h)};
+}
+__device__ __forceinline__ double cgp_norm(double a) { return a; }
+// the two words of a value in flight
+__device__ __forceinline__ unsigned cgp_half(CgpPair a, int i) { return __float_as_uint(i ? a.l : a.h); }
+__device__ __forceinline__ unsigned cgp_half(double a, int i) {
+  const u64 b = (u64)__double_as_longlong(a);
+  return i ? (unsigned)(b >> 32) : (unsigned)b;
+}
+__device__ __forceinline__ void cgp_join(unsigned w0, unsigned w1, CgpPair& r) {
+  r = {__uint_as_float(w0), __uint_as_float(w1)};
+}
+__device__ __forceinline__ void cgp_join(unsigned w0, unsigned w1, double& r) {
+  r = __longlong_as_double((long long)(((u64)w1 << 32) | w0));
+}
+__device__ __forceinline__ CgpPair cgp_div(CgpPair a, CgpPair b) {
+  const float r = __frcp_rn(b.h), q = a.h * r;
+  const float rem = fmaf(-q, b.h, a.h) + fmaf(-q, b.l, a.l);
+  return cgp_norm({q, rem * r});
+}
+// FP32 seed (error below 2^-22), one cubic step in FP64; a divisor outside the seed's range
+// takes the divide.
+__device__ __forceinline__ double cgp_div(double a, double b) {
+  const int e = (int)((__double_as_longlong(b) >> 52) & 0x7ff);
+  if (e < 1023 - 100 || e > 1023 + 100) return a / b;
+  const double r = (double)__frcp_rn((float)b);
+  const double d = fma(-b, r, 1.0);
+  return a * fma(r, fma(d, d, d), r);
+}
+__device__ __forceinline__ CgpPair cgp_mul(CgpPair a, CgpPair b) {
+  const float p = a.h * b.h;
+  return cgp_norm({p, fmaf(a.h, b.h, -p) + fmaf(a.h, b.l, a.l * b.h)});
+}
+__device__ __forceinline__ double cgp_mul(double a, double b) { return a * b; }
+__device__ __forceinline__ CgpPair cgp_neg(CgpPair a) { return {-a.h, -a.l}; }
+__device__ __forceinline__ double cgp_neg(double a) { return -a; }
+__device__ __forceinline__ bool cgp_finite(CgpPair a) { return isfinite(a.h) && isfinite(a.l); }
+__device__ __forceinline__ bool cgp_finite(double a) { return ((__double_as_longlong(a) >> 52) & 0x7ff) != 0x7ff; }
+__device__ __forceinline__ bool cgp_zero(CgpPair a) { return a.h == 0.0f; }
+__device__ __forceinline__ bool cgp_zero(double a) { return (__double_as_longlong(a) << 1) == 0; }
+__device__ __forceinline__ bool cgp_negative(CgpPair a) { return a.h < 0.0f; }
+__device__ __forceinline__ bool cgp_negative(double a) { return __double_as_longlong(a) < 0; }
+__device__ __forceinline__ double cgp_double(CgpPair a) { return (double)a.h + (double)a.l; }
+__device__ __forceinline__ double cgp_double(double a) { return a; }
+__device__ __forceinline__ void cgp_set(double x, CgpPair& r) {
+  r.h = (float)x;
+  r.l = (float)(x - (double)r.h);
+}
+__device__ __forceinline__ void cgp_set(double x, double& r) { r = x; }
+__device__ __forceinline__ float cgp_value(CgpPair a) { return a.h; }
+__device__ __forceinline__ double cgp_value(double a) { return a; }
+
+template <typename T> struct CgpNum;
+template <> struct CgpNum<float> { typedef CgpPair type; };
+template <> struct CgpNum<double> { typedef double type; };
+
+// What a CTA's threads share: the sums in flight (N) and the scalars of the run, which one
+// warp each computes (64 cycles of a scheduler per FP64 instruction and warp) for the others.
+template <typename T>
+struct CgpShared {
+  typedef typename CgpNum<T>::type N;
+  union {
+    double d[4][CGP_T / 32];
+    N n[4][CGP_T / 32];
+  } red;
+  union {                                  // the CTAs' partial sums, [CTA][value]
+    double d[CGP_MAXC * 4];
+    N n[CGP_MAXC * 4];
+  } part;
+  double tot[4];                           // start: the four sums
+  N sr, ss, rr, alpha, beta, cb;           // scaled by `scale`, except the quotients
+  double ref2, thr;                        // thr: scaled tol^2 ref^2
+  float scale;                             // FP32 runs: of the sums (a power of two)
+  int fin[4], conv, status;
+};
+template <typename T> __device__ __forceinline__ auto cgp_red(CgpShared<T>& sh, double*) -> decltype((sh.red.d)) { return sh.red.d; }
+__device__ __forceinline__ auto cgp_red(CgpShared<float>& sh, CgpPair*) -> decltype((sh.red.n)) { return sh.red.n; }
+template <typename T> __device__ __forceinline__ double* cgp_part(CgpShared<T>& sh, double*) { return sh.part.d; }
+__device__ __forceinline__ CgpPair* cgp_part(CgpShared<float>& sh, CgpPair*) { return sh.part.n; }
+
+// Warp sums of four values at once, value ((lane >> 3) & 3) in a lane: 6 additions and
+// shuffles instead of 20.
 template <typename T>
 __device__ __forceinline__ T cgp_warp4(const T (&v)[4], int lane) {
   const bool h16 = lane & 16, h8 = lane & 8;
@@ -79,112 +200,163 @@ __device__ __forceinline__ T cgp_warp4(const T (&v)[4], int lane) {
   return c;
 }
 
-// Sums of v over all threads of all CTAs into sh.tot (valid in warps 0 .. NV - 1, value w in
-// warp w, lane 0 writes it); a barrier of the grid.  Returns false (in every thread) when a
-// wait gave up.  The caller synchronises the CTA before using sh.tot in other warps.
-template <int NV, int NT, typename T>
-__device__ bool cgp_allreduce(const T (&v)[4], CgpShared& sh, unsigned* words, u64* slots, unsigned epoch,
-                              CgState* st) {
+// Sums of v (times scale) over all threads of all CTAs, and a barrier of the grid.  Warp
+// w < NV gets the total of value w and calls tail(w, total) with all its lanes; what tail
+// writes to shared memory is visible to every thread on return.  `during` runs while the
+// words of the other CTAs are on their way.  R: representation of the sums.  Returns false
+// (in every thread) when a wait gave up.
+template <int NV, int NT, typename R, typename T, class During, class Tail>
+__device__ __forceinline__ bool cgp_allreduce(const T (&v)[4], T scale, CgpShared<T>& sh, u64* slots, unsigned epoch,
+                                              CgState* st, During during, Tail tail) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nc = gridDim.x;
   u64* base = slots + (size_t)(epoch & 1) * CGP_MAXC * CGP_SLOT;
+  auto& red = cgp_red(sh, (R*)nullptr);
+  R* part = cgp_part(sh, (R*)nullptr);
   if (NV == 4) {
     const T w = cgp_warp4<T>(v, lane);
-    if ((lane & 7) == 0) sh.red[lane >> 3][wid] = (double)w;
+    if ((lane & 7) == 0) cgp_from(w * scale, red[lane >> 3][wid]);
   } else {
     const T w = warp_sum(v[0]);
-    if (lane == 0) sh.red[0][wid] = (double)w;
+    if (lane == 0) cgp_from(w * scale, red[0][wid]);
   }
   __syncthreads();
   if (wid < NV) {
-    double t = lane < NT / 32 ? sh.red[wid][lane] : 0.0;
+    R t = red[wid][lane & (NT / 32 - 1)];
 #pragma unroll
-    for (int o = NT / 64; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    if (lane < 2) {
-      const u64 bits = (u64)__double_as_longlong(t);
-      const u64 word = ((u64)epoch << 32) | (lane ? (bits >> 32) : (bits & 0xffffffffull));
-      __threadfence();                     // the CTA's stores before the barrier above come first
-      *(volatile u64*)(base + blockIdx.x * CGP_SLOT + 2 * wid + lane) = word;
+    for (int o = NT / 64; o > 0; o >>= 1) t = cgp_add(t, cgp_shfl(t, o));
+    t = cgp_norm(t);
+    if (lane < 2) cgp_put(base + blockIdx.x * CGP_SLOT + 2 * wid + lane, cgp_word(epoch, cgp_half(t, lane)));
+  }
+  during();
+  // read every CTA's words: first all of this thread's loads, then wait for what is missing
+  constexpr int K = (CGP_MAXC * NV + NT - 1) / NT;
+  u64 lo[K], hi[K];
+  bool ok = true;
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const int w = threadIdx.x + k * NT;
+    if (w < nc * NV) cgp_get2(base + (w / NV) * CGP_SLOT + 2 * (w % NV), lo[k], hi[k]);
+  }
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const int w = threadIdx.x + k * NT;
+    if (w < nc * NV && ok) {
+      const u64* p = base + (w / NV) * CGP_SLOT + 2 * (w % NV);
+      if ((unsigned)(lo[k] >> 32) != epoch || (unsigned)(hi[k] >> 32) != epoch) ok = cgp_wait2(p, lo[k], hi[k], epoch, st);
+      cgp_join((unsigned)lo[k], (unsigned)hi[k], part[w]);
     }
   }
-  // read every CTA's words of these NV values
-  int bad = 0;
-  for (int w = threadIdx.x; w < nc * 2 * NV; w += NT) {
-    const volatile u64* p = base + (w / (2 * NV)) * CGP_SLOT + (w % (2 * NV));
-    u64 word = *p;
-    if ((unsigned)(word >> 32) != epoch) {
-      const u64 t0 = cgp_now();
-      for (;;) {
-        word = *p;
-        if ((unsigned)(word >> 32) == epoch) break;
-        if (*(volatile int*)&st->status == CG_TIMEOUT) { bad = 1; break; }
-        if (cgp_now() - t0 > CGP_WAIT_NS) {
-          atomicExch(&st->status, CG_TIMEOUT);
-          bad = 1;
-          break;
-        }
-      }
-      if (bad) break;
-    }
-    words[w] = (unsigned)word;
-  }
-  __threadfence();                         // later reads see what the others wrote before
-  if (__syncthreads_or(bad)) return false;
+  if (__syncthreads_or(!ok)) return false;
   if (wid < NV) {
-    double t = 0.0;
-    for (int c = lane; c < nc; c += 32) {
-      const unsigned* p = words + c * 2 * NV + 2 * wid;
-      t += __longlong_as_double((long long)(((u64)p[1] << 32) | p[0]));
+    R x[CGP_MAXC / 32];
+#pragma unroll
+    for (int k = 0; k < CGP_MAXC / 32; ++k) {
+      const int c = lane + 32 * k;
+      cgp_from(T(0), x[k]);
+      if (c < nc) x[k] = part[c * NV + wid];
     }
-    t = warp_sum(t);
-    if (lane == 0) sh.tot[wid] = t;
+#pragma unroll
+    for (int h = 1; h < CGP_MAXC / 32; h <<= 1)
+#pragma unroll
+      for (int k = 0; k + h < CGP_MAXC / 32; k += 2 * h)
+        if (32 * (k + h) < nc) x[k] = cgp_add(x[k], x[k + h]);
+    R t = x[0];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t = cgp_add(t, cgp_shfl(t, o));
+    tail(wid, cgp_norm(t));
   }
+  __syncthreads();
   return true;
 }
 
-// The scalar steps, by thread 0 of every CTA (all take the same values); CTA 0 keeps the
-// history.  Start: the state from the sums s^T r, s^T s, r^T r, x0^T x0.
-__device__ void cgp_start_scalars(CgpShared& sh, double shift) {
-  sh.sr = sh.tot[0];
-  sh.ss = sh.tot[1];
-  sh.rr = sh.tot[2];
-  const double b2 = shift * shift * sh.tot[3];
-  sh.ref2 = b2 > 0.0 ? b2 : sh.tot[2];
-  sh.alpha = sh.beta = 0.0;
-  sh.status = (isfinite(sh.tot[0]) && isfinite(sh.tot[1]) && isfinite(sh.tot[2])) ? CG_RUN : CG_NONFINITE;
-}
-// Direction: p^T q in tot[0].
-__device__ void cgp_dir_scalars(CgpShared& sh) {
-  const double pq = sh.tot[0];
-  if (sh.sr == 0.0) sh.status = CG_CONV;
-  else if (!isfinite(pq)) sh.status = CG_NONFINITE;
-  else if (!(pq > 0.0)) sh.status = CG_BREAK;
-  else sh.alpha = cgp_div(sh.sr, pq);
-}
-// Update: s^T r, s^T q, s^T s, r^T r.
-__device__ void cgp_update_scalars(CgpShared& sh, int it, int beta_mode, double tol2, double* hist) {
-  if (hist && blockIdx.x == 0) {
-    hist[2 * it] = sh.alpha;
-    hist[2 * it + 1] = it == 0 ? 0.0 : sh.beta;
+// ---- the scalar steps (tails of the all-reduces; every CTA takes the same ones)
+// Start: s^T r, s^T s, r^T r, x0^T x0 in sh.tot; by every thread, after the all-reduce.
+template <typename T>
+__device__ void cgp_start(CgpShared<T>& sh, double shift, double tol2) {
+  if (threadIdx.x == 0) {
+    const double sr = sh.tot[0], ss = sh.tot[1], rr = sh.tot[2];
+    sh.status = (cgp_finite(sr) && cgp_finite(ss) && cgp_finite(rr)) ? CG_RUN : CG_NONFINITE;
+    const double b2 = shift * shift * sh.tot[3];
+    sh.ref2 = b2 > 0.0 ? b2 : rr;
+    double sc = 1.0;
+    if (sizeof(T) == 4) {                      // 2^-exponent of the largest sum, within 2^+-120
+      const double m = fmax(fmax(fabs(sr), ss), rr);
+      const int e = (int)((__double_as_longlong(m) >> 52) & 0x7ff) - 1023;
+      const int k = max(-120, min(120, -e));
+      sh.scale = __uint_as_float((unsigned)(127 + k) << 23);
+      sc = (double)sh.scale;
+    } else {
+      sh.scale = 1.0f;
+    }
+    cgp_set(sr * sc, sh.sr);
+    cgp_set(ss * sc, sh.ss);
+    cgp_set(rr * sc, sh.rr);
+    sh.thr = tol2 > 0.0 ? tol2 * sh.ref2 * sc : -1.0;
+    cgp_set(0.0, sh.alpha);
+    cgp_set(0.0, sh.beta);
   }
-  const double den = beta_mode == BF_BETA_PRINTED ? sh.ss : sh.sr;
-  sh.beta = cgp_div(-sh.alpha * sh.tot[1], den);
-  sh.sr = sh.tot[0];
-  sh.ss = sh.tot[2];
-  sh.rr = sh.tot[3];
-  if (!(isfinite(sh.tot[0]) && isfinite(sh.tot[1]) && isfinite(sh.tot[2]) && isfinite(sh.tot[3])))
-    sh.status = CG_NONFINITE;
-  else if (tol2 > 0.0 && sh.tot[3] <= tol2 * sh.ref2)
-    sh.status = CG_CONV;
+  __syncthreads();
 }
-__device__ void cgp_write_state(const CgpShared& sh, CgState* st, int iters) {
-  st->sr = sh.sr;
-  st->ss = sh.ss;
-  st->rr = sh.rr;
+// Direction (warp 0): p^T q -> the breakdown tests and alpha.
+template <typename T>
+__device__ __forceinline__ void cgp_direction(CgpShared<T>& sh, typename CgpNum<T>::type pq, int lane) {
+  int status = CG_RUN;
+  const typename CgpNum<T>::type sr = sh.sr;
+  if (cgp_zero(sr)) status = CG_CONV;
+  else if (!cgp_finite(pq)) status = CG_NONFINITE;
+  else if (cgp_zero(pq) || cgp_negative(pq)) status = CG_BREAK;
+  const typename CgpNum<T>::type alpha = cgp_div(sr, pq);
+  if (lane == 0) {
+    sh.status = status;
+    if (status == CG_RUN) sh.alpha = alpha;
+  }
+}
+// beta's factor -alpha / (s^T r or s^T s), by the last warp beside the update.
+template <typename T>
+__device__ __forceinline__ void cgp_prepare_beta(CgpShared<T>& sh, int beta_mode) {
+  if (threadIdx.x == blockDim.x - 1)
+    sh.cb = cgp_neg(cgp_div(sh.alpha, beta_mode == BF_BETA_PRINTED ? sh.ss : sh.sr));
+}
+// Update (warps 0 .. 3): s^T r, s^T q, s^T s, r^T r -> beta and the stopping tests.
+template <typename T>
+__device__ __forceinline__ void cgp_update_tail(CgpShared<T>& sh, int w, typename CgpNum<T>::type t, int lane) {
+  typename CgpNum<T>::type b = t;
+  if (w == 1) b = cgp_mul(sh.cb, t);
+  if (lane != 0) return;
+  sh.fin[w] = cgp_finite(t);
+  if (w == 0) sh.sr = t;
+  else if (w == 1) sh.beta = b;
+  else if (w == 2) sh.ss = t;
+  else {
+    sh.rr = t;
+    sh.conv = sh.thr >= 0.0 && cgp_double(t) <= sh.thr;
+  }
+}
+// After the update's all-reduce, by every thread: the status.
+template <typename T>
+__device__ __forceinline__ int cgp_status(const CgpShared<T>& sh) {
+  if (!(sh.fin[0] & sh.fin[1] & sh.fin[2] & sh.fin[3])) return CG_NONFINITE;
+  return sh.conv ? CG_CONV : CG_RUN;
+}
+template <typename T>
+__device__ void cgp_history(const CgpShared<T>& sh, double* hist, int it) {
+  if (hist && blockIdx.x == 0 && threadIdx.x == blockDim.x - 1) {   // beta: before this update
+    hist[2 * it] = cgp_double(sh.alpha);
+    hist[2 * it + 1] = it == 0 ? 0.0 : cgp_double(sh.beta);
+  }
+}
+template <typename T>
+__device__ void cgp_write_state(const CgpShared<T>& sh, CgState* st, int iters, int status) {
+  if (blockIdx.x != 0 || threadIdx.x != 0) return;
+  const double inv = 1.0 / (double)sh.scale;
+  st->sr = cgp_double(sh.sr) * inv;
+  st->ss = cgp_double(sh.ss) * inv;
+  st->rr = cgp_double(sh.rr) * inv;
   st->ref2 = sh.ref2;
-  st->alpha = sh.alpha;
-  st->beta = sh.beta;
+  st->alpha = cgp_double(sh.alpha);
+  st->beta = cgp_double(sh.beta);
   st->iter = iters;
-  atomicCAS(&st->status, CG_RUN, sh.status);    // a timeout recorded by another CTA stays
+  atomicCAS(&st->status, CG_RUN, status);      // a timeout recorded by another CTA stays
 }
 
 // ---------------------------------------------------------------- images
@@ -224,7 +396,8 @@ struct CgpImage {
   CgArgs<float> cg;
   CgpRect rc;
   int nx, ny, kmax, vec;
-  u64* slots;
+  u64* slots;                // [2][CGP_MAXC][CGP_SLOT], by epoch parity
+  u64* frames;               // [n]: s of the rectangles' frames
 };
 
 template <class OP>
@@ -254,8 +427,8 @@ template <class OP>
 __global__ void __launch_bounds__(CGP_T, 1) k_cgp_image(const __grid_constant__ OP op, const __grid_constant__ CgpImage a) {
   constexpr int HALO = OP::HALO, LP = OP::LP;
   extern __shared__ __align__(16) float cgp_smem[];
-  __shared__ CgpShared sh;
-  __shared__ unsigned words[CGP_MAXC * CGP_SLOT];
+  typedef CgpPair N;
+  __shared__ CgpShared<float> sh;
   const int W = a.rc.W, H = a.rc.H, xs = W + 2 * LP;
   const int nx = a.nx, ny = a.ny;
   float* P = cgp_smem;
@@ -284,10 +457,44 @@ __global__ void __launch_bounds__(CGP_T, 1) k_cgp_image(const __grid_constant__ 
     D[q] = (bx + x < nx && by + y < ny) ? a.cg.d[(int64_t)(by + y) * nx + bx + x] : 1.0f;
   }
   __syncthreads();
-  // a run's values of s to the frame that the neighbours read
-  auto frame = [&](int x, int y, int cnt, const float (&s)[RUN_P]) {
-    if (x < 8 || x >= W - 8 || y < HALO || y >= H - HALO)
-      run_store(a.cg.s, (int64_t)(by + y) * nx + bx + x, cnt, a.vec, s);
+  // a run's values of s that the neighbours read
+  auto frame = [&](int x, int y, int cnt, const float (&s)[RUN_P], unsigned tag) {
+    const bool rows = y < HALO || y >= H - HALO;
+    u64* f = a.frames + (int64_t)(by + y) * nx + bx + x;
+#pragma unroll
+    for (int j = 0; j < RUN_P; ++j)
+      if (j < cnt && (rows || x + j < HALO || x + j >= W - HALO)) cgp_put(f + j, cgp_word(tag, __float_as_uint(s[j])));
+  };
+  // this thread's halo pixels: tile offset, and index in the image (-1: none or outside)
+  const int nhalo = 2 * HALO * (W + 2 * HALO) + 2 * HALO * H;
+  int htile[CGP_HALO_REGS], himg[CGP_HALO_REGS];
+  u64 hw[CGP_HALO_REGS];
+#pragma unroll
+  for (int k = 0; k < CGP_HALO_REGS; ++k) {
+    const int h = threadIdx.x + k * CGP_T;
+    himg[k] = htile[k] = -1;
+    hw[k] = 0ull;
+    if (h < nhalo) {
+      int tx, ty;
+      cgp_halo_pos<HALO>(h, W, H, tx, ty);
+      const int gx = bx + tx, gy = by + ty;
+      htile[k] = (ty + HALO) * xs + tx + LP;
+      if ((unsigned)gx < (unsigned)nx && (unsigned)gy < (unsigned)ny) himg[k] = gy * nx + gx;
+    }
+  }
+  // the halo words: loads issued ...
+  auto halo_get = [&]() {
+#pragma unroll
+    for (int k = 0; k < CGP_HALO_REGS; ++k)
+      if (himg[k] >= 0) hw[k] = cgp_get(a.frames + himg[k]);
+  };
+  // ... and awaited
+  auto halo_wait = [&](unsigned tag) {
+    bool ok = true;
+#pragma unroll
+    for (int k = 0; k < CGP_HALO_REGS; ++k)
+      if (himg[k] >= 0 && (unsigned)(hw[k] >> 32) != tag && ok) ok = cgp_wait(a.frames + himg[k], hw[k], tag, a.cg.st);
+    return ok;
   };
   // ---- r = -L x0, s = T r
   unsigned epoch = 1;
@@ -313,32 +520,19 @@ __global__ void __launch_bounds__(CGP_T, 1) k_cgp_image(const __grid_constant__ 
       }
       *reinterpret_cast<float4*>(S + y * W + x) = make_float4(s[0], s[1], s[2], s[3]);
       *reinterpret_cast<float4*>(X + y * W + x) = make_float4(xi[0], xi[1], xi[2], xi[3]);
-      if (cnt) frame(x, y, cnt, s);
+      if (cnt) frame(x, y, cnt, s, 1u);
     }
-    if (!cgp_allreduce<4, CGP_T>(v, sh, words, a.slots, epoch, a.cg.st)) return;
-    __syncthreads();
-    if (threadIdx.x == 0) cgp_start_scalars(sh, (double)a.cg.shift);
-    __syncthreads();
+    if (!cgp_allreduce<4, CGP_T, double>(v, 1.0f, sh, a.slots, epoch, a.cg.st, halo_get, [&](int w, double t) {
+          if (lane == 0) sh.tot[w] = t;
+        }))
+      return;
+    cgp_start(sh, (double)a.cg.shift, tol2);
   }
-  // this thread's halo pixels: offset in the image (-1: outside) and in the tile
-  const int nhalo = 2 * HALO * (W + 2 * HALO) + 2 * HALO * H;
-  int it = 0;
-  for (; it < a.kmax && sh.status == CG_RUN; ++it) {
-    const float beta = it ? (float)sh.beta : 0.0f;
+  int it = 0, status = sh.status;
+  const float scale = sh.scale;
+  for (; it < a.kmax && status == CG_RUN; ++it) {
+    const float beta = cgp_value(sh.beta);     // 0 before the first step
     // ---- p = s + beta p
-    float hs[CGP_HALO_REGS];
-#pragma unroll
-    for (int k = 0; k < CGP_HALO_REGS; ++k) {
-      const int h = threadIdx.x + k * CGP_T;
-      hs[k] = 0.0f;
-      if (h < nhalo) {
-        int tx, ty;
-        cgp_halo_pos<HALO>(h, W, H, tx, ty);
-        const int gx = bx + tx, gy = by + ty;
-        if ((unsigned)gx < (unsigned)nx && (unsigned)gy < (unsigned)ny)
-          hs[k] = __ldcg(a.cg.s + (int64_t)gy * nx + gx);
-      }
-    }
     for (int u = wid; u < nunits; u += CGP_T / 32) {
       const int x = (u % ux_n) * 32 + rx, y = (u / ux_n) * 4 + ry;
       const float4 s = *reinterpret_cast<const float4*>(S + y * W + x);
@@ -353,17 +547,14 @@ __global__ void __launch_bounds__(CGP_T, 1) k_cgp_image(const __grid_constant__ 
       }
       *pp = p;
     }
+    const bool ok = halo_wait((unsigned)it + 1u);
 #pragma unroll
-    for (int k = 0; k < CGP_HALO_REGS; ++k) {
-      const int h = threadIdx.x + k * CGP_T;
-      if (h < nhalo) {
-        int tx, ty;
-        cgp_halo_pos<HALO>(h, W, H, tx, ty);
-        float* pp = P + (ty + HALO) * xs + tx + LP;
-        *pp = it ? fmaf(beta, *pp, hs[k]) : hs[k];
+    for (int k = 0; k < CGP_HALO_REGS; ++k)
+      if (htile[k] >= 0) {
+        const float s = himg[k] >= 0 ? __uint_as_float((unsigned)hw[k]) : 0.0f;
+        P[htile[k]] = it ? fmaf(beta, P[htile[k]], s) : s;
       }
-    }
-    __syncthreads();
+    if (__syncthreads_or(!ok)) return;
     // ---- q = (L + sigma I) p, p^T q
     float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     op.prepare(P, EX, W, H);
@@ -382,12 +573,15 @@ __global__ void __launch_bounds__(CGP_T, 1) k_cgp_image(const __grid_constant__ 
       }
       *reinterpret_cast<float4*>(Q + y * W + x) = make_float4(q[0], q[1], q[2], q[3]);
     }
-    if (!cgp_allreduce<1, CGP_T>(v, sh, words, a.slots, ++epoch, a.cg.st)) return;
-    if (threadIdx.x == 0) cgp_dir_scalars(sh);
-    __syncthreads();
-    if (sh.status != CG_RUN) break;
+    if (!cgp_allreduce<1, CGP_T, N>(v, scale, sh, a.slots, ++epoch, a.cg.st, [] {},
+                                    [&](int, N t) { cgp_direction(sh, t, lane); }))
+      return;
+    status = sh.status;
+    if (status != CG_RUN) break;
     // ---- x += alpha p, s -= alpha T q, the sums
-    const float alpha = (float)sh.alpha;
+    const float alpha = cgp_value(sh.alpha);
+    cgp_prepare_beta(sh, beta_mode);
+    cgp_history(sh, a.cg.hist, it);
     v[0] = 0.0f;
     for (int u = wid; u < nunits; u += CGP_T / 32) {
       const int x = (u % ux_n) * 32 + rx, y = (u / ux_n) * 4 + ry;
@@ -412,12 +606,12 @@ __global__ void __launch_bounds__(CGP_T, 1) k_cgp_image(const __grid_constant__ 
       }
       *reinterpret_cast<float4*>(X + y * W + x) = make_float4(xv[0], xv[1], xv[2], xv[3]);
       *reinterpret_cast<float4*>(S + y * W + x) = make_float4(s[0], s[1], s[2], s[3]);
-      if (cnt) frame(x, y, cnt, s);
+      if (cnt) frame(x, y, cnt, s, (unsigned)it + 2u);
     }
-    if (!cgp_allreduce<4, CGP_T>(v, sh, words, a.slots, ++epoch, a.cg.st)) return;
-    __syncthreads();
-    if (threadIdx.x == 0) cgp_update_scalars(sh, it, beta_mode, tol2, a.cg.hist);
-    __syncthreads();
+    if (!cgp_allreduce<4, CGP_T, N>(v, scale, sh, a.slots, ++epoch, a.cg.st, halo_get,
+                                    [&](int w, N t) { cgp_update_tail(sh, w, t, lane); }))
+      return;
+    status = cgp_status(sh);
   }
   for (int u = wid; u < nunits; u += CGP_T / 32) {
     const int x = (u % ux_n) * 32 + rx, y = (u / ux_n) * 4 + ry;
@@ -426,7 +620,7 @@ __global__ void __launch_bounds__(CGP_T, 1) k_cgp_image(const __grid_constant__ 
     const float xv[4] = {x4.x, x4.y, x4.z, x4.w};
     if (cnt) run_store(a.cg.x, (int64_t)(by + y) * nx + bx + x, cnt, a.vec && (((uintptr_t)a.cg.x & 15) == 0), xv);
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) cgp_write_state(sh, a.cg.st, it);
+  cgp_write_state(sh, a.cg.st, it, status);
 }
 
 // ---------------------------------------------------------------- signals
@@ -441,6 +635,7 @@ struct CgpLine {
   T ls[BF_MAX_R1D + 1];
   int n, R, W, kmax;
   u64* slots;
+  u64* frames;                                 // [n] words (FP64: [n][2]): s at the pieces' ends
 };
 
 __host__ __device__ inline size_t cgp_line_elems(int W, int R) {
@@ -450,8 +645,9 @@ __host__ __device__ inline size_t cgp_line_elems(int W, int R) {
 template <typename T>
 __global__ void __launch_bounds__(CGP_TL, 1) k_cgp_line(const __grid_constant__ CgpLine<T> a) {
   extern __shared__ __align__(16) float cgp_smem[];
-  __shared__ CgpShared sh;
-  __shared__ unsigned words[CGP_MAXC * CGP_SLOT];
+  typedef typename CgpNum<T>::type N;
+  __shared__ CgpShared<T> sh;
+  const int lane = threadIdx.x & 31;
   const int W = a.W, R = a.R, n = a.n;
   const int beta_mode = a.cg.st->beta_mode;
   const double tol2 = a.cg.st->tol2;
@@ -485,13 +681,50 @@ __global__ void __launch_bounds__(CGP_TL, 1) k_cgp_line(const __grid_constant__ 
   __syncthreads();
   auto lap = [&](int q) {                      // (L p) of sample q of the piece
     const T pi = P[q + R];
-    T acc = T(0);
+    T acc[4] = {T(0), T(0), T(0), T(0)};       // four chains: an FP64 FMA is long
     for (int t = 1; t <= R; ++t) {
       const T* wt = WF + (t - 1) * (W + R) + q + R;
-      acc = fma(wt[0], pi - P[q + R + t], acc);
-      acc = fma(wt[-t], pi - P[q + R - t], acc);
+      const T f = pi - P[q + R + t], g = pi - P[q + R - t];
+      if (t & 1) {
+        acc[0] = fma(wt[0], f, acc[0]);
+        acc[1] = fma(wt[-t], g, acc[1]);
+      } else {
+        acc[2] = fma(wt[0], f, acc[2]);
+        acc[3] = fma(wt[-t], g, acc[3]);
+      }
     }
-    return acc;
+    return (acc[0] + acc[1]) + (acc[2] + acc[3]);
+  };
+  // s at the ends of the piece, for the neighbours, and the halo
+  auto frame = [&](int q, T s, unsigned tag) {
+    if (q >= R && q < len - R) return;
+    if (sizeof(T) == 4) {
+      cgp_put(a.frames + b + q, cgp_word(tag, __float_as_uint((float)s)));
+    } else {
+      const u64 bits = (u64)__double_as_longlong((double)s);
+      cgp_put(a.frames + 2 * (int64_t)(b + q), cgp_word(tag, (unsigned)bits));
+      cgp_put(a.frames + 2 * (int64_t)(b + q) + 1, cgp_word(tag, (unsigned)(bits >> 32)));
+    }
+  };
+  static_assert(2 * BF_MAX_R1D <= CGP_TL, "one halo sample per thread");
+  const int hi_ = threadIdx.x < R ? b - R + threadIdx.x : b + W + threadIdx.x - R;
+  const bool halo = threadIdx.x < 2 * R, hin = halo && (unsigned)hi_ < (unsigned)n;
+  T* hp = P + (threadIdx.x < R ? threadIdx.x : W + threadIdx.x);
+  u64 hw[2] = {0ull, 0ull};
+  auto halo_get = [&]() {
+    if (hin) {
+      if (sizeof(T) == 4) hw[0] = cgp_get(a.frames + hi_);
+      else cgp_get2(a.frames + 2 * (int64_t)hi_, hw[0], hw[1]);
+    }
+  };
+  auto halo_wait = [&](unsigned tag) {
+    bool ok = true;
+    if (hin) {
+      if ((unsigned)(hw[0] >> 32) != tag) ok = cgp_wait(a.frames + (sizeof(T) / 4) * (int64_t)hi_, hw[0], tag, a.cg.st);
+      if (ok && sizeof(T) == 8 && (unsigned)(hw[1] >> 32) != tag)
+        ok = cgp_wait(a.frames + 2 * (int64_t)hi_ + 1, hw[1], tag, a.cg.st);
+    }
+    return ok;
   };
   unsigned epoch = 1;
   {
@@ -501,42 +734,48 @@ __global__ void __launch_bounds__(CGP_TL, 1) k_cgp_line(const __grid_constant__ 
       X[q] = xi;
       RR[q] = r;
       S[q] = s;
-      if (q < R || q >= len - R) a.cg.s[b + q] = s;
+      frame(q, s, 1u);
       v[0] = fma(s, r, v[0]);
       v[1] = fma(s, s, v[1]);
       v[2] = fma(r, r, v[2]);
       v[3] = fma(xi, xi, v[3]);
     }
-    if (!cgp_allreduce<4, CGP_TL>(v, sh, words, a.slots, epoch, a.cg.st)) return;
-    __syncthreads();
-    if (threadIdx.x == 0) cgp_start_scalars(sh, (double)a.cg.shift);
-    __syncthreads();
+    if (!cgp_allreduce<4, CGP_TL, double>(v, T(1), sh, a.slots, epoch, a.cg.st, halo_get, [&](int w, double t) {
+          if (lane == 0) sh.tot[w] = t;
+        }))
+      return;
+    cgp_start(sh, (double)a.cg.shift, tol2);
   }
-  int it = 0;
-  for (; it < a.kmax && sh.status == CG_RUN; ++it) {
-    const T beta = it ? (T)sh.beta : T(0);
-    for (int h = threadIdx.x; h < 2 * R; h += CGP_TL) {        // halo
-      const int i = h < R ? b - R + h : b + W + h - R;
-      T* pp = P + (h < R ? h : W + h);
-      const T s = (unsigned)i < (unsigned)n ? __ldcg(a.cg.s + i) : T(0);
-      *pp = it ? fma(beta, *pp, s) : s;
-    }
+  int it = 0, status = sh.status;
+  const T scale = (T)sh.scale;
+  for (; it < a.kmax && status == CG_RUN; ++it) {
+    const T beta = (T)cgp_value(sh.beta);      // 0 before the first step
     for (int q = threadIdx.x; q < W; q += CGP_TL) {
       const T s = q < len ? S[q] : T(0);
       P[q + R] = it ? fma(beta, P[q + R], s) : s;
     }
-    __syncthreads();
+    const bool ok = halo_wait((unsigned)it + 1u);
+    if (halo) {
+      const T s = !hin ? T(0)
+                       : (sizeof(T) == 4 ? (T)__uint_as_float((unsigned)hw[0])
+                                         : (T)__longlong_as_double((long long)((hw[1] << 32) | (hw[0] & 0xffffffffull))));
+      *hp = it ? fma(beta, *hp, s) : s;
+    }
+    if (__syncthreads_or(!ok)) return;
     T v[4] = {T(0), T(0), T(0), T(0)};
     for (int q = threadIdx.x; q < len; q += CGP_TL) {
       const T p = P[q + R], qq = fma(a.cg.shift, p, lap(q));
       Q[q] = qq;
       v[0] = fma(p, qq, v[0]);
     }
-    if (!cgp_allreduce<1, CGP_TL>(v, sh, words, a.slots, ++epoch, a.cg.st)) return;
-    if (threadIdx.x == 0) cgp_dir_scalars(sh);
-    __syncthreads();
-    if (sh.status != CG_RUN) break;
-    const T alpha = (T)sh.alpha;
+    if (!cgp_allreduce<1, CGP_TL, N>(v, scale, sh, a.slots, ++epoch, a.cg.st, [] {},
+                                    [&](int, N t) { cgp_direction(sh, t, lane); }))
+      return;
+    status = sh.status;
+    if (status != CG_RUN) break;
+    const T alpha = (T)cgp_value(sh.alpha);
+    cgp_prepare_beta(sh, beta_mode);
+    cgp_history(sh, a.cg.hist, it);
     v[0] = T(0);
     for (int q = threadIdx.x; q < len; q += CGP_TL) {
       const T qq = Q[q];
@@ -544,19 +783,19 @@ __global__ void __launch_bounds__(CGP_TL, 1) k_cgp_line(const __grid_constant__ 
       const T r = fma(-alpha, qq, RR[q]), s = a.cg.dinv ? r * DI[q] : r;
       RR[q] = r;
       S[q] = s;
-      if (q < R || q >= len - R) a.cg.s[b + q] = s;
+      frame(q, s, (unsigned)it + 2u);
       v[0] = fma(s, r, v[0]);
       v[1] = fma(s, qq, v[1]);
       v[2] = fma(s, s, v[2]);
       v[3] = fma(r, r, v[3]);
     }
-    if (!cgp_allreduce<4, CGP_TL>(v, sh, words, a.slots, ++epoch, a.cg.st)) return;
-    __syncthreads();
-    if (threadIdx.x == 0) cgp_update_scalars(sh, it, beta_mode, tol2, a.cg.hist);
-    __syncthreads();
+    if (!cgp_allreduce<4, CGP_TL, N>(v, scale, sh, a.slots, ++epoch, a.cg.st, halo_get,
+                                    [&](int w, N t) { cgp_update_tail(sh, w, t, lane); }))
+      return;
+    status = cgp_status(sh);
   }
   for (int q = threadIdx.x; q < len; q += CGP_TL) a.cg.x[b + q] = X[q];
-  if (blockIdx.x == 0 && threadIdx.x == 0) cgp_write_state(sh, a.cg.st, it);
+  cgp_write_state(sh, a.cg.st, it, status);
 }
 
 // ---------------------------------------------------------------- host
@@ -602,18 +841,18 @@ bool cgp_rect(int nx, int ny, CgpRect* out, int* nreg) {
   return best >= 0;
 }
 
-// Samples per CTA of a signal: at least 64 (a smaller piece only adds partial sums to add),
-// 0 if it does not fit.
+// Samples per CTA of a signal: at least 128 (four warps, one per scheduler; a smaller piece
+// only adds partial sums to add), 0 if it does not fit.
 int cgp_line_width(const bf_graph* g) {
   const int maxc = cgp_max_ctas();
   if (maxc < 1) return 0;
-  int64_t W = std::max<int64_t>(64, (g->n + maxc - 1) / maxc);
+  int64_t W = std::max<int64_t>(128, (g->n + maxc - 1) / maxc);
   W = std::max<int64_t>((W + 31) / 32 * 32, 2 * g->rx);
   return cgp_line_elems((int)std::min<int64_t>(W, 1 << 20), g->rx) * g->esize > CGP_SMEM_MAX ? 0 : (int)W;
 }
 
 bool cgp_is_line(const bf_graph* g) {
-  return g->kind == BF_KIND_BILATERAL && g->p.ndim == 1 && g->ry == 0 && g->n < (1 << 30);
+  return g->kind == BF_KIND_BILATERAL && g->p.ndim == 1 && g->ry == 0 && g->n < (1 << 28);
 }
 bool cgp_is_image(const bf_graph* g) {
   return g->kind == BF_KIND_BILATERAL && fast_shape(g) == FAST_R3_2D && g->p.weight_mode == BF_W_ONTHEFLY;
@@ -658,6 +897,7 @@ static int launch_line(const bf_graph* g, const CgArgs<T>& cg, int kmax, cudaStr
   a.W = cgp_line_width(g);
   a.kmax = kmax;
   a.slots = (u64*)cg.partials;
+  a.frames = (u64*)cg.p_old;
   void* args[] = {&a};
   const int grid = (a.n + a.W - 1) / a.W;
   return cgp_coop(k_cgp_line<T>, grid, CGP_TL, cgp_line_elems(a.W, a.R) * sizeof(T), s, args);
@@ -684,6 +924,7 @@ int cgp_launch<float>(const bf_graph* g, const CgArgs<float>& cg, int kmax, cuda
   a.kmax = kmax;
   a.vec = g->nx % 4 == 0;
   a.slots = (u64*)cg.partials;
+  a.frames = (u64*)cg.p_old;
   void* args[] = {&op, &a};
   return cgp_coop(k_cgp_image<CgpBilateral>, nreg, CGP_T, cgp_image_floats<CgpBilateral>(a.rc.W, a.rc.H) * 4, s, args);
 }
