@@ -27,6 +27,7 @@
 
 #include "bf_cg.cuh"
 #include "bf_run.cuh"
+#include "bf_window_fast.cuh"
 
 namespace {
 
@@ -381,14 +382,174 @@ struct CgpBilateral {
       G[q] = in ? (c.use_guide ? guide[(int64_t)gy * nx + gx] : 0.0f) : __int_as_float(0x7f800000);
     }
   }
-  __device__ void prepare(const float*, float*, int, int) const {}
+  __device__ void prepare(const float*, float*, int, int, int, int, int, int) const {}
   // (L p) of the run at (x, y) of the rectangle
-  __device__ void sums(const float* P, const float* G, int W, int H, int x, int y, float (&vi)[RUN_P],
-                       float (&acc)[RUN_P]) const {
+  __device__ void sums(const float* P, const float* G, int W, int H, int x, int y, int, int, int, int,
+                       float (&vi)[RUN_P], float (&acc)[RUN_P]) const {
     const int xs = W + 2 * LP;
     float ws[RUN_P];
     const int o = y * xs + x;
     run_sums<true, false>(c, P + o, G + o, xs, vi, acc, ws);
+  }
+};
+
+// The guided filter's operator (Section 3, Eq. 6) of radius R in the difference form of
+// bf_guided.cu, by runs of four: stage A gives d_k and a_k of the windows centred on the
+// rectangle and R pixels around it, stage B sums the windows that contain a pixel.  Bound by
+// shared memory (about 90 wavefronts per 32 pixels) and the FP32 pipe (225 of its cycles per
+// scheduler at R = 2).  Rectangles whose halo leaves the image test every member.
+template <int R>
+struct CgpGuided {
+  static constexpr int HALO = 2 * R, LP = 8;
+  const float* guide;
+  const float* mu;
+  const float* ivar;
+  static __host__ __device__ size_t tile(int W, int H) { return (size_t)(W + 2 * LP) * (H + 2 * HALO); }
+  static __host__ __device__ size_t extra(int W, int H) { return 5 * tile(W, H); }
+  static __device__ float inv_count(int gx, int gy, int nx, int ny) {
+    const int cy = min(gy + R, ny - 1) - max(gy - R, 0) + 1, cx = min(gx + R, nx - 1) - max(gx - R, 0) + 1;
+    return 1.0f / (float)(cx * cy);
+  }
+  static __device__ bool border(int W, int H, int bx, int by, int nx, int ny) {
+    return bx - HALO < 0 || by - HALO < 0 || bx + W + HALO > nx || by + H + HALO > ny;
+  }
+  // tiles: guide, mean, 1 / (variance + eps) / N, d_k, a_k
+  __device__ void stage(float* EX, int W, int H, int bx, int by, int nx, int ny) const {
+    const int xs = W + 2 * LP, nt = (int)tile(W, H);
+    for (int q = threadIdx.x; q < nt; q += CGP_T) {
+      const int hy = q / xs, hx = q - hy * xs;
+      const int gy = by - HALO + hy, gx = bx - LP + hx;
+      const bool in = (unsigned)gx < (unsigned)nx && (unsigned)gy < (unsigned)ny;
+      const int64_t gp = (int64_t)gy * nx + gx;
+      EX[q] = in ? guide[gp] : 0.0f;
+      EX[nt + q] = in ? mu[gp] : 0.0f;
+      EX[2 * nt + q] = in ? ivar[gp] * inv_count(gx, gy, nx, ny) : 0.0f;
+      EX[3 * nt + q] = EX[4 * nt + q] = 0.0f;
+    }
+  }
+  // entry e of 12 values held as pairs
+  static __device__ __forceinline__ float at(const run_f2 (&p)[6], int e) { return (e & 1) ? run_hi(p[e / 2]) : run_lo(p[e / 2]); }
+  template <bool CHECK>
+  __device__ __forceinline__ void stage_a(const float* P, const float* G, const float* MU, int xs, int o, int gx0, int gy,
+                                          int nx, int ny, float (&ds)[RUN_P], float (&cs)[RUN_P]) const {
+    run_f2 ds2[RUN_P], cs2[RUN_P], xk2[RUN_P], mk2[RUN_P];
+#pragma unroll
+    for (int j = 0; j < RUN_P; ++j) {
+      const float xk = P[o + j], mk = MU[o + j];
+      xk2[j] = f2_pack(xk, xk);
+      mk2[j] = f2_pack(mk, mk);
+      ds2[j] = cs2[j] = 0ull;
+      ds[j] = cs[j] = 0.0f;
+    }
+#pragma unroll
+    for (int dy = -R; dy <= R; ++dy) {
+      if (CHECK && (unsigned)(gy + dy) >= (unsigned)ny) continue;
+      run_f2 xr[6], gr[6];
+      run_ld(P + o + dy * xs - 4, xr);
+      run_ld(G + o + dy * xs - 4, gr);
+#pragma unroll
+      for (int j = 0; j < RUN_P; ++j) {
+#pragma unroll
+        for (int a = 0; a < 6; ++a) {
+          const int lo = j + 4 - R, hi = j + 4 + R;
+          const bool i0 = 2 * a >= lo && 2 * a <= hi, i1 = 2 * a + 1 >= lo && 2 * a + 1 <= hi;
+          if (i0 && i1 && !CHECK) {
+            const run_f2 xd = run_sub(xr[a], xk2[j]);
+            ds2[j] = run_add(ds2[j], xd);
+            cs2[j] = run_fma(run_sub(gr[a], mk2[j]), xd, cs2[j]);
+          } else {
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+              const int e = 2 * a + b;
+              if (!(b ? i1 : i0) || (CHECK && (unsigned)(gx0 + e - 4) >= (unsigned)nx)) continue;
+              const float xd = at(xr, e) - run_lo(xk2[j]);
+              ds[j] += xd;
+              cs[j] = fmaf(at(gr, e) - run_lo(mk2[j]), xd, cs[j]);
+            }
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < RUN_P; ++j) {
+      ds[j] += run_lo(ds2[j]) + run_hi(ds2[j]);
+      cs[j] += run_lo(cs2[j]) + run_hi(cs2[j]);
+    }
+  }
+  __device__ void prepare(const float* P, float* EX, int W, int H, int bx, int by, int nx, int ny) const {
+    const int xs = W + 2 * LP, nt = (int)tile(W, H), per = W / 4 + 2;
+    const float *G = EX, *MU = EX + nt, *IV = EX + 2 * nt;
+    float *DK = EX + 3 * nt, *AK = EX + 4 * nt;
+    const bool chk = border(W, H, bx, by, nx, ny);
+    for (int r = threadIdx.x; r < per * (H + 2 * R); r += CGP_T) {
+      const int ry = r / per, x = 4 * (r - ry * per) - 4, y = ry - R;     // windows (x .. x + 3, y)
+      const int o = (y + HALO) * xs + x + LP;
+      float ds[RUN_P], cs[RUN_P];
+      if (chk) stage_a<true>(P, G, MU, xs, o, bx + x, by + y, nx, ny, ds, cs);
+      else stage_a<false>(P, G, MU, xs, o, bx + x, by + y, nx, ny, ds, cs);
+#pragma unroll
+      for (int j = 0; j < RUN_P; ++j) {
+        const int gx = bx + x + j, gy = by + y;
+        const bool in = !chk || ((unsigned)gx < (unsigned)nx && (unsigned)gy < (unsigned)ny);
+        const float inv = chk ? (in ? inv_count(gx, gy, nx, ny) : 0.0f) : 1.0f / (float)((2 * R + 1) * (2 * R + 1));
+        DK[o + j] = in ? ds[j] * inv : 0.0f;
+        AK[o + j] = in ? cs[j] * IV[o + j] : 0.0f;
+      }
+    }
+    __syncthreads();
+  }
+  template <bool CHECK>
+  __device__ __forceinline__ void stage_b(const float* P, const float* EX, int nt, int xs, int o, int gx0, int gy, int nx,
+                                          int ny, float (&vi)[RUN_P], float (&acc)[RUN_P]) const {
+    const float *G = EX, *MU = EX + nt, *DK = EX + 3 * nt, *AK = EX + 4 * nt;
+    run_f2 xi2[RUN_P], gi2[RUN_P], l2[RUN_P];
+#pragma unroll
+    for (int j = 0; j < RUN_P; ++j) {
+      vi[j] = P[o + j];
+      const float gi = G[o + j];
+      xi2[j] = f2_pack(vi[j], vi[j]);
+      gi2[j] = f2_pack(gi, gi);
+      l2[j] = 0ull;
+      acc[j] = 0.0f;
+    }
+#pragma unroll
+    for (int dy = -R; dy <= R; ++dy) {
+      if (CHECK && (unsigned)(gy + dy) >= (unsigned)ny) continue;
+      run_f2 xr[6], mr[6], dr[6], ar[6];
+      const int ro = o + dy * xs - 4;
+      run_ld(P + ro, xr);
+      run_ld(MU + ro, mr);
+      run_ld(DK + ro, dr);
+      run_ld(AK + ro, ar);
+#pragma unroll
+      for (int j = 0; j < RUN_P; ++j) {
+#pragma unroll
+        for (int a = 0; a < 6; ++a) {
+          const int lo = j + 4 - R, hi = j + 4 + R;
+          const bool i0 = 2 * a >= lo && 2 * a <= hi, i1 = 2 * a + 1 >= lo && 2 * a + 1 <= hi;
+          if (i0 && i1 && !CHECK) {
+            const run_f2 t = run_sub(run_sub(xi2[j], xr[a]), dr[a]);
+            l2[j] = run_add(l2[j], run_fma(run_sub(mr[a], gi2[j]), ar[a], t));
+          } else {
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+              const int e = 2 * a + b;
+              if (!(b ? i1 : i0) || (CHECK && (unsigned)(gx0 + e - 4) >= (unsigned)nx)) continue;
+              const float t = (vi[j] - at(xr, e)) - at(dr, e);
+              acc[j] += fmaf(at(mr, e) - run_lo(gi2[j]), at(ar, e), t);
+            }
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < RUN_P; ++j) acc[j] += run_lo(l2[j]) + run_hi(l2[j]);
+  }
+  __device__ void sums(const float* P, const float* EX, int W, int H, int x, int y, int bx, int by, int nx, int ny,
+                       float (&vi)[RUN_P], float (&acc)[RUN_P]) const {
+    const int xs = W + 2 * LP, nt = (int)tile(W, H), o = (y + HALO) * xs + x + LP;
+    if (border(W, H, bx, by, nx, ny)) stage_b<true>(P, EX, nt, xs, o, bx + x, by + y, nx, ny, vi, acc);
+    else stage_b<false>(P, EX, nt, xs, o, bx + x, by + y, nx, ny, vi, acc);
   }
 };
 
@@ -500,12 +661,12 @@ __global__ void __launch_bounds__(CGP_T, 1) k_cgp_image(const __grid_constant__ 
   unsigned epoch = 1;
   {
     float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-    op.prepare(P, EX, W, H);
+    op.prepare(P, EX, W, H, bx, by, nx, ny);
     for (int u = wid; u < nunits; u += CGP_T / 32) {
       const int x = (u % ux_n) * 32 + rx, y = (u / ux_n) * 4 + ry;
       const int cnt = run_count(bx + x, by + y, nx, ny);
       float xi[RUN_P], acc[RUN_P], s[RUN_P];
-      op.sums(P, EX, W, H, x, y, xi, acc);
+      op.sums(P, EX, W, H, x, y, bx, by, nx, ny, xi, acc);
 #pragma unroll
       for (int j = 0; j < RUN_P; ++j) {
         s[j] = 0.0f;
@@ -557,12 +718,12 @@ __global__ void __launch_bounds__(CGP_T, 1) k_cgp_image(const __grid_constant__ 
     if (__syncthreads_or(!ok)) return;
     // ---- q = (L + sigma I) p, p^T q
     float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-    op.prepare(P, EX, W, H);
+    op.prepare(P, EX, W, H, bx, by, nx, ny);
     for (int u = wid; u < nunits; u += CGP_T / 32) {
       const int x = (u % ux_n) * 32 + rx, y = (u / ux_n) * 4 + ry;
       const int cnt = run_count(bx + x, by + y, nx, ny);
       float pi[RUN_P], acc[RUN_P], q[RUN_P];
-      op.sums(P, EX, W, H, x, y, pi, acc);
+      op.sums(P, EX, W, H, x, y, bx, by, nx, ny, pi, acc);
 #pragma unroll
       for (int j = 0; j < RUN_P; ++j) {
         q[j] = 0.0f;
@@ -857,6 +1018,19 @@ bool cgp_is_line(const bf_graph* g) {
 bool cgp_is_image(const bf_graph* g) {
   return g->kind == BF_KIND_BILATERAL && fast_shape(g) == FAST_R3_2D && g->p.weight_mode == BF_W_ONTHEFLY;
 }
+// guided images of radius 1 .. 3 in FP32: the radius, else 0
+int cgp_guided(const bf_graph* g) {
+  return g->kind == BF_KIND_GUIDED && g->esize == 4 && g->ry > 0 && g->rx <= 3 ? g->rx : 0;
+}
+bool cgp_split(const bf_graph* g, CgpRect* rc, int* nreg) {
+  if (cgp_is_image(g)) return cgp_rect<CgpBilateral>(g->nx, g->ny, rc, nreg);
+  switch (cgp_guided(g)) {
+    case 1: return cgp_rect<CgpGuided<1>>(g->nx, g->ny, rc, nreg);
+    case 2: return cgp_rect<CgpGuided<2>>(g->nx, g->ny, rc, nreg);
+    case 3: return cgp_rect<CgpGuided<3>>(g->nx, g->ny, rc, nreg);
+  }
+  return false;
+}
 
 template <class F, class A>
 int cgp_coop(F fn, int grid, int threads, size_t smem, cudaStream_t s, A& args) {
@@ -873,9 +1047,7 @@ size_t cgp_words(const bf_graph* g) {
   if (cgp_max_ctas() < 1) return 0;
   CgpRect rc;
   int nreg = 0;
-  bool ok = false;
-  if (cgp_is_line(g)) ok = cgp_line_width(g) > 0;
-  else if (cgp_is_image(g)) ok = cgp_rect<CgpBilateral>(g->nx, g->ny, &rc, &nreg);
+  const bool ok = cgp_is_line(g) ? cgp_line_width(g) > 0 : cgp_split(g, &rc, &nreg);
   return ok ? 2 * CGP_MAXC * CGP_SLOT : 0;
 }
 
@@ -903,6 +1075,12 @@ static int launch_line(const bf_graph* g, const CgArgs<T>& cg, int kmax, cudaStr
   return cgp_coop(k_cgp_line<T>, grid, CGP_TL, cgp_line_elems(a.W, a.R) * sizeof(T), s, args);
 }
 
+template <class OP>
+static int cgp_image(OP op, CgpImage& a, int nreg, cudaStream_t s) {
+  void* args[] = {&op, &a};
+  return cgp_coop(k_cgp_image<OP>, nreg, CGP_T, cgp_image_floats<OP>(a.rc.W, a.rc.H) * 4, s, args);
+}
+
 template <>
 int cgp_launch<double>(const bf_graph* g, const CgArgs<double>& cg, int kmax, cudaStream_t s) {
   return launch_line<double>(g, cg, kmax, s);
@@ -914,10 +1092,7 @@ int cgp_launch<float>(const bf_graph* g, const CgArgs<float>& cg, int kmax, cuda
   CgpImage a;
   memset(&a, 0, sizeof(a));
   int nreg = 0;
-  if (!cgp_rect<CgpBilateral>(g->nx, g->ny, &a.rc, &nreg)) return bf_fail(BF_EINVAL, "cg_filter: image does not fit");
-  CgpBilateral op;
-  op.c = run_const(g->gf);
-  op.guide = cg.guide;
+  if (!cgp_split(g, &a.rc, &nreg)) return bf_fail(BF_EINVAL, "cg_filter: image does not fit");
   a.cg = cg;
   a.nx = g->nx;
   a.ny = g->ny;
@@ -925,6 +1100,15 @@ int cgp_launch<float>(const bf_graph* g, const CgArgs<float>& cg, int kmax, cuda
   a.vec = g->nx % 4 == 0;
   a.slots = (u64*)cg.partials;
   a.frames = (u64*)cg.p_old;
-  void* args[] = {&op, &a};
-  return cgp_coop(k_cgp_image<CgpBilateral>, nreg, CGP_T, cgp_image_floats<CgpBilateral>(a.rc.W, a.rc.H) * 4, s, args);
+  if (cgp_is_image(g)) {
+    CgpBilateral op;
+    op.c = run_const(g->gf);
+    op.guide = cg.guide;
+    return cgp_image(op, a, nreg, s);
+  }
+  switch (cgp_guided(g)) {
+    case 1: return cgp_image(CgpGuided<1>{cg.guide, (const float*)g->gmu, (const float*)g->givar}, a, nreg, s);
+    case 2: return cgp_image(CgpGuided<2>{cg.guide, (const float*)g->gmu, (const float*)g->givar}, a, nreg, s);
+  }
+  return cgp_image(CgpGuided<3>{cg.guide, (const float*)g->gmu, (const float*)g->givar}, a, nreg, s);
 }

@@ -102,3 +102,20 @@ def test_early_stop_and_streams():
         bf().cg_filter(G2, x1, 15, out=ob, sync=False, stream=t)
     torch.cuda.synchronize()
     assert torch.equal(a, oa) and torch.equal(b, ob)
+
+
+@pytest.mark.parametrize("radius", [1, 2, 3])
+@pytest.mark.parametrize("shape", [(3, 4), (5, 33), (40, 61), (66, 130)])
+def test_guided_images(shape, radius):
+    from oracle.guided import GuidedGraph
+    img = np.random.default_rng(radius).uniform(0, 1, shape)
+    img[:, shape[1] // 2:] *= 0.3
+    g = torch.as_tensor(img.astype(np.float32), device="cuda")
+    G = bf().guided_graph(g, radius, 0.01)
+    O = GuidedGraph(host(g), shape, radius, 0.01)
+    iters = min(7, max(1, img.size // 4))
+    for kw in ({}, {"shift": 0.5}, {"precond": "identity"}):
+        x, info, _ = bf().cg_filter(G, g.reshape(-1), iters, **kw)
+        ref = solvers.cg(O, host(g).reshape(-1), iters, **kw)
+        assert info.iters == ref["iters"]
+        assert rel_l2(host(x), ref["x"]) < TOL_F32
