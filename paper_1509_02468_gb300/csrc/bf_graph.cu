@@ -567,13 +567,18 @@ __global__ void __launch_bounds__(BF_THREADS, 2) k_apply_rb(const Geom<float> g,
 }
 
 // Persistent, double-buffered form of k_apply_rb for the L operator with weights on the
-// fly (unscaled operand): one CTA per SM walks tiles of 32 x th pixels; while it computes
-// one tile the halo of its next tile is copied by cp.async (X in 16-byte pieces, zero
-// outside the image; the guide in 4-byte pieces, +inf outside the image so that the range
-// term gives a zero weight there and no mask is needed).  At K = 16 one thread carries all
-// 16 columns of its 4-pixel strip (each weight computed once, 256 threads, ~200 registers);
-// the other widths split the columns into groups of 8 (512 threads, <= 128 registers), as
-// two halo buffers of a 16-column-per-thread tile would not fit in shared memory at K = 32.
+// fly (unscaled operand): one CTA per SM walks tiles of 32 x th pixels; while its computing
+// warps work on one tile, two further warps copy the halo of its next tile by cp.async (X in
+// 16-byte pieces, zero outside the image; the guide in 4-byte pieces, +inf outside the image
+// so that the range term gives a zero weight there and no mask is needed).  With every warp
+// copying its share first, the FP32 pipe stood still for a fifth of the time (2048 x 2048,
+// K = 16: 369 us; with one, two, four copying warps 353, 310, 323 us; the pipe's share of
+// the time is 0.57).  The first tile is copied by all warps.  At K = 16 one thread carries
+// all 16 columns of its 4-pixel strip (each weight computed once, 256 threads; 16 warps of 8
+// columns each: 332 us, strips of 8 pixels: 330 us); the other widths split the columns into
+// groups of 8 (512 threads), as two halo buffers of a 16-column-per-thread tile would not
+// fit in shared memory at K = 32.
+#define PIPE_STAGERS 64
 template <int K>
 struct PipeTile {
   static constexpr int threads = (K == 16) ? 256 : 512;
@@ -601,39 +606,45 @@ __device__ __forceinline__ float rb_exp_ftz(float gi, float gj, float a_r, float
   return r;
 }
 
-template <int K>
-__device__ __forceinline__ void pipe_stage(const Geom<float>& g, const ApplyArgs<float>& a, int bx, int by,
-                                           unsigned char* buf) {
+// The halo tile at (bx, by) into buf, by nw warps (this one is w); GUIDE: the guide too.
+template <int K, bool GUIDE>
+__device__ __forceinline__ void pipe_stage(const Geom<float>& g, const ApplyArgs<float>& a, int bx, int by, int lane,
+                                           int w, int nw, unsigned char* buf) {
   typedef PipeTile<K> TT;
-  constexpr int NC4 = TT::nc4;
+  constexpr int NC4 = TT::nc4, STEP = 32 / NC4;         // pixels per instruction
   const unsigned sx = (unsigned)__cvta_generic_to_shared(buf);
   const unsigned sg = sx + (unsigned)TT::xbytes;
-  for (int idx = threadIdx.x; idx < TT::hp * NC4; idx += TT::threads) {
-    const int hp = idx / NC4, c = idx - hp * NC4;
+  const int c = lane % NC4;
+#pragma unroll 4
+  for (int hp = lane / NC4 + w * STEP; hp < TT::hp; hp += nw * STEP) {
     const int hy = hp / TT::hw, hx = hp - hy * TT::hw;
     const int gy = by - 3 + hy, gx = bx - 3 + hx;
-    const bool in = (gx >= 0 && gx < g.nx && gy >= 0 && gy < g.ny);
+    const bool in = ((unsigned)gx < (unsigned)g.nx && (unsigned)gy < (unsigned)g.ny);
     const float* src = in ? a.X + ((int64_t)gy * g.nx + gx) * a.ldx + c * 4 : a.X;
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(sx + (unsigned)(c * TT::cst + hp) * 16u),
-                 "l"(src), "r"(in ? 16 : 0)
-                 : "memory");
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(sx + (unsigned)(c * TT::cst + hp) * 16u), "l"(src),
+                 "r"(in ? 16 : 0) : "memory");
   }
+  if (!GUIDE) return;
   float* sgp = reinterpret_cast<float*>(buf + TT::xbytes);
-  for (int hp = threadIdx.x; hp < TT::hp; hp += TT::threads) {
-    const int hy = hp / TT::hw, hx = hp - hy * TT::hw;
-    const int gy = by - 3 + hy, gx = bx - 3 + hx;
-    if (gx >= 0 && gx < g.nx && gy >= 0 && gy < g.ny) {
-      asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(sg + (unsigned)hp * 4u),
-                   "l"(a.guide + (int64_t)gy * g.nx + gx)
-                   : "memory");
-    } else {
-      sgp[hp] = __int_as_float(0x7f800000);
+  for (int gyh = w; gyh < TT::hh; gyh += nw) {
+    const int gy = by - 3 + gyh;
+#pragma unroll
+    for (int h0 = 0; h0 < TT::hw; h0 += 32) {
+      const int h = h0 + lane, gx = bx - 3 + h, hp = gyh * TT::hw + h;
+      if (h >= TT::hw) continue;
+      if ((unsigned)gx < (unsigned)g.nx && (unsigned)gy < (unsigned)g.ny) {
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(sg + (unsigned)hp * 4u),
+                     "l"(a.guide + (int64_t)gy * g.nx + gx)
+                     : "memory");
+      } else {
+        sgp[hp] = __int_as_float(0x7f800000);
+      }
     }
   }
 }
 
 template <int K>
-__global__ void __launch_bounds__(PipeTile<K>::threads, 1) k_apply_pipe(const Geom<float> g, const ApplyArgs<float> a) {
+__global__ void __launch_bounds__(PipeTile<K>::threads + PIPE_STAGERS, 1) k_apply_pipe(const Geom<float> g, const ApplyArgs<float> a) {
   bf_pdl_enter();
   typedef PipeTile<K> TT;
   constexpr int CS = TT::cs, NG = TT::ng, CS4 = CS / 4;
@@ -642,17 +653,22 @@ __global__ void __launch_bounds__(PipeTile<K>::threads, 1) k_apply_pipe(const Ge
   const int ntiles = ntx * ((g.ny + TT::th - 1) / TT::th);
   const int lx = threadIdx.x & 31;
   const int rest = threadIdx.x >> 5;
+  constexpr int CW = TT::threads / 32, SW = PIPE_STAGERS / 32;
+  const bool stager = rest >= CW;                       // the last warps copy, the others compute
   const int grp = rest % NG, strip = rest / NG;
   const int row0 = strip * RB_P;
   int t = blockIdx.x;
-  if (t < ntiles) pipe_stage<K>(g, a, (t % ntx) * TT::tw, (t / ntx) * TT::th, smem);
-  asm volatile("cp.async.commit_group;" ::: "memory");
+  if (t < ntiles) pipe_stage<K, true>(g, a, (t % ntx) * TT::tw, (t / ntx) * TT::th, lx, rest, CW + SW, smem);
+  asm volatile("cp.async.wait_all;" ::: "memory");
   for (int b = 0; t < ntiles; t += gridDim.x, b ^= 1) {
-    const int tn = t + gridDim.x;
-    if (tn < ntiles) pipe_stage<K>(g, a, (tn % ntx) * TT::tw, (tn / ntx) * TT::th, smem + (b ^ 1) * TT::stage);
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    asm volatile("cp.async.wait_group 1;" ::: "memory");
-    __syncthreads();
+    __syncthreads();                                     // tile t has landed, the other buffer is free
+    if (stager) {
+      const int tn = t + gridDim.x;
+      if (tn < ntiles)
+        pipe_stage<K, true>(g, a, (tn % ntx) * TT::tw, (tn / ntx) * TT::th, lx, rest - CW, SW, smem + (b ^ 1) * TT::stage);
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      continue;
+    }
     const float4* sx = reinterpret_cast<const float4*>(smem + b * TT::stage);
     const float* sg = reinterpret_cast<const float*>(smem + b * TT::stage + TT::xbytes);
     const int bx = (t % ntx) * TT::tw, by = (t / ntx) * TT::th;
@@ -709,9 +725,146 @@ __global__ void __launch_bounds__(PipeTile<K>::threads, 1) k_apply_pipe(const Ge
         *reinterpret_cast<float4*>(yp + 4 * c4) = o;
       }
     }
-    __syncthreads();
   }
-  asm volatile("cp.async.wait_group 0;" ::: "memory");
+}
+
+// ---- the same walk with STORED weights (modes FP32 and BF16): the weights between a strip's
+// four pixels and a halo pixel are loaded from the planes of wf a few halo pixels ahead of
+// their use.  A warp's load of one tap is 32 consecutive weights; a forward weight plane is
+// read once by the pixel and once, as the backward tap, by the neighbour (an L1 or L2 hit).
+// Bound by the FP32 pipe (2 K lane operations per pixel and neighbour) and the weights'
+// bytes.  (k_apply_rb, which loads each weight where it is used, stood on their latency:
+// 1024 x 1024, K = 16, BF16: 470 us.)
+// The weight at byte offset `off` of the planes; volatile, so that the loads of a row stay
+// where they are issued.
+template <int WM>
+__device__ __forceinline__ float pipe_ld_w(const char* wf, unsigned off) {
+  if (WM == BF_W_STORED_BF16) {
+    unsigned short h;
+    asm volatile("ld.global.nc.u16 %0, [%1];" : "=h"(h) : "l"(wf + off));
+    return __uint_as_float((unsigned)h << 16);
+  }
+  float w;
+  asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(w) : "l"(wf + off));
+  return w;
+}
+
+// Weights between the halo pixel (row r of the strip's rows, column x + dx) and the strip's
+// pixels (column x, rows y0 ..; off: byte offset of pixel (x, y0) in a plane).  MASK: 0 unless
+// pixel and neighbour lie in the image (nothing else is read then).
+template <int WM, bool MASK>
+__device__ __forceinline__ void pipe_step_w(const void* wf, int n, int nx, int ny, int x, int y0, unsigned off, int r,
+                                            int dx, float (&w)[RB_P]) {
+  constexpr int ES = WM == BF_W_STORED_BF16 ? 2 : 4;
+  // opaque: the offsets of a strip's 192 loads would be kept for all its steps, and spilled
+  asm volatile("" : "+r"(n), "+r"(nx));
+#pragma unroll
+  for (int p = 0; p < RB_P; ++p) {
+    const int dy = r - 3 - p;
+    if (dy < -3 || dy > 3 || (dy == 0 && dx == 0)) continue;
+    const bool fwd = dy > 0 || (dy == 0 && dx > 0);
+    const int f = fwd ? ShapeR3::fwd_index(dy, dx) : ShapeR3::fwd_index(-dy, -dx);
+    const int e = f * n + p * nx + (fwd ? 0 : dy * nx + dx);
+    bool in = true;
+    if (MASK)
+      in = x < nx && y0 + p < ny && (unsigned)(x + dx) < (unsigned)nx && (unsigned)(y0 + p + dy) < (unsigned)ny;
+    w[p] = in ? pipe_ld_w<WM>((const char*)wf, off + (unsigned)(e * ES)) : 0.0f;
+  }
+}
+
+template <int K, int WM, bool MASK>
+__device__ __forceinline__ void pipe_tile_w(const Geom<float>& g, const ApplyArgs<float>& a, const float4* sx, int bx,
+                                            int by, int lx, int grp, int row0) {
+  typedef PipeTile<K> TT;
+  constexpr int CS = TT::cs, CS4 = CS / 4;
+  const int x = bx + lx, y0 = by + row0;
+  const int n = (int)a.n, nx = g.nx;
+  const unsigned off = (unsigned)(y0 * nx + x) * (WM == BF_W_STORED_BF16 ? 2u : 4u);
+  unsigned long long acc2[RB_P][CS / 2], xi2[RB_P][CS / 2];
+  // steps (row, dx) in order, the weights loaded AHEAD steps before they are used
+  constexpr int AHEAD = MASK ? 1 : (CS >= 8 ? 2 : 4), RING = AHEAD + 1, STEPS = 7 * (RB_P + 6);
+  float w[RING][RB_P];
+#pragma unroll
+  for (int q = 0; q < AHEAD; ++q) pipe_step_w<WM, MASK>(a.wf, n, nx, g.ny, x, y0, off, q / 7, q % 7 - 3, w[q]);
+#pragma unroll
+  for (int p = 0; p < RB_P; ++p) {
+    const int hp = (row0 + p + 3) * TT::hw + lx + 3;
+#pragma unroll
+    for (int c4 = 0; c4 < CS4; ++c4) {
+      const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(sx + (grp * CS4 + c4) * TT::cst + hp);
+      xi2[p][2 * c4] = v.x;
+      xi2[p][2 * c4 + 1] = v.y;
+    }
+#pragma unroll
+    for (int c = 0; c < CS / 2; ++c) acc2[p][c] = 0ull;
+  }
+#pragma unroll
+  for (int r = 0; r < RB_P + 6; ++r) {
+#pragma unroll
+  for (int dx = -3; dx <= 3; ++dx) {
+    const int q = 7 * r + dx + 3;
+    if (q + AHEAD < STEPS)
+      pipe_step_w<WM, MASK>(a.wf, n, nx, g.ny, x, y0, off, (q + AHEAD) / 7, (q + AHEAD) % 7 - 3, w[(q + AHEAD) % RING]);
+    const int hp = (row0 + r) * TT::hw + lx + 3 + dx;
+    unsigned long long xj2[CS / 2];
+#pragma unroll
+    for (int c4 = 0; c4 < CS4; ++c4) {
+      const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(sx + (grp * CS4 + c4) * TT::cst + hp);
+      xj2[2 * c4] = v.x;
+      xj2[2 * c4 + 1] = v.y;
+    }
+#pragma unroll
+    for (int p = 0; p < RB_P; ++p) {
+      const int dy = r - 3 - p;
+      if (dy < -3 || dy > 3 || (dy == 0 && dx == 0)) continue;
+      const unsigned long long w2 = f2_pack(w[q % RING][p], w[q % RING][p]);
+#pragma unroll
+      for (int c = 0; c < CS / 2; ++c) acc2[p][c] = f2_diff_fma(w2, xi2[p][c], xj2[c], acc2[p][c]);
+    }
+  }
+  }
+#pragma unroll
+  for (int p = 0; p < RB_P; ++p) {
+    if (MASK && (x >= g.nx || y0 + p >= g.ny)) continue;
+    float* yp = a.Y + ((int64_t)(y0 + p) * g.nx + x) * a.ldy + grp * CS;
+#pragma unroll
+    for (int c4 = 0; c4 < CS4; ++c4)
+      *reinterpret_cast<ulonglong2*>(yp + 4 * c4) = make_ulonglong2(acc2[p][2 * c4], acc2[p][2 * c4 + 1]);
+  }
+}
+
+template <int K, int WM>
+__global__ void __launch_bounds__(PipeTile<K>::threads + PIPE_STAGERS, 1)
+k_apply_pipe_w(const __grid_constant__ Geom<float> g, const ApplyArgs<float> a) {
+  bf_pdl_enter();
+  typedef PipeTile<K> TT;
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int ntx = (g.nx + TT::tw - 1) / TT::tw;
+  const int ntiles = ntx * ((g.ny + TT::th - 1) / TT::th);
+  const int lx = threadIdx.x & 31;
+  const int rest = threadIdx.x >> 5;
+  constexpr int CW = TT::threads / 32, SW = PIPE_STAGERS / 32;
+  const bool stager = rest >= CW;
+  const int grp = rest % TT::ng, row0 = (rest / TT::ng) * RB_P;
+  int t = blockIdx.x;
+  if (t < ntiles) pipe_stage<K, false>(g, a, (t % ntx) * TT::tw, (t / ntx) * TT::th, lx, rest, CW + SW, smem);
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  for (int b = 0; t < ntiles; t += gridDim.x, b ^= 1) {
+    __syncthreads();                                     // tile t has landed, the other buffer is free
+    if (stager) {
+      const int tn = t + gridDim.x;
+      if (tn < ntiles)
+        pipe_stage<K, false>(g, a, (tn % ntx) * TT::tw, (tn / ntx) * TT::th, lx, rest - CW, SW, smem + (b ^ 1) * TT::stage);
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      continue;
+    }
+    const float4* sx = reinterpret_cast<const float4*>(smem + b * TT::stage);
+    const int bx = (t % ntx) * TT::tw, by = (t / ntx) * TT::th;
+    if (bx >= 3 && bx + TT::tw + 3 <= g.nx && by >= 3 && by + TT::th + 3 <= g.ny)
+      pipe_tile_w<K, WM, false>(g, a, sx, bx, by, lx, grp, row0);
+    else
+      pipe_tile_w<K, WM, true>(g, a, sx, bx, by, lx, grp, row0);
+  }
 }
 
 static int num_sms() {
@@ -734,7 +887,21 @@ static int launch_apply_pipe(const bf_graph* g, const ApplyArgs<float>& a, cudaS
   }
   const int64_t ntiles = ((g->nx + TT::tw - 1) / TT::tw) * (int64_t)((g->ny + TT::th - 1) / TT::th);
   const int grid = (int)std::min<int64_t>(ntiles, num_sms());
-  BF_LAUNCH_PDL(k_apply_pipe<K>, grid, TT::threads, TT::smem, s, g->gf, a);
+  BF_LAUNCH_PDL(k_apply_pipe<K>, grid, TT::threads + PIPE_STAGERS, TT::smem, s, g->gf, a);
+  BF_CUDA(cudaGetLastError());
+  return BF_OK;
+}
+
+template <int K, int WM>
+static int launch_apply_pipe_w(const bf_graph* g, const ApplyArgs<float>& a, cudaStream_t s) {
+  typedef PipeTile<K> TT;
+  {
+    const int rc_ = bf_smem_attr((const void*)k_apply_pipe_w<K, WM>, (int)TT::smem, "cudaFuncSetAttribute(k_apply_pipe_w)");
+    if (rc_) return rc_;
+  }
+  const int64_t ntiles = ((g->nx + TT::tw - 1) / TT::tw) * (int64_t)((g->ny + TT::th - 1) / TT::th);
+  const int grid = (int)std::min<int64_t>(ntiles, num_sms());
+  BF_LAUNCH_PDL((k_apply_pipe_w<K, WM>), grid, TT::threads + PIPE_STAGERS, TT::smem, s, g->gf, a);
   BF_CUDA(cudaGetLastError());
   return BF_OK;
 }
@@ -755,9 +922,13 @@ static int launch_apply_rb(const bf_graph* g, const ApplyArgs<float>& a, cudaStr
 
 template <int K>
 static int launch_apply_rb_w(const bf_graph* g, const ApplyArgs<float>& a, cudaStream_t s) {
-  if (g->p.weight_mode == BF_W_ONTHEFLY && a.op == BF_OP_L && !a.scale && g->gf.a_r > 0.0f &&
-      ((uintptr_t)a.X & 15) == 0 && ((uintptr_t)a.Y & 15) == 0 && a.ldx % 4 == 0 && a.ldy % 4 == 0)
-    return launch_apply_pipe<K>(g, a, s);
+  if (a.op == BF_OP_L && !a.scale && ((uintptr_t)a.X & 15) == 0 && ((uintptr_t)a.Y & 15) == 0 && a.ldx % 4 == 0 &&
+      a.ldy % 4 == 0) {
+    // (the stored kernel's byte offsets are 32-bit)
+    if (g->p.weight_mode == BF_W_STORED_F32 && g->n < 44000000) return launch_apply_pipe_w<K, BF_W_STORED_F32>(g, a, s);
+    if (g->p.weight_mode == BF_W_STORED_BF16 && g->n < 44000000) return launch_apply_pipe_w<K, BF_W_STORED_BF16>(g, a, s);
+    if (g->p.weight_mode == BF_W_ONTHEFLY && g->gf.a_r > 0.0f) return launch_apply_pipe<K>(g, a, s);
+  }
   if (g->p.weight_mode == BF_W_ONTHEFLY) return launch_apply_rb<K, false>(g, a, s);
   return launch_apply_rb<K, true>(g, a, s);
 }

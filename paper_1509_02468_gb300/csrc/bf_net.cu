@@ -13,7 +13,12 @@
 // by bf_net_adam (Adam, Kingma and Ba).
 //
 // Kernels work on 32 x 8 pixel tiles with a one-pixel halo staged channel-major in shared
-// memory; activations are stored pixel-major [n][16].
+// memory; activations are stored pixel-major [n][16].  Both the layers and the weight
+// gradients are bound by shared memory unless a thread reuses what it loads: a thread owns a
+// run of four pixels (layers: times four output channels, so 18 loads feed 144 products per
+// input channel; gradients: all nine taps of one weight pair).  At 256 x 256 a pair's
+// training step took 241 us (layers 16 -> 16 of 20 us, their gradient 52 us, three serial
+// sums over the tiles of 33 us each).
 #include <cuda_bf16.h>
 #include <math.h>
 
@@ -28,7 +33,8 @@
 #define NET_TH 8
 #define NET_HW (NET_TW + 2)
 #define NET_HH (NET_TH + 2)
-#define NET_HP (NET_HW * NET_HH)
+#define NET_XS 36                          // staged row stride (16-byte aligned runs)
+#define NET_HP (NET_XS * NET_HH + 4)       // channel stride: 12 banks apart
 #define NET_W1 0
 #define NET_W2 (NET_CH * NET_CIN * 9)
 #define NET_W3 (NET_W2 + NET_CH * NET_CH * 9)
@@ -76,8 +82,8 @@ __device__ __forceinline__ float bf16_round(float x) { return __bfloat162float(_
 // Stage the input tile (with halo) channel-major: s[c * NET_HP + hp].
 template <int CIN, int IN>
 __device__ __forceinline__ void net_stage(const NetArgs& a, int col, int bx, int by, float* s) {
-  for (int hp = threadIdx.x; hp < NET_HP; hp += NET_TW * NET_TH) {
-    const int hy = hp / NET_HW, hx = hp - hy * NET_HW;
+  for (int q = threadIdx.x; q < NET_HW * NET_HH; q += NET_TW * NET_TH) {
+    const int hy = q / NET_HW, hx = q - hy * NET_HW, hp = hy * NET_XS + hx;
     const int gy = by - 1 + hy, gx = bx - 1 + hx;
     const bool inside = gx >= 0 && gx < a.nx && gy >= 0 && gy < a.ny;
     const int64_t i = (int64_t)gy * a.nx + gx;
@@ -123,9 +129,20 @@ __device__ __forceinline__ void net_stage(const NetArgs& a, int col, int bx, int
   }
 }
 
-// One 3 x 3 conv layer (CIN -> COUT) on a tile; blockIdx.z is the column.
+// The six staged values of one row of a run's window.
+__device__ __forceinline__ void net_row(const float* row, float (&x)[6]) {
+  const float4 a = *reinterpret_cast<const float4*>(row);
+  const float2 b = *reinterpret_cast<const float2*>(row + 4);
+  x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w;
+  x[4] = b.x; x[5] = b.y;
+}
+
+// One 3 x 3 conv layer (CIN -> COUT) on a tile; blockIdx.z is the column.  COUT = 16: warp w
+// computes output channels 4 (w / 2) .. + 3 of the runs of half a tile.  COUT = 1: the four
+// warp pairs each take a quarter of the input channels, and the quarters are added.
 template <int CIN, int COUT, int IN, int OUT>
 __global__ void __launch_bounds__(NET_TW * NET_TH) k_net_conv(const NetArgs a) {
+  static_assert(COUT == NET_CH || (COUT == 1 && CIN % 4 == 0), "layer shapes of the net");
   constexpr int COUTP = (COUT + 3) & ~3;
   if (a.stop && *a.stop != 0) return;
   __shared__ __align__(16) float sx[CIN * NET_HP];
@@ -140,51 +157,74 @@ __global__ void __launch_bounds__(NET_TW * NET_TH) k_net_conv(const NetArgs a) {
   }
   net_stage<CIN, IN>(a, col, bx, by, sx);
   __syncthreads();
-  const int lx = threadIdx.x % NET_TW, ly = threadIdx.x / NET_TW;
-  const int x = bx + lx, y = by + ly;
-  if (x >= a.nx || y >= a.ny) return;
-  float acc[COUTP];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, grp = wid >> 1;
+  const int lx = 4 * (lane & 7), ly = 4 * (wid & 1) + (lane >> 3);
+  if (COUT == 1) {
+    constexpr int CQ = CIN / 4;
+    __shared__ __align__(16) float red[4][NET_TW * NET_TH];
+    float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    for (int c = grp * CQ; c < (grp + 1) * CQ; ++c) {
 #pragma unroll
-  for (int o = 0; o < COUTP; ++o) acc[o] = 0.0f;
+      for (int ty = 0; ty < 3; ++ty) {
+        float x[6];
+        net_row(sx + c * NET_HP + (ly + ty) * NET_XS + lx, x);
+#pragma unroll
+        for (int tx = 0; tx < 3; ++tx) {
+          const float w = sw[(c * 9 + 3 * ty + tx) * COUTP];
+#pragma unroll
+          for (int p = 0; p < 4; ++p) acc[p] = fmaf(w, x[p + tx], acc[p]);
+        }
+      }
+    }
+    *reinterpret_cast<float4*>(&red[grp][ly * NET_TW + lx]) = make_float4(acc[0], acc[1], acc[2], acc[3]);
+    __syncthreads();
+    const int x = bx + (threadIdx.x & 31), y = by + (threadIdx.x >> 5);
+    if (x >= a.nx || y >= a.ny) return;
+    const float v = (red[0][threadIdx.x] + red[1][threadIdx.x]) + (red[2][threadIdx.x] + red[3][threadIdx.x]);
+    const int64_t i = (int64_t)y * a.nx + x;
+    if (OUT == OUT_PRECOND) a.z[i * a.ldz + col] = a.rho[col] * v;
+    else a.out[(int64_t)col * a.n + i] = v;
+    return;
+  }
+  float acc[4][4];                                          // [pixel][output channel]
+#pragma unroll
+  for (int p = 0; p < 4; ++p)
+#pragma unroll
+    for (int o = 0; o < 4; ++o) acc[p][o] = 0.0f;
   for (int c = 0; c < CIN; ++c) {
 #pragma unroll
-    for (int t = 0; t < 9; ++t) {
-      const int ty = t / 3, tx = t - 3 * (t / 3);
-      const float xv = sx[c * NET_HP + (ly + ty) * NET_HW + lx + tx];
-      const float4* w4 = reinterpret_cast<const float4*>(sw + (c * 9 + t) * COUTP);
+    for (int ty = 0; ty < 3; ++ty) {
+      float x[6];
+      net_row(sx + c * NET_HP + (ly + ty) * NET_XS + lx, x);
 #pragma unroll
-      for (int o4 = 0; o4 < COUTP / 4; ++o4) {
-        const float4 wv = w4[o4];
-        acc[4 * o4 + 0] = fmaf(wv.x, xv, acc[4 * o4 + 0]);
-        acc[4 * o4 + 1] = fmaf(wv.y, xv, acc[4 * o4 + 1]);
-        acc[4 * o4 + 2] = fmaf(wv.z, xv, acc[4 * o4 + 2]);
-        acc[4 * o4 + 3] = fmaf(wv.w, xv, acc[4 * o4 + 3]);
+      for (int tx = 0; tx < 3; ++tx) {
+        const float4 w = *reinterpret_cast<const float4*>(sw + (c * 9 + 3 * ty + tx) * COUTP + 4 * grp);
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+          acc[p][0] = fmaf(w.x, x[p + tx], acc[p][0]);
+          acc[p][1] = fmaf(w.y, x[p + tx], acc[p][1]);
+          acc[p][2] = fmaf(w.z, x[p + tx], acc[p][2]);
+          acc[p][3] = fmaf(w.w, x[p + tx], acc[p][3]);
+        }
       }
     }
   }
-  const int64_t i = (int64_t)y * a.nx + x;
-  if (OUT == OUT_PRECOND) {
-    a.z[i * a.ldz + col] = a.rho[col] * acc[0];
-  } else {
-    float* dst = a.out + ((int64_t)col * a.n + i) * COUT;
-    const float* mk = (OUT == OUT_MASKED) ? a.mask + ((int64_t)col * a.n + i) * COUT : nullptr;
-    if (COUT % 4 == 0) {
+  const int y = by + ly;
+  if (y >= a.ny) return;
 #pragma unroll
-      for (int o4 = 0; o4 < COUT / 4; ++o4) {
-        float4 v = make_float4(acc[4 * o4], acc[4 * o4 + 1], acc[4 * o4 + 2], acc[4 * o4 + 3]);
-        if (OUT == OUT_MASKED) {
-          const float4 m = reinterpret_cast<const float4*>(mk)[o4];
-          v.x = m.x > 0.0f ? v.x : 0.0f;
-          v.y = m.y > 0.0f ? v.y : 0.0f;
-          v.z = m.z > 0.0f ? v.z : 0.0f;
-          v.w = m.w > 0.0f ? v.w : 0.0f;
-        }
-        reinterpret_cast<float4*>(dst)[o4] = v;
-      }
-    } else {
-#pragma unroll
-      for (int o = 0; o < COUT; ++o) dst[o] = (OUT == OUT_MASKED) ? (mk[o] > 0.0f ? acc[o] : 0.0f) : acc[o];
+  for (int p = 0; p < 4; ++p) {
+    const int x = bx + lx + p;
+    if (x >= a.nx) continue;
+    const int64_t o = ((int64_t)col * a.n + (int64_t)y * a.nx + x) * COUT + 4 * grp;
+    float4 v = make_float4(acc[p][0], acc[p][1], acc[p][2], acc[p][3]);
+    if (OUT == OUT_MASKED) {
+      const float4 m = *reinterpret_cast<const float4*>(a.mask + o);
+      v.x = m.x > 0.0f ? v.x : 0.0f;
+      v.y = m.y > 0.0f ? v.y : 0.0f;
+      v.z = m.z > 0.0f ? v.z : 0.0f;
+      v.w = m.w > 0.0f ? v.w : 0.0f;
     }
+    *reinterpret_cast<float4*>(a.out + o) = v;
   }
 }
 
@@ -266,45 +306,82 @@ __global__ void k_net_loss_final(const double* partials, int nblocks, const doub
 }
 
 // Per-block weight gradient dW[o][c][t] = sum_px G[px][o] X[px + t][c] over the block's
-// tile (X staged like a conv input); partials[block][(o * CIN + c) * 9 + t].
+// tile (X staged like a conv input); partials[block][off + (o * CIN + c) * 9 + t].  A thread
+// owns the nine taps of one pair (o, c) over a share of the tile's runs of four pixels (each
+// sum in two parts, even and odd pixels); the shares are added in order.
 template <int CIN, int COUT, int IN>
-__global__ void __launch_bounds__(NET_TW * NET_TH) k_net_wgrad(const NetArgs a, const float* G, float* partials) {
-  __shared__ __align__(16) float sx[CIN * NET_HP];
-  __shared__ float sg[COUT * NET_TW * NET_TH];               // [o][px]
+__global__ void __launch_bounds__(NET_TW * NET_TH) k_net_wgrad(const NetArgs a, const float* G, float* partials, int off) {
+  constexpr int NP = COUT * CIN, NG = (NET_TW * NET_TH / NP < 16) ? NET_TW * NET_TH / NP : 16;
+  constexpr int NRUN = NET_TW * NET_TH / 4, GS = NET_TW * NET_TH + 4;   // gradient channel stride
+  constexpr int XF = CIN * NET_HP, GF = COUT * GS, RF = NG > 1 ? NG * NP * 9 : 0;
+  __shared__ __align__(16) float sh[(XF + GF > RF) ? XF + GF : RF];
+  float* sx = sh;
+  float* sg = sh + XF;                                       // [o][px]
   const int bx = blockIdx.x * NET_TW, by = blockIdx.y * NET_TH;
   net_stage<CIN, IN>(a, 0, bx, by, sx);
   for (int e = threadIdx.x; e < COUT * NET_TW * NET_TH; e += NET_TW * NET_TH) {
-    const int o = e / (NET_TW * NET_TH), p = e - o * (NET_TW * NET_TH);
+    const int p = e / COUT, o = e - p * COUT;
     const int ly = p / NET_TW, lx = p - ly * NET_TW;
     const int x = bx + lx, y = by + ly;
-    sg[e] = (x < a.nx && y < a.ny) ? G[((int64_t)y * a.nx + x) * COUT + o] : 0.0f;
+    sg[o * GS + p] = (x < a.nx && y < a.ny) ? G[((int64_t)y * a.nx + x) * COUT + o] : 0.0f;
   }
   __syncthreads();
-  const int blk = blockIdx.y * gridDim.x + blockIdx.x;
-  for (int e = threadIdx.x; e < COUT * CIN * 9; e += NET_TW * NET_TH) {
-    const int o = e / (CIN * 9), ct = e - o * (CIN * 9), c = ct / 9, t = ct - c * 9;
-    const int ty = t / 3, tx = t - 3 * ty;
-    float s0 = 0.0f, s1 = 0.0f;
-    for (int ly = 0; ly < NET_TH; ++ly) {
-      const float* xs = sx + c * NET_HP + (ly + ty) * NET_HW + tx;
-      const float* gs = sg + o * NET_TW * NET_TH + ly * NET_TW;
-#pragma unroll 8
-      for (int lx = 0; lx < NET_TW; lx += 2) {
-        s0 = fmaf(gs[lx], xs[lx], s0);
-        s1 = fmaf(gs[lx + 1], xs[lx + 1], s1);
+  const int grp = threadIdx.x / NP, pair = threadIdx.x - grp * NP;
+  const int o = pair % COUT, c = pair / COUT;
+  float s[2][9];
+#pragma unroll
+  for (int t = 0; t < 9; ++t) s[0][t] = s[1][t] = 0.0f;
+  if (grp < NG) {
+    for (int r = grp; r < NRUN; r += NG) {
+      const int ly = r / (NET_TW / 4), lx = 4 * (r - ly * (NET_TW / 4));
+      const float4 g4 = *reinterpret_cast<const float4*>(sg + o * GS + ly * NET_TW + lx);
+      const float g[4] = {g4.x, g4.y, g4.z, g4.w};
+#pragma unroll
+      for (int ty = 0; ty < 3; ++ty) {
+        float x[6];
+        net_row(sx + c * NET_HP + (ly + ty) * NET_XS + lx, x);
+#pragma unroll
+        for (int tx = 0; tx < 3; ++tx)
+#pragma unroll
+          for (int p = 0; p < 4; ++p) s[p & 1][3 * ty + tx] = fmaf(g[p], x[p + tx], s[p & 1][3 * ty + tx]);
       }
     }
-    partials[(int64_t)blk * (COUT * CIN * 9) + e] = s0 + s1;
+  }
+  float* out = partials + (int64_t)(blockIdx.y * gridDim.x + blockIdx.x) * NET_NW + off;
+  if (NG == 1) {
+#pragma unroll
+    for (int t = 0; t < 9; ++t) out[(o * CIN + c) * 9 + t] = s[0][t] + s[1][t];
+    return;
+  }
+  __syncthreads();                                           // the tiles are read
+  if (grp < NG) {
+#pragma unroll
+    for (int t = 0; t < 9; ++t) sh[grp * (NP * 9) + (o * CIN + c) * 9 + t] = s[0][t] + s[1][t];
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < NP * 9; e += NET_TW * NET_TH) {
+    float v = 0.0f;
+    for (int k = 0; k < NG; ++k) v += sh[k * (NP * 9) + e];
+    out[e] = v;
   }
 }
 
-// grad[off + e] += sum_b partials[b][e]
-__global__ void k_net_wgrad_reduce(const float* partials, int nblocks, int ne, float* grad) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= ne) return;
+// grad[e] += sum_b partials[b][e] over all layers: 32 entries per block, eight threads each
+// taking every eighth tile in FP64 (an FP64 addition is long: one thread per entry took 33 us
+// at 256 tiles).
+__global__ void __launch_bounds__(256) k_net_wgrad_reduce(const float* partials, int nblocks, float* grad) {
+  __shared__ double red[8][32];
+  const int lane = threadIdx.x & 31, part = threadIdx.x >> 5, e = blockIdx.x * 32 + lane;
   double s = 0.0;
-  for (int b = 0; b < nblocks; ++b) s += (double)partials[(int64_t)b * ne + e];
-  grad[e] += (float)s;
+  if (e < NET_NW)
+    for (int b = part; b < nblocks; b += 8) s += (double)partials[(int64_t)b * NET_NW + e];
+  red[part][lane] = s;
+  __syncthreads();
+  if (part == 0 && e < NET_NW) {
+    double t = 0.0;
+    for (int k = 0; k < 8; ++k) t += red[k][lane];
+    grad[e] += (float)t;
+  }
 }
 
 __global__ void k_net_adam(float* w, float* wq, float* m, float* v, float* grad, int n, float lr, float b1,
@@ -343,7 +420,7 @@ struct Bufs {
   float* rho;       // [cols]
   double* zz;       // [1]
   double* dpart;    // [cols][nb][2]
-  float* wpart;     // [tiles][2304]
+  float* wpart;     // [tiles][NET_NW]
 };
 
 int net_ws(bf_net* net, const bf_graph* g, int cols, bool train, Bufs* b) {
@@ -356,7 +433,7 @@ int net_ws(bf_net* net, const bf_graph* g, int cols, bool train, Bufs* b) {
   const size_t ntile = (size_t)((g->nx + NET_TW - 1) / NET_TW) * (size_t)((g->ny + NET_TH - 1) / NET_TH);
   size_t bytes = 2 * act + al(cols * sizeof(float)) + al(sizeof(double)) +
                  al((size_t)cols * nb_red * 2 * sizeof(double));
-  if (train) bytes += 2 * vec + 2 * act1 + al(ntile * NET_CH * NET_CH * 9 * sizeof(float));
+  if (train) bytes += 2 * vec + 2 * act1 + al(ntile * NET_NW * sizeof(float));
   if (bytes > net->ws_bytes) {
     if (net->ws) cudaFree(net->ws);
     net->ws = nullptr;
@@ -560,15 +637,11 @@ extern "C" int bf_net_accumulate(bf_net* net, const bf_graph* g, const float* r,
   const dim3 tg((unsigned)((a.nx + NET_TW - 1) / NET_TW), (unsigned)((a.ny + NET_TH - 1) / NET_TH));
   const int ntile = (int)(tg.x * tg.y);
   a.in = b.A2;
-  BF_LAUNCH((k_net_wgrad<NET_CH, 1, IN_RELU><<<tg, NET_TW * NET_TH, 0, s>>>(a, b.G3, b.wpart)));
-  BF_LAUNCH((k_net_wgrad_reduce<<<(NET_CH * 9 + 127) / 128, 128, 0, s>>>(b.wpart, ntile, NET_CH * 9, net->grad + NET_W3)));
+  BF_LAUNCH((k_net_wgrad<NET_CH, 1, IN_RELU><<<tg, NET_TW * NET_TH, 0, s>>>(a, b.G3, b.wpart, NET_W3)));
   a.in = b.A1;
-  BF_LAUNCH((k_net_wgrad<NET_CH, NET_CH, IN_RELU><<<tg, NET_TW * NET_TH, 0, s>>>(a, b.G2, b.wpart)));
-  BF_LAUNCH((k_net_wgrad_reduce<<<(NET_CH * NET_CH * 9 + 127) / 128, 128, 0, s>>>(b.wpart, ntile, NET_CH * NET_CH * 9,
-                                                                                   net->grad + NET_W2)));
-  BF_LAUNCH((k_net_wgrad<NET_CIN, NET_CH, IN_NET><<<tg, NET_TW * NET_TH, 0, s>>>(a, b.G1, b.wpart)));
-  BF_LAUNCH((k_net_wgrad_reduce<<<(NET_CH * NET_CIN * 9 + 127) / 128, 128, 0, s>>>(b.wpart, ntile, NET_CH * NET_CIN * 9,
-                                                                                    net->grad + NET_W1)));
+  BF_LAUNCH((k_net_wgrad<NET_CH, NET_CH, IN_RELU><<<tg, NET_TW * NET_TH, 0, s>>>(a, b.G2, b.wpart, NET_W2)));
+  BF_LAUNCH((k_net_wgrad<NET_CIN, NET_CH, IN_NET><<<tg, NET_TW * NET_TH, 0, s>>>(a, b.G1, b.wpart, NET_W1)));
+  BF_LAUNCH((k_net_wgrad_reduce<<<(NET_NW + 31) / 32, 256, 0, s>>>(b.wpart, ntile, net->grad)));
   BF_CUDA(cudaGetLastError());
   return BF_OK;
 }
