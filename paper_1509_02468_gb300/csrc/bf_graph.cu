@@ -607,10 +607,9 @@ __device__ __forceinline__ float rb_exp_ftz(float gi, float gj, float a_r, float
 }
 
 // The halo tile at (bx, by) into buf, by nw warps (this one is w); GUIDE: the guide too.
-template <int K, bool GUIDE>
+template <class TT, bool GUIDE>
 __device__ __forceinline__ void pipe_stage(const Geom<float>& g, const ApplyArgs<float>& a, int bx, int by, int lane,
                                            int w, int nw, unsigned char* buf) {
-  typedef PipeTile<K> TT;
   constexpr int NC4 = TT::nc4, STEP = 32 / NC4;         // pixels per instruction
   const unsigned sx = (unsigned)__cvta_generic_to_shared(buf);
   const unsigned sg = sx + (unsigned)TT::xbytes;
@@ -658,14 +657,14 @@ __global__ void __launch_bounds__(PipeTile<K>::threads + PIPE_STAGERS, 1) k_appl
   const int grp = rest % NG, strip = rest / NG;
   const int row0 = strip * RB_P;
   int t = blockIdx.x;
-  if (t < ntiles) pipe_stage<K, true>(g, a, (t % ntx) * TT::tw, (t / ntx) * TT::th, lx, rest, CW + SW, smem);
+  if (t < ntiles) pipe_stage<TT, true>(g, a, (t % ntx) * TT::tw, (t / ntx) * TT::th, lx, rest, CW + SW, smem);
   asm volatile("cp.async.wait_all;" ::: "memory");
   for (int b = 0; t < ntiles; t += gridDim.x, b ^= 1) {
     __syncthreads();                                     // tile t has landed, the other buffer is free
     if (stager) {
       const int tn = t + gridDim.x;
       if (tn < ntiles)
-        pipe_stage<K, true>(g, a, (tn % ntx) * TT::tw, (tn / ntx) * TT::th, lx, rest - CW, SW, smem + (b ^ 1) * TT::stage);
+        pipe_stage<TT, true>(g, a, (tn % ntx) * TT::tw, (tn / ntx) * TT::th, lx, rest - CW, SW, smem + (b ^ 1) * TT::stage);
       asm volatile("cp.async.wait_all;" ::: "memory");
       continue;
     }
@@ -737,6 +736,26 @@ __global__ void __launch_bounds__(PipeTile<K>::threads + PIPE_STAGERS, 1) k_appl
 // 1024 x 1024, K = 16, BF16: 470 us.)
 // The weight at byte offset `off` of the planes; volatile, so that the loads of a row stay
 // where they are issued.
+// Its tile: 12 computing warps (128 registers a thread with the two that copy), strips of two
+// pixels where a thread carries 16 columns: with four, the loads could only be issued two
+// steps ahead, 0.1 us before use, and the kernel waited for them (216 us).
+template <int K>
+struct PipeTileW {
+  static constexpr int threads = 384;
+  static constexpr int cs = K >= 16 ? 16 : K;
+  static constexpr int P = cs == 16 ? 2 : 4;
+  static constexpr int AHEAD = cs == 16 ? 8 : 5;          // steps between a load and its use
+  static constexpr int ng = K / cs;
+  static constexpr int strips = threads / (32 * ng);
+  static constexpr int tw = 32, th = P * strips;
+  static constexpr int hw = tw + 6, hh = th + 6, hp = hw * hh;
+  static constexpr int nc4 = K / 4;
+  static constexpr int cst = hp + ((10 - hp % 8) % 8);    // column-group stride, as in PipeTile
+  static constexpr size_t xbytes = (size_t)cst * nc4 * 16;
+  static constexpr size_t stage = xbytes;
+  static constexpr size_t smem = 2 * stage;
+};
+
 template <int WM>
 __device__ __forceinline__ float pipe_ld_w(const char* wf, unsigned off) {
   if (WM == BF_W_STORED_BF16) {
@@ -752,14 +771,14 @@ __device__ __forceinline__ float pipe_ld_w(const char* wf, unsigned off) {
 // Weights between the halo pixel (row r of the strip's rows, column x + dx) and the strip's
 // pixels (column x, rows y0 ..; off: byte offset of pixel (x, y0) in a plane).  MASK: 0 unless
 // pixel and neighbour lie in the image (nothing else is read then).
-template <int WM, bool MASK>
+template <int WM, bool MASK, int P>
 __device__ __forceinline__ void pipe_step_w(const void* wf, int n, int nx, int ny, int x, int y0, unsigned off, int r,
-                                            int dx, float (&w)[RB_P]) {
+                                            int dx, float (&w)[P]) {
   constexpr int ES = WM == BF_W_STORED_BF16 ? 2 : 4;
   // opaque: the offsets of a strip's 192 loads would be kept for all its steps, and spilled
   asm volatile("" : "+r"(n), "+r"(nx));
 #pragma unroll
-  for (int p = 0; p < RB_P; ++p) {
+  for (int p = 0; p < P; ++p) {
     const int dy = r - 3 - p;
     if (dy < -3 || dy > 3 || (dy == 0 && dx == 0)) continue;
     const bool fwd = dy > 0 || (dy == 0 && dx > 0);
@@ -775,19 +794,19 @@ __device__ __forceinline__ void pipe_step_w(const void* wf, int n, int nx, int n
 template <int K, int WM, bool MASK>
 __device__ __forceinline__ void pipe_tile_w(const Geom<float>& g, const ApplyArgs<float>& a, const float4* sx, int bx,
                                             int by, int lx, int grp, int row0) {
-  typedef PipeTile<K> TT;
-  constexpr int CS = TT::cs, CS4 = CS / 4;
+  typedef PipeTileW<K> TT;
+  constexpr int CS = TT::cs, CS4 = CS / 4, P = TT::P;
   const int x = bx + lx, y0 = by + row0;
   const int n = (int)a.n, nx = g.nx;
   const unsigned off = (unsigned)(y0 * nx + x) * (WM == BF_W_STORED_BF16 ? 2u : 4u);
-  unsigned long long acc2[RB_P][CS / 2], xi2[RB_P][CS / 2];
+  unsigned long long acc2[P][CS / 2], xi2[P][CS / 2];
   // steps (row, dx) in order, the weights loaded AHEAD steps before they are used
-  constexpr int AHEAD = MASK ? 1 : (CS >= 8 ? 2 : 4), RING = AHEAD + 1, STEPS = 7 * (RB_P + 6);
-  float w[RING][RB_P];
+  constexpr int AHEAD = MASK ? 2 : TT::AHEAD, RING = AHEAD + 1, STEPS = 7 * (P + 6);
+  float w[RING][P];
 #pragma unroll
-  for (int q = 0; q < AHEAD; ++q) pipe_step_w<WM, MASK>(a.wf, n, nx, g.ny, x, y0, off, q / 7, q % 7 - 3, w[q]);
+  for (int q = 0; q < AHEAD; ++q) pipe_step_w<WM, MASK, P>(a.wf, n, nx, g.ny, x, y0, off, q / 7, q % 7 - 3, w[q]);
 #pragma unroll
-  for (int p = 0; p < RB_P; ++p) {
+  for (int p = 0; p < P; ++p) {
     const int hp = (row0 + p + 3) * TT::hw + lx + 3;
 #pragma unroll
     for (int c4 = 0; c4 < CS4; ++c4) {
@@ -799,12 +818,12 @@ __device__ __forceinline__ void pipe_tile_w(const Geom<float>& g, const ApplyArg
     for (int c = 0; c < CS / 2; ++c) acc2[p][c] = 0ull;
   }
 #pragma unroll
-  for (int r = 0; r < RB_P + 6; ++r) {
+  for (int r = 0; r < P + 6; ++r) {
 #pragma unroll
   for (int dx = -3; dx <= 3; ++dx) {
     const int q = 7 * r + dx + 3;
     if (q + AHEAD < STEPS)
-      pipe_step_w<WM, MASK>(a.wf, n, nx, g.ny, x, y0, off, (q + AHEAD) / 7, (q + AHEAD) % 7 - 3, w[(q + AHEAD) % RING]);
+      pipe_step_w<WM, MASK, P>(a.wf, n, nx, g.ny, x, y0, off, (q + AHEAD) / 7, (q + AHEAD) % 7 - 3, w[(q + AHEAD) % RING]);
     const int hp = (row0 + r) * TT::hw + lx + 3 + dx;
     unsigned long long xj2[CS / 2];
 #pragma unroll
@@ -814,7 +833,7 @@ __device__ __forceinline__ void pipe_tile_w(const Geom<float>& g, const ApplyArg
       xj2[2 * c4 + 1] = v.y;
     }
 #pragma unroll
-    for (int p = 0; p < RB_P; ++p) {
+    for (int p = 0; p < P; ++p) {
       const int dy = r - 3 - p;
       if (dy < -3 || dy > 3 || (dy == 0 && dx == 0)) continue;
       const unsigned long long w2 = f2_pack(w[q % RING][p], w[q % RING][p]);
@@ -824,7 +843,7 @@ __device__ __forceinline__ void pipe_tile_w(const Geom<float>& g, const ApplyArg
   }
   }
 #pragma unroll
-  for (int p = 0; p < RB_P; ++p) {
+  for (int p = 0; p < P; ++p) {
     if (MASK && (x >= g.nx || y0 + p >= g.ny)) continue;
     float* yp = a.Y + ((int64_t)(y0 + p) * g.nx + x) * a.ldy + grp * CS;
 #pragma unroll
@@ -834,10 +853,10 @@ __device__ __forceinline__ void pipe_tile_w(const Geom<float>& g, const ApplyArg
 }
 
 template <int K, int WM>
-__global__ void __launch_bounds__(PipeTile<K>::threads + PIPE_STAGERS, 1)
+__global__ void __launch_bounds__(PipeTileW<K>::threads + PIPE_STAGERS, 1)
 k_apply_pipe_w(const __grid_constant__ Geom<float> g, const ApplyArgs<float> a) {
   bf_pdl_enter();
-  typedef PipeTile<K> TT;
+  typedef PipeTileW<K> TT;
   extern __shared__ __align__(16) unsigned char smem[];
   const int ntx = (g.nx + TT::tw - 1) / TT::tw;
   const int ntiles = ntx * ((g.ny + TT::th - 1) / TT::th);
@@ -845,16 +864,16 @@ k_apply_pipe_w(const __grid_constant__ Geom<float> g, const ApplyArgs<float> a) 
   const int rest = threadIdx.x >> 5;
   constexpr int CW = TT::threads / 32, SW = PIPE_STAGERS / 32;
   const bool stager = rest >= CW;
-  const int grp = rest % TT::ng, row0 = (rest / TT::ng) * RB_P;
+  const int grp = rest % TT::ng, row0 = (rest / TT::ng) * TT::P;
   int t = blockIdx.x;
-  if (t < ntiles) pipe_stage<K, false>(g, a, (t % ntx) * TT::tw, (t / ntx) * TT::th, lx, rest, CW + SW, smem);
+  if (t < ntiles) pipe_stage<TT, false>(g, a, (t % ntx) * TT::tw, (t / ntx) * TT::th, lx, rest, CW + SW, smem);
   asm volatile("cp.async.wait_all;" ::: "memory");
   for (int b = 0; t < ntiles; t += gridDim.x, b ^= 1) {
     __syncthreads();                                     // tile t has landed, the other buffer is free
     if (stager) {
       const int tn = t + gridDim.x;
       if (tn < ntiles)
-        pipe_stage<K, false>(g, a, (tn % ntx) * TT::tw, (tn / ntx) * TT::th, lx, rest - CW, SW, smem + (b ^ 1) * TT::stage);
+        pipe_stage<TT, false>(g, a, (tn % ntx) * TT::tw, (tn / ntx) * TT::th, lx, rest - CW, SW, smem + (b ^ 1) * TT::stage);
       asm volatile("cp.async.wait_all;" ::: "memory");
       continue;
     }
@@ -894,7 +913,8 @@ static int launch_apply_pipe(const bf_graph* g, const ApplyArgs<float>& a, cudaS
 
 template <int K, int WM>
 static int launch_apply_pipe_w(const bf_graph* g, const ApplyArgs<float>& a, cudaStream_t s) {
-  typedef PipeTile<K> TT;
+  typedef PipeTileW<K> TT;
+  static_assert(TT::smem <= 227 * 1024, "stored-weight apply tile does not fit in shared memory");
   {
     const int rc_ = bf_smem_attr((const void*)k_apply_pipe_w<K, WM>, (int)TT::smem, "cudaFuncSetAttribute(k_apply_pipe_w)");
     if (rc_) return rc_;

@@ -66,7 +66,10 @@ struct NetArgs {
   int64_t ldr;
   const float* guide;
   const float* d;
-  const float* rho;      // [cols]
+  float* rho;            // [cols]
+  const double* rpart;   // IN_NET layers: block sums of k_net_sums, [cols][nrp][2]
+  int nrp;
+  double* zz;            // [1] or NULL
   const float* in;       // [cols][n][cin] activations
   float* out;            // [cols][n][cout]
   const float* mask;     // OUT_MASKED: [cols][n][cout] pre-activations
@@ -79,9 +82,34 @@ struct NetArgs {
 
 __device__ __forceinline__ float bf16_round(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
 
+// rho[col] = sqrt(mean) and zz = sum z^2 (column 0) from the block sums of k_net_sums, added
+// in the same order by every block of the first layer (a launch of its own took longer);
+// block (0, 0) of the column keeps them for the kernels after it.
+__device__ __forceinline__ float net_rho(const NetArgs& a, int col) {
+  __shared__ float sh;
+  if (threadIdx.x < 32) {
+    double a0 = 0.0, a1 = 0.0;
+    for (int b = threadIdx.x; b < a.nrp; b += 32) {
+      a0 += a.rpart[((int64_t)col * a.nrp + b) * 2];
+      a1 += a.rpart[((int64_t)col * a.nrp + b) * 2 + 1];
+    }
+    a0 = warp_sum(a0);
+    a1 = warp_sum(a1);
+    if (threadIdx.x == 0) {
+      sh = (float)sqrt(a0 / (double)a.n);
+      if (blockIdx.x == 0 && blockIdx.y == 0) {
+        a.rho[col] = sh;
+        if (a.zz && col == 0) *a.zz = a1;
+      }
+    }
+  }
+  __syncthreads();
+  return sh;
+}
+
 // Stage the input tile (with halo) channel-major: s[c * NET_HP + hp].
 template <int CIN, int IN>
-__device__ __forceinline__ void net_stage(const NetArgs& a, int col, int bx, int by, float* s) {
+__device__ __forceinline__ void net_stage(const NetArgs& a, const float* in, int col, float rh, int bx, int by, float* s) {
   for (int q = threadIdx.x; q < NET_HW * NET_HH; q += NET_TW * NET_TH) {
     const int hy = q / NET_HW, hx = q - hy * NET_HW, hp = hy * NET_XS + hx;
     const int gy = by - 1 + hy, gx = bx - 1 + hx;
@@ -90,7 +118,6 @@ __device__ __forceinline__ void net_stage(const NetArgs& a, int col, int bx, int
     if (IN == IN_NET) {
       float c0 = 0.0f, c1 = 0.0f, c2 = 0.0f;
       if (inside) {
-        const float rh = a.rho[col];
         const float di = a.d[i];
         c0 = rh > 0.0f ? a.r[i * a.ldr + col] / (di * rh) : 0.0f;
         c1 = a.guide[i];
@@ -100,7 +127,7 @@ __device__ __forceinline__ void net_stage(const NetArgs& a, int col, int bx, int
       s[1 * NET_HP + hp] = c1;
       s[2 * NET_HP + hp] = c2;
     } else {
-      const float* src = a.in + ((int64_t)col * a.n + i) * CIN;
+      const float* src = in + ((int64_t)col * a.n + i) * CIN;
 #pragma unroll
       for (int c4 = 0; c4 < CIN; c4 += 4) {
         float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
@@ -144,6 +171,7 @@ template <int CIN, int COUT, int IN, int OUT>
 __global__ void __launch_bounds__(NET_TW * NET_TH) k_net_conv(const NetArgs a) {
   static_assert(COUT == NET_CH || (COUT == 1 && CIN % 4 == 0), "layer shapes of the net");
   constexpr int COUTP = (COUT + 3) & ~3;
+  bf_pdl_enter();
   if (a.stop && *a.stop != 0) return;
   __shared__ __align__(16) float sx[CIN * NET_HP];
   __shared__ __align__(16) float sw[CIN * 9 * COUTP];       // [c][tap][o]
@@ -155,7 +183,8 @@ __global__ void __launch_bounds__(NET_TW * NET_TH) k_net_conv(const NetArgs a) {
     if (o < COUT) wv = a.transpose ? a.w[(c * COUT + o) * 9 + (8 - t)] : a.w[(o * CIN + c) * 9 + t];
     sw[e] = wv;
   }
-  net_stage<CIN, IN>(a, col, bx, by, sx);
+  const float rh = IN == IN_NET ? net_rho(a, col) : 0.0f;
+  net_stage<CIN, IN>(a, a.in, col, rh, bx, by, sx);
   __syncthreads();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, grp = wid >> 1;
   const int lx = 4 * (lane & 7), ly = 4 * (wid & 1) + (lane >> 3);
@@ -231,6 +260,7 @@ __global__ void __launch_bounds__(NET_TW * NET_TH) k_net_conv(const NetArgs a) {
 // Per-block sums for rho (sum (r/d)^2) and, with z, sum z^2; blockIdx.y is the column.
 __global__ void __launch_bounds__(256) k_net_sums(const float* r, int64_t ldr, const float* d, const float* z,
                                                   int64_t n, double* partials, const int* stop) {
+  bf_pdl_enter();
   if (stop && *stop != 0) return;
   __shared__ double red[2 * 8];
   const int col = blockIdx.y;
@@ -258,27 +288,10 @@ __global__ void __launch_bounds__(256) k_net_sums(const float* r, int64_t ldr, c
   }
 }
 
-// rho[col] = sqrt(mean), zz = sum z^2 (column 0), summed over blocks in order.
-__global__ void k_net_rho(const double* partials, int nblocks, int64_t n, float* rho, double* zz,
-                          const int* stop) {
-  if (stop && *stop != 0) return;
-  const int col = blockIdx.x;
-  double a0 = 0.0, a1 = 0.0;
-  for (int b = threadIdx.x; b < nblocks; b += 32) {
-    a0 += partials[((int64_t)col * nblocks + b) * 2];
-    a1 += partials[((int64_t)col * nblocks + b) * 2 + 1];
-  }
-  a0 = warp_sum(a0);
-  a1 = warp_sum(a1);
-  if (threadIdx.x == 0) {
-    rho[col] = (float)sqrt(a0 / (double)n);
-    if (zz && col == 0) *zz = a1;
-  }
-}
-
 // G3 = 2 rho (rho O - z) / zz and per-block sums of (rho O - z)^2.
 __global__ void __launch_bounds__(256) k_net_loss(const float* O, const float* z, const float* rho,
                                                   const double* zz, int64_t n, float* G3, double* partials) {
+  bf_pdl_enter();
   __shared__ double red[8];
   const float rh = rho[0];
   const float sc = (float)(2.0 * (double)rh / *zz);
@@ -298,27 +311,22 @@ __global__ void __launch_bounds__(256) k_net_loss(const float* O, const float* z
   }
 }
 
-__global__ void k_net_loss_final(const double* partials, int nblocks, const double* zz, double* loss) {
-  double t = 0.0;
-  for (int b = threadIdx.x; b < nblocks; b += 32) t += partials[b];
-  t = warp_sum(t);
-  if (threadIdx.x == 0) *loss += t / *zz;
-}
-
+#define NET_WGRAD_FLOATS (NET_CH * NET_HP + NET_CH * (NET_TW * NET_TH + 4))
 // Per-block weight gradient dW[o][c][t] = sum_px G[px][o] X[px + t][c] over the block's
 // tile (X staged like a conv input); partials[block][off + (o * CIN + c) * 9 + t].  A thread
 // owns the nine taps of one pair (o, c) over a share of the tile's runs of four pixels (each
 // sum in two parts, even and odd pixels); the shares are added in order.
 template <int CIN, int COUT, int IN>
-__global__ void __launch_bounds__(NET_TW * NET_TH) k_net_wgrad(const NetArgs a, const float* G, float* partials, int off) {
+__device__ __forceinline__ void net_wgrad(const NetArgs& a, const float* in, const float* G, float* partials, int off,
+                                          float* sh) {
   constexpr int NP = COUT * CIN, NG = (NET_TW * NET_TH / NP < 16) ? NET_TW * NET_TH / NP : 16;
   constexpr int NRUN = NET_TW * NET_TH / 4, GS = NET_TW * NET_TH + 4;   // gradient channel stride
   constexpr int XF = CIN * NET_HP, GF = COUT * GS, RF = NG > 1 ? NG * NP * 9 : 0;
-  __shared__ __align__(16) float sh[(XF + GF > RF) ? XF + GF : RF];
+  static_assert(XF + GF <= NET_WGRAD_FLOATS && RF <= NET_WGRAD_FLOATS, "shared memory of k_net_wgrad");
   float* sx = sh;
   float* sg = sh + XF;                                       // [o][px]
   const int bx = blockIdx.x * NET_TW, by = blockIdx.y * NET_TH;
-  net_stage<CIN, IN>(a, 0, bx, by, sx);
+  net_stage<CIN, IN>(a, in, 0, IN == IN_NET ? a.rho[0] : 0.0f, bx, by, sx);
   for (int e = threadIdx.x; e < COUT * NET_TW * NET_TH; e += NET_TW * NET_TH) {
     const int p = e / COUT, o = e - p * COUT;
     const int ly = p / NET_TW, lx = p - ly * NET_TW;
@@ -366,11 +374,34 @@ __global__ void __launch_bounds__(NET_TW * NET_TH) k_net_wgrad(const NetArgs a, 
   }
 }
 
+// The three layers' gradients of a tile in one launch, blockIdx.z the layer (the largest
+// first): dW2 = corr(G2, relu(A1)), dW1 = corr(G1, C), dW3 = corr(G3, relu(A2)).
+__global__ void __launch_bounds__(NET_TW * NET_TH)
+k_net_wgrad(const NetArgs a, const float* A1, const float* A2, const float* G1, const float* G2, const float* G3,
+            float* partials) {
+  bf_pdl_enter();
+  __shared__ __align__(16) float sh[NET_WGRAD_FLOATS];
+  if (blockIdx.z == 0) net_wgrad<NET_CH, NET_CH, IN_RELU>(a, A1, G2, partials, NET_W2, sh);
+  else if (blockIdx.z == 1) net_wgrad<NET_CIN, NET_CH, IN_NET>(a, nullptr, G1, partials, NET_W1, sh);
+  else net_wgrad<NET_CH, 1, IN_RELU>(a, A2, G3, partials, NET_W3, sh);
+}
+
 // grad[e] += sum_b partials[b][e] over all layers: 32 entries per block, eight threads each
 // taking every eighth tile in FP64 (an FP64 addition is long: one thread per entry took 33 us
 // at 256 tiles).
-__global__ void __launch_bounds__(256) k_net_wgrad_reduce(const float* partials, int nblocks, float* grad) {
+// The block past the entries adds the pair's loss, the sum of k_net_loss's block sums / zz.
+__global__ void __launch_bounds__(256) k_net_wgrad_reduce(const float* partials, int nblocks, float* grad,
+                                                          const double* lpart, int nl, const double* zz, double* loss) {
+  bf_pdl_enter();
   __shared__ double red[8][32];
+  if (blockIdx.x == gridDim.x - 1) {
+    if (threadIdx.x >= 32) return;
+    double t = 0.0;
+    for (int b = threadIdx.x; b < nl; b += 32) t += lpart[b];
+    t = warp_sum(t);
+    if (threadIdx.x == 0) *loss += t / *zz;
+    return;
+  }
   const int lane = threadIdx.x & 31, part = threadIdx.x >> 5, e = blockIdx.x * 32 + lane;
   double s = 0.0;
   if (e < NET_NW)
@@ -423,9 +454,12 @@ struct Bufs {
   float* wpart;     // [tiles][NET_NW]
 };
 
+// blocks of the sums over the pixels: few, as every block of the first layer adds them
+int net_sum_blocks(int64_t n) { return (int)std::min<int64_t>((n + 255) / 256, 256); }
+
 int net_ws(bf_net* net, const bf_graph* g, int cols, bool train, Bufs* b) {
   const int64_t n = g->n;
-  const int nb_red = (int)std::min<int64_t>((n + 255) / 256, 1024);
+  const int nb_red = net_sum_blocks(n);
   auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
   const size_t act = al((size_t)cols * n * NET_CH * sizeof(float));
   const size_t vec = al((size_t)n * sizeof(float));
@@ -476,18 +510,17 @@ NetArgs net_args(const bf_net* net, const bf_graph* g) {
 template <int CIN, int COUT, int IN, int OUT>
 int launch_conv(const NetArgs& a, int cols, cudaStream_t s) {
   const dim3 grid((unsigned)((a.nx + NET_TW - 1) / NET_TW), (unsigned)((a.ny + NET_TH - 1) / NET_TH), (unsigned)cols);
-  BF_LAUNCH((k_net_conv<CIN, COUT, IN, OUT><<<grid, NET_TW * NET_TH, 0, s>>>(a)));
+  BF_LAUNCH_PDL((k_net_conv<CIN, COUT, IN, OUT>), grid, NET_TW * NET_TH, 0, s, a);
   BF_CUDA(cudaGetLastError());
   return BF_OK;
 }
 
-// rho of `cols` columns of r (and zz of z when given)
+// the block sums for rho of `cols` columns of r (and zz of z when given)
 int net_sums(const bf_graph* g, const float* r, int64_t ldr, const float* z, int cols, const Bufs& b,
              cudaStream_t s, const int* stop = nullptr) {
   const int64_t n = g->n;
-  const int nb = (int)std::min<int64_t>((n + 255) / 256, 1024);
-  BF_LAUNCH((k_net_sums<<<dim3(nb, cols), 256, 0, s>>>(r, ldr, (const float*)g->d, z, n, b.dpart, stop)));
-  BF_LAUNCH((k_net_rho<<<cols, 32, 0, s>>>(b.dpart, nb, n, b.rho, z ? b.zz : nullptr, stop)));
+  const int nb = net_sum_blocks(n);
+  BF_LAUNCH_PDL(k_net_sums, dim3(nb, cols), 256, 0, s, r, ldr, (const float*)g->d, z, n, b.dpart, stop);
   BF_CUDA(cudaGetLastError());
   return BF_OK;
 }
@@ -519,6 +552,9 @@ int bf_net_apply_f32(const bf_net* net_c, const bf_graph* g, const float* R, int
     a.r = R + c0;
     a.ldr = ldr;
     a.rho = b.rho;
+    a.rpart = b.dpart;
+    a.nrp = net_sum_blocks(g->n);
+    a.zz = nullptr;
     a.w = net->wq + NET_W1;
     a.out = b.A1;
     if ((rc = launch_conv<NET_CIN, NET_CH, IN_NET, OUT_ACT>(a, cols, s))) return rc;
@@ -603,6 +639,9 @@ extern "C" int bf_net_accumulate(bf_net* net, const bf_graph* g, const float* r,
   a.r = r;
   a.ldr = 1;
   a.rho = b.rho;
+  a.rpart = b.dpart;
+  a.nrp = net_sum_blocks(g->n);
+  a.zz = b.zz;
   // forward, keeping the pre-activations
   a.w = net->wq + NET_W1;
   a.out = b.A1;
@@ -617,9 +656,8 @@ extern "C" int bf_net_accumulate(bf_net* net, const bf_graph* g, const float* r,
   if ((rc = launch_conv<NET_CH, 1, IN_RELU, OUT_ACT>(a, 1, s))) return rc;
   // loss and dL/dO
   const int64_t n = g->n;
-  const int nb = (int)std::min<int64_t>((n + 255) / 256, 1024);
-  BF_LAUNCH((k_net_loss<<<nb, 256, 0, s>>>(b.O, z, b.rho, b.zz, n, b.G3, b.dpart)));
-  BF_LAUNCH((k_net_loss_final<<<1, 32, 0, s>>>(b.dpart, nb, b.zz, net->loss)));
+  const int nb = net_sum_blocks(n);
+  BF_LAUNCH_PDL(k_net_loss, nb, 256, 0, s, b.O, z, b.rho, b.zz, n, b.G3, b.dpart);
   // backward: G2 = conv^T(G3, W3) * (A2 > 0), G1 = conv^T(G2, W2) * (A1 > 0)
   a.transpose = 1;
   a.in = b.G3;
@@ -633,15 +671,12 @@ extern "C" int bf_net_accumulate(bf_net* net, const bf_graph* g, const float* r,
   a.mask = b.A1;
   if ((rc = launch_conv<NET_CH, NET_CH, IN_PLAIN, OUT_MASKED>(a, 1, s))) return rc;
   a.transpose = 0;
-  // weight gradients: dW3 = corr(G3, relu(A2)), dW2 = corr(G2, relu(A1)), dW1 = corr(G1, C)
+  // weight gradients
   const dim3 tg((unsigned)((a.nx + NET_TW - 1) / NET_TW), (unsigned)((a.ny + NET_TH - 1) / NET_TH));
   const int ntile = (int)(tg.x * tg.y);
-  a.in = b.A2;
-  BF_LAUNCH((k_net_wgrad<NET_CH, 1, IN_RELU><<<tg, NET_TW * NET_TH, 0, s>>>(a, b.G3, b.wpart, NET_W3)));
-  a.in = b.A1;
-  BF_LAUNCH((k_net_wgrad<NET_CH, NET_CH, IN_RELU><<<tg, NET_TW * NET_TH, 0, s>>>(a, b.G2, b.wpart, NET_W2)));
-  BF_LAUNCH((k_net_wgrad<NET_CIN, NET_CH, IN_NET><<<tg, NET_TW * NET_TH, 0, s>>>(a, b.G1, b.wpart, NET_W1)));
-  BF_LAUNCH((k_net_wgrad_reduce<<<(NET_NW + 31) / 32, 256, 0, s>>>(b.wpart, ntile, net->grad)));
+  BF_LAUNCH_PDL(k_net_wgrad, dim3(tg.x, tg.y, 3), NET_TW * NET_TH, 0, s, a, b.A1, b.A2, b.G1, b.G2, b.G3, b.wpart);
+  BF_LAUNCH_PDL(k_net_wgrad_reduce, (NET_NW + 31) / 32 + 1, 256, 0, s, b.wpart, ntile, net->grad, b.dpart, nb, b.zz,
+                net->loss);
   BF_CUDA(cudaGetLastError());
   return BF_OK;
 }
