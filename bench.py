@@ -917,7 +917,7 @@ def _run_batched(bf, torch, stream, kmax=50, reps=3):
                                "includes the host read of the barrier flag",
             "plain_mpix_s": total / (ms_p * 1e-3) / 1e6, "plain_ms": ms_p,
             "batched_kernels_per_run": lb, "tile_shape_timings_ms": tune_ms,
-            "tile_shape": ["32x8", "64x4", "16x16"][variant]}
+            "tile_shape": ["64x16", "32x32", "128x8"][variant]}
 
 
 def run_case(args):

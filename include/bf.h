@@ -407,7 +407,7 @@ int bf_batch_cg_persistent(bf_batch* b, const float* const* x0, float* const* x_
 int bf_batch_lobpcg(bf_batch* b, const float* const* X0, int k, int kmax, const bf_lobpcg_opts* opts,
                     double* const* theta_out, float* const* y_out, int nstreams, bf_info* infos, void* stream);
 /* Autotuner: time `iters` iterations with each candidate tile shape of the image class
- * (32 x 8, 64 x 4, 16 x 16 pixels) on these vectors and keep the fastest; ms_out (host,
+ * (64 x 16, 32 x 32, 128 x 8 pixels) on these vectors and keep the fastest; ms_out (host,
  * 3 floats) receives the timings.  Synchronises the stream. */
 int bf_batch_tune(bf_batch* b, const float* const* x0, float* const* x_out, int iters,
                   float* ms_out, void* stream);

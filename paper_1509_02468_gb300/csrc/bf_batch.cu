@@ -21,6 +21,7 @@
 #include <vector>
 
 #include "bf_internal.cuh"
+#include "bf_run.cuh"
 #include "bf_window_fast.cuh"
 
 namespace {
@@ -92,6 +93,185 @@ __device__ __forceinline__ bool inst_sum_last(const double (&blk)[NV], const BAr
   return threadIdx.x == 0;
 }
 
+// The window constants of a class, by kernel parameter.
+struct BGeom {
+  Geom<float> g;
+  RunConst rc;               // image class
+};
+
+// Tiles of the image class: TW x TH pixels by runs of four (bf_run.cuh), a warp 32 x 4.
+template <int TW, int TH>
+struct RunShape {
+  static constexpr int tw = TW, th = TH, xs = TW + 8, hh = TH + 2 * RUN_R, hp = xs * hh;
+  static_assert((TW / 32) * (TH / 4) == BF_THREADS / 32, "a warp per 32 x 4 pixels");
+};
+
+// Stage f(gp) (0 outside the image) and the guide (+inf outside) of the tile and its halo;
+// vec: rows are whole aligned vectors, f4(gp) gives four values at once.
+template <class SH, class F, class F4>
+__device__ __forceinline__ void bstage_run(const RunConst& c, const BInst& in, int bx, int by, bool vec, float* sx,
+                                           float* sg, F f, F4 f4) {
+  const float inf = __int_as_float(0x7f800000);
+  if (vec) {
+    for (int q = threadIdx.x; q < SH::hp / 4; q += BF_THREADS) {
+      const int hy = q / (SH::xs / 4), h4 = q - hy * (SH::xs / 4);
+      const int gy = by - RUN_R + hy, gx = bx - 4 + 4 * h4;
+      float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f), gv = make_float4(inf, inf, inf, inf);
+      if ((unsigned)gx < (unsigned)in.nx && (unsigned)gy < (unsigned)in.ny) {
+        const int64_t gp = (int64_t)gy * in.nx + gx;
+        v = f4(gp);
+        gv = c.use_guide ? *reinterpret_cast<const float4*>(in.guide + gp) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      }
+      *reinterpret_cast<float4*>(sx + 4 * q) = v;
+      *reinterpret_cast<float4*>(sg + 4 * q) = gv;
+    }
+    return;
+  }
+  for (int hy = threadIdx.x >> 5; hy < SH::hh; hy += BF_THREADS / 32) {
+#pragma unroll
+    for (int h0 = 0; h0 < SH::xs; h0 += 32) {
+      const int hx = h0 + (threadIdx.x & 31);
+      if (hx >= SH::xs) continue;
+      const int gy = by - RUN_R + hy, gx = bx - 4 + hx;
+      float v = 0.0f, gv = inf;
+      if ((unsigned)gx < (unsigned)in.nx && (unsigned)gy < (unsigned)in.ny) {
+        const int64_t gp = (int64_t)gy * in.nx + gx;
+        v = f(gp);
+        gv = c.use_guide ? in.guide[gp] : 0.0f;
+      }
+      sx[hy * SH::xs + hx] = v;
+      sg[hy * SH::xs + hx] = gv;
+    }
+  }
+}
+__device__ __forceinline__ float4 bld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+
+// Walk the group's tiles: stage(bx, by) fills (sx, sg), epi(x0, y, cnt, i0, vi, acc) takes
+// the sums of the thread's run.
+template <class SH, class Stage, class Epi>
+__device__ __forceinline__ void brun_tiles(const RunConst& c, const BInst& in, const BJob& jb, float* sx, float* sg,
+                                           Stage stage, Epi epi) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int cx = 32 * (wid % (SH::tw / 32)) + 4 * (lane & 7), ry = 4 * (wid / (SH::tw / 32)) + (lane >> 3);
+  for (int t = 0; t < jb.nt; ++t) {
+    const int bx = jb.bx + t * SH::tw;
+    if (t) __syncthreads();                         // the previous tile is read
+    stage(bx, jb.by);
+    __syncthreads();
+    float vi[RUN_P], acc[RUN_P], ws[RUN_P];
+    run_sums<true, false>(c, sx + ry * SH::xs + cx, sg + ry * SH::xs + cx, SH::xs, vi, acc, ws);
+    const int x0 = bx + cx, y = jb.by + ry, cnt = run_count(x0, y, in.nx, in.ny);
+    if (cnt) epi(cnt, (int64_t)y * in.nx + x0, vi, acc);
+  }
+}
+
+// State of an instance from the sums s^T r, s^T s, r^T r, x0^T x0.
+__device__ __forceinline__ void binit_state(BState& st, const double* tot, float shift) {
+  st.sr = tot[0];
+  st.ss = tot[1];
+  st.rr = tot[2];
+  const double b2 = (double)shift * (double)shift * tot[3];
+  st.ref2 = b2 > 0.0 ? b2 : tot[2];
+  st.beta = 0.0;
+  st.alpha = 0.0;
+  st.iter = 0;
+  st.status = (isfinite(tot[0]) && isfinite(tot[1]) && isfinite(tot[2])) ? B_RUN : B_NONFINITE;
+}
+__device__ __forceinline__ void bdir_state(BState& st, double pq) {
+  st.pq = pq;
+  if (st.sr == 0.0) st.status = B_CONV;
+  else if (!isfinite(pq)) st.status = B_NONFINITE;
+  else if (!(pq > 0.0)) st.status = B_BREAK;
+  else st.alpha = st.sr / pq;
+}
+
+// bcg_init_job and bcg_dir_job (below) of the image class, by runs: a tile of 1024 pixels per
+// pass instead of 256 with one pixel per thread (64 instances of 64 .. 512 pixels a side:
+// the class's direction kernel 88 us before).
+template <class SH>
+__device__ __forceinline__ void bcg_init_run(const RunConst& c, const BArgs& a, int job, unsigned char* smem) {
+  __shared__ double red[4 * (BF_THREADS / 32)];
+  __shared__ int last;
+  float* sx = reinterpret_cast<float*>(smem);
+  float* sg = sx + SH::hp;
+  const BJob jb = a.jobs[job];
+  BInst& in = a.inst[jb.inst];
+  const bool rows = in.nx % 4 == 0, vec = rows && ((uintptr_t)in.x0 & 15) == 0, vecx = rows && ((uintptr_t)in.x & 15) == 0;
+  float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+  brun_tiles<SH>(
+      c, in, jb, sx, sg,
+      [&](int bx, int by) {
+        bstage_run<SH>(c, in, bx, by, vec, sx, sg, [&](int64_t gp) { return in.x0[gp]; },
+                       [&](int64_t gp) { return bld4(in.x0 + gp); });
+      },
+      [&](int cnt, int64_t i0, const float (&xi)[RUN_P], const float (&acc)[RUN_P]) {
+        float r[RUN_P], sv[RUN_P], di[RUN_P];
+        if (in.dinv) run_load(in.dinv, i0, cnt, rows, di);
+#pragma unroll
+        for (int j = 0; j < RUN_P; ++j) {
+          r[j] = sv[j] = 0.0f;
+          if (j >= cnt) continue;
+          r[j] = -acc[j];
+          sv[j] = in.dinv ? r[j] * di[j] : r[j];
+          v[0] = fmaf(sv[j], r[j], v[0]);
+          v[1] = fmaf(sv[j], sv[j], v[1]);
+          v[2] = fmaf(r[j], r[j], v[2]);
+          v[3] = fmaf(xi[j], xi[j], v[3]);
+        }
+        run_store(in.x, i0, cnt, vecx, xi);
+        run_store(in.r, i0, cnt, rows, r);
+        run_store(in.s, i0, cnt, rows, sv);
+      });
+  double blk[4], tot[4];
+  block_sum<4, float>(v, red, blk);
+  if (inst_sum_last<4>(blk, a, in, job, tot, &last, in.job0, in.njobs)) binit_state(in.st, tot, a.shift);
+}
+
+template <class SH>
+__device__ __forceinline__ void bcg_dir_run(const RunConst& c, const BArgs& a, int job, unsigned char* smem) {
+  const BJob jb = a.jobs[job];
+  BInst& in = a.inst[jb.inst];
+  if (in.st.status != B_RUN) return;
+  __shared__ double red[BF_THREADS / 32];
+  __shared__ int last;
+  float* sx = reinterpret_cast<float*>(smem);
+  float* sg = sx + SH::hp;
+  const int it = in.st.iter;
+  const float* p_old = in.p[it & 1];
+  const float* s = in.s;
+  float* p_new = in.p[(it + 1) & 1];
+  const float beta = (float)in.st.beta;
+  const bool vec = in.nx % 4 == 0;
+  float v[1] = {0.0f};
+  brun_tiles<SH>(
+      c, in, jb, sx, sg,
+      [&](int bx, int by) {
+        if (it == 0)
+          bstage_run<SH>(c, in, bx, by, vec, sx, sg, [&](int64_t gp) { return s[gp]; },
+                         [&](int64_t gp) { return bld4(s + gp); });
+        else
+          bstage_run<SH>(c, in, bx, by, vec, sx, sg, [&](int64_t gp) { return fmaf(beta, p_old[gp], s[gp]); },
+                         [&](int64_t gp) {
+                           const float4 o = bld4(p_old + gp), t = bld4(s + gp);
+                           return make_float4(fmaf(beta, o.x, t.x), fmaf(beta, o.y, t.y), fmaf(beta, o.z, t.z),
+                                              fmaf(beta, o.w, t.w));
+                         });
+      },
+      [&](int cnt, int64_t i0, const float (&pi)[RUN_P], const float (&acc)[RUN_P]) {
+        float q[RUN_P];
+#pragma unroll
+        for (int j = 0; j < RUN_P; ++j) {
+          q[j] = fmaf(a.shift, pi[j], acc[j]);
+          if (j < cnt) v[0] = fmaf(pi[j], q[j], v[0]);
+        }
+        run_store(p_new, i0, cnt, vec, pi);
+        run_store(in.q, i0, cnt, vec, q);
+      });
+  double blk[1], tot[1];
+  block_sum<1, float>(v, red, blk);
+  if (inst_sum_last<1>(blk, a, in, job, tot, &last, in.job0, in.njobs)) bdir_state(in.st, tot[0]);
+}
+
 template <class SH, class F>
 __device__ __forceinline__ void bstage(const BInst& in, int bx, int by, float* sx, float* sg, float* sval, F f) {
   for (int hp = threadIdx.x; hp < SH::hp; hp += BF_THREADS) {
@@ -149,25 +329,9 @@ __device__ __forceinline__ void bcg_init_job(const Geom<float>& g, const BArgs& 
   }
   double blk[4], tot[4];
   block_sum<4, float>(v, red, blk);
-  if (inst_sum_last<4>(blk, a, in, job, tot, &last, in.job0, in.njobs)) {
-    BState& st = in.st;
-    st.sr = tot[0];
-    st.ss = tot[1];
-    st.rr = tot[2];
-    const double b2 = (double)a.shift * (double)a.shift * tot[3];
-    st.ref2 = b2 > 0.0 ? b2 : tot[2];
-    st.beta = 0.0;
-    st.alpha = 0.0;
-    st.iter = 0;
-    st.status = (isfinite(tot[0]) && isfinite(tot[1]) && isfinite(tot[2])) ? B_RUN : B_NONFINITE;
-  }
+  if (inst_sum_last<4>(blk, a, in, job, tot, &last, in.job0, in.njobs)) binit_state(in.st, tot, a.shift);
 }
 
-template <class SH>
-__global__ void __launch_bounds__(BF_THREADS) k_bcg_init(const Geom<float> g, const BArgs a) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  bcg_init_job<SH>(g, a, blockIdx.x, smem);
-}
 
 // p = s + beta p_old on tile + halo (first iteration: p = s), q = (L + shift I) p, p^T q, alpha.
 // (An instance's status changes only in the last block of its jobs in a phase, after all
@@ -213,20 +377,32 @@ __device__ __forceinline__ void bcg_dir_job(const Geom<float>& g, const BArgs& a
   }
   double blk[1], tot[1];
   block_sum<1, float>(v, red, blk);
-  if (inst_sum_last<1>(blk, a, in, job, tot, &last, in.job0, in.njobs)) {
-    BState& st = in.st;
-    st.pq = tot[0];
-    if (st.sr == 0.0) st.status = B_CONV;
-    else if (!isfinite(tot[0])) st.status = B_NONFINITE;
-    else if (!(tot[0] > 0.0)) st.status = B_BREAK;
-    else st.alpha = st.sr / tot[0];
-  }
+  if (inst_sum_last<1>(blk, a, in, job, tot, &last, in.job0, in.njobs)) bdir_state(in.st, tot[0]);
+}
+
+template <class SH> struct BIsRun { static constexpr bool value = false; };
+template <int TW, int TH> struct BIsRun<RunShape<TW, TH>> { static constexpr bool value = true; };
+
+template <class SH>
+__device__ __forceinline__ void bcg_init_any(const BGeom& g, const BArgs& a, int job, unsigned char* smem) {
+  if constexpr (BIsRun<SH>::value) bcg_init_run<SH>(g.rc, a, job, smem);
+  else bcg_init_job<SH>(g.g, a, job, smem);
+}
+template <class SH>
+__device__ __forceinline__ void bcg_dir_any(const BGeom& g, const BArgs& a, int job, unsigned char* smem) {
+  if constexpr (BIsRun<SH>::value) bcg_dir_run<SH>(g.rc, a, job, smem);
+  else bcg_dir_job<SH>(g.g, a, job, smem);
 }
 
 template <class SH>
-__global__ void __launch_bounds__(BF_THREADS) k_bcg_dir(const Geom<float> g, const BArgs a) {
+__global__ void __launch_bounds__(BF_THREADS) k_bcg_init(const __grid_constant__ BGeom g, const BArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
-  bcg_dir_job<SH>(g, a, blockIdx.x, smem);
+  bcg_init_any<SH>(g, a, blockIdx.x, smem);
+}
+template <class SH>
+__global__ void __launch_bounds__(BF_THREADS) k_bcg_dir(const __grid_constant__ BGeom g, const BArgs a) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  bcg_dir_any<SH>(g, a, blockIdx.x, smem);
 }
 
 // x += alpha p, r -= alpha q, s = T r on a chunk of up to BUPD_CHUNK consecutive samples of
@@ -241,17 +417,37 @@ __device__ __forceinline__ void bcg_update_job(const BArgs& a, int job) {
   const float* p = in.p[(in.st.iter + 1) & 1];
   const int64_t i0 = jb.bx, i1 = i0 + jb.by;
   float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-  for (int64_t i = i0 + threadIdx.x; i < i1; i += BF_THREADS) {
-    const float pi = p[i], q = in.q[i];
-    in.x[i] = fmaf(alpha, pi, in.x[i]);
-    const float r = fmaf(-alpha, q, in.r[i]);
-    const float sv = in.dinv ? r * in.dinv[i] : r;
+  auto one = [&](float pi, float q, float di, float& x, float& r, float& sv) {
+    x = fmaf(alpha, pi, x);
+    r = fmaf(-alpha, q, r);
+    sv = in.dinv ? r * di : r;
+    v[0] = fmaf(sv, r, v[0]);
+    v[1] = fmaf(sv, q, v[1]);
+    v[2] = fmaf(sv, sv, v[2]);
+    v[3] = fmaf(r, r, v[3]);
+  };
+  // four samples per access where x allows it (the chunks start on multiples of four and
+  // the other vectors are aligned), the rest one by one
+  const int64_t iv = ((uintptr_t)in.x & 15) == 0 ? i0 + ((i1 - i0) & ~(int64_t)3) : i0;
+#pragma unroll 2
+  for (int64_t i = i0 + 4 * threadIdx.x; i < iv; i += 4 * BF_THREADS) {
+    const float4 p4 = bld4(p + i), q4 = bld4(in.q + i);
+    const float4 d4 = in.dinv ? bld4(in.dinv + i) : make_float4(1.0f, 1.0f, 1.0f, 1.0f);
+    float4 x4 = bld4(in.x + i), r4 = bld4(in.r + i), s4;
+    one(p4.x, q4.x, d4.x, x4.x, r4.x, s4.x);
+    one(p4.y, q4.y, d4.y, x4.y, r4.y, s4.y);
+    one(p4.z, q4.z, d4.z, x4.z, r4.z, s4.z);
+    one(p4.w, q4.w, d4.w, x4.w, r4.w, s4.w);
+    *reinterpret_cast<float4*>(in.x + i) = x4;
+    *reinterpret_cast<float4*>(in.r + i) = r4;
+    *reinterpret_cast<float4*>(in.s + i) = s4;
+  }
+  for (int64_t i = iv + threadIdx.x; i < i1; i += BF_THREADS) {
+    float x = in.x[i], r = in.r[i], sv;
+    one(p[i], in.q[i], in.dinv ? in.dinv[i] : 1.0f, x, r, sv);
+    in.x[i] = x;
     in.r[i] = r;
     in.s[i] = sv;
-    v[0] += sv * r;
-    v[1] += sv * q;
-    v[2] += sv * sv;
-    v[3] += r * r;
   }
   double blk[4], tot[4];
   block_sum<4, float>(v, red, blk);
@@ -274,13 +470,14 @@ __global__ void __launch_bounds__(BF_THREADS) k_bcg_update(const BArgs a) {
 }
 
 // candidate tile shapes of the image class (the autotuner's choices)
-typedef WinShapeT<3, 3, false, 32, 8> R3_32x8;
-typedef WinShapeT<3, 3, false, 64, 4> R3_64x4;
-typedef WinShapeT<3, 3, false, 16, 16> R3_16x16;
+typedef RunShape<64, 16> R3_64x16;
+typedef RunShape<32, 32> R3_32x32;
+typedef RunShape<128, 8> R3_128x8;
 enum { CLS_R3 = 0, CLS_R5 = 1, CLS_X1 = 2, NCLS = 3 };
 #define BUPD_CHUNK 4096           // samples per block of the update kernel (16 per thread)
-#define BTILE_GROUP 8             // consecutive tiles of one row per block of the operator kernels
-const int R3_TW[3] = {32, 64, 16}, R3_TH[3] = {8, 4, 16};
+// consecutive tiles of one row per block of the operator kernels, by class
+const int BTILE_GROUP[NCLS] = {1, 8, 8};
+const int R3_TW[3] = {64, 32, 128}, R3_TH[3] = {16, 32, 8};
 
 // ---- persistent form: one cooperative launch for the whole run ----------------------------
 // Every CTA walks the work lists of all classes phase by phase (start; then per iteration
@@ -291,7 +488,7 @@ const int R3_TW[3] = {32, 64, 16}, R3_TH[3] = {8, 4, 16};
 #define BAR_WAIT_NS 1000000000ull      // 1 s
 
 struct BGeoms {
-  Geom<float> g[NCLS];
+  BGeom g[NCLS];
 };
 
 struct BPArgs {
@@ -358,14 +555,14 @@ __device__ __forceinline__ void b_phase(const BGeoms& G, const BPArgs& pa, int p
       if (phase == 2) {
         bcg_update_job(pa.up[c], job);
       } else if (c == CLS_R3) {
-        if (phase == 0) bcg_init_job<SHR3>(G.g[c], pa.op[c], job, smem);
-        else bcg_dir_job<SHR3>(G.g[c], pa.op[c], job, smem);
+        if (phase == 0) bcg_init_any<SHR3>(G.g[c], pa.op[c], job, smem);
+        else bcg_dir_any<SHR3>(G.g[c], pa.op[c], job, smem);
       } else if (c == CLS_R5) {
-        if (phase == 0) bcg_init_job<ShapeR5>(G.g[c], pa.op[c], job, smem);
-        else bcg_dir_job<ShapeR5>(G.g[c], pa.op[c], job, smem);
+        if (phase == 0) bcg_init_any<ShapeR5>(G.g[c], pa.op[c], job, smem);
+        else bcg_dir_any<ShapeR5>(G.g[c], pa.op[c], job, smem);
       } else {
-        if (phase == 0) bcg_init_job<ShapeX1>(G.g[c], pa.op[c], job, smem);
-        else bcg_dir_job<ShapeX1>(G.g[c], pa.op[c], job, smem);
+        if (phase == 0) bcg_init_any<ShapeX1>(G.g[c], pa.op[c], job, smem);
+        else bcg_dir_any<ShapeX1>(G.g[c], pa.op[c], job, smem);
       }
       __syncthreads();                 // the job's shared memory is free
     }
@@ -393,7 +590,7 @@ struct bf_batch {
   int device;
   std::vector<const bf_graph*> graphs;
   std::vector<int> cls;              // class of each instance
-  Geom<float> geom[NCLS];
+  BGeom geom[NCLS];
   bool has[NCLS];
   int r3_variant;                    // tile shape of the image class (autotuned)
   int njobs[NCLS];                   // operator jobs (groups of tiles) per class
@@ -408,6 +605,8 @@ struct bf_batch {
   std::vector<cudaStream_t> lob_streams;   // batched LOBPCG: internal streams
   std::vector<cudaEvent_t> lob_events;     // one per internal stream, and one for the start
   std::vector<BInst> h_inst;
+  cudaStream_t cls_stream[NCLS];     // streams and events of the classes' chains
+  cudaEvent_t cls_join[NCLS], cls_fork;
   // captured run
   cudaGraphExec_t exec;
   uint64_t graph_kernels;            // kernels in the captured graph
@@ -422,6 +621,9 @@ template <class SH>
 size_t bsmem() { return 3 * SH::hp * sizeof(float); }
 
 int build_jobs(bf_batch* b) {
+  // a captured run holds pointers to the work lists that are rebuilt here
+  if (b->exec) cudaGraphExecDestroy(b->exec);
+  b->exec = nullptr;
   std::vector<BJob> jobs[NCLS], upd[NCLS];
   for (int c = 0; c < NCLS; ++c) b->ntiles[c] = 0;
   for (int i = 0; i < b->count; ++i) {
@@ -431,8 +633,8 @@ int build_jobs(bf_batch* b) {
     BInst& in = b->h_inst[i];
     in.job0 = (int)jobs[c].size();
     for (int by = 0; by < in.ny; by += th)
-      for (int bx = 0; bx < in.nx; bx += BTILE_GROUP * tw) {
-        const int nt = std::min(BTILE_GROUP, (in.nx - bx + tw - 1) / tw);
+      for (int bx = 0; bx < in.nx; bx += BTILE_GROUP[c] * tw) {
+        const int nt = std::min(BTILE_GROUP[c], (in.nx - bx + tw - 1) / tw);
         jobs[c].push_back(BJob{i, bx, by, nt});
         b->ntiles[c] += nt;
       }
@@ -486,14 +688,13 @@ void launch_phase(int phase, const bf_batch* b, int c, const BArgs& a, cudaStrea
   }
 }
 
-void launch_all(int phase, const bf_batch* b, const bf_cg_opts& o, int r3v, cudaStream_t s) {
-  for (int c = 0; c < NCLS; ++c) {
-    if (!b->has[c]) continue;
+void launch_class(int phase, const bf_batch* b, int c, const bf_cg_opts& o, int r3v, cudaStream_t s) {
+  {
     const BArgs a = make_args(b, c, o);
     if (c == CLS_R3) {
-      if (r3v == 0) launch_phase<R3_32x8>(phase, b, c, a, s);
-      else if (r3v == 1) launch_phase<R3_64x4>(phase, b, c, a, s);
-      else launch_phase<R3_16x16>(phase, b, c, a, s);
+      if (r3v == 0) launch_phase<R3_64x16>(phase, b, c, a, s);
+      else if (r3v == 1) launch_phase<R3_32x32>(phase, b, c, a, s);
+      else launch_phase<R3_128x8>(phase, b, c, a, s);
     } else if (c == CLS_R5) {
       launch_phase<ShapeR5>(phase, b, c, a, s);
     } else {
@@ -502,13 +703,43 @@ void launch_all(int phase, const bf_batch* b, const bf_cg_opts& o, int r3v, cuda
   }
 }
 
-int enqueue_run(const bf_batch* b, int kmax, const bf_cg_opts& o, cudaStream_t s) {
-  launch_all(0, b, o, b->r3_variant, s);
-  for (int it = 0; it < kmax; ++it) {
-    launch_all(1, b, o, b->r3_variant, s);
-    launch_all(2, b, o, b->r3_variant, s);
+// The classes share no instance: each class's chain of launches runs on a stream of its own,
+// forked from s and joined to it (the signals' chain is as long as the images' but fills a
+// fraction of the SMs).
+int enqueue_run(bf_batch* b, int kmax, const bf_cg_opts& o, cudaStream_t s) {
+  cudaStream_t cs[NCLS];
+  int first = -1;
+  bool forked = false;
+  for (int c = 0; c < NCLS; ++c) {
+    cs[c] = s;
+    if (!b->has[c]) continue;
+    if (first < 0) {
+      first = c;
+      continue;
+    }
+    if (!b->cls_fork) BF_CUDA(cudaEventCreateWithFlags(&b->cls_fork, cudaEventDisableTiming));
+    if (!b->cls_stream[c]) BF_CUDA(cudaStreamCreateWithFlags(&b->cls_stream[c], cudaStreamNonBlocking));
+    if (!b->cls_join[c]) BF_CUDA(cudaEventCreateWithFlags(&b->cls_join[c], cudaEventDisableTiming));
+    if (!forked) BF_CUDA(cudaEventRecord(b->cls_fork, s));
+    forked = true;
+    cs[c] = b->cls_stream[c];
+    BF_CUDA(cudaStreamWaitEvent(cs[c], b->cls_fork, 0));
   }
-  BF_CUDA(cudaGetLastError());
+  for (int c = 0; c < NCLS; ++c) {
+    if (!b->has[c]) continue;
+    launch_class(0, b, c, o, b->r3_variant, cs[c]);
+    for (int it = 0; it < kmax; ++it) {
+      launch_class(1, b, c, o, b->r3_variant, cs[c]);
+      launch_class(2, b, c, o, b->r3_variant, cs[c]);
+    }
+  }
+  const cudaError_t e = cudaGetLastError();
+  for (int c = 0; c < NCLS; ++c) {
+    if (cs[c] == s) continue;
+    BF_CUDA(cudaEventRecord(b->cls_join[c], cs[c]));
+    BF_CUDA(cudaStreamWaitEvent(s, b->cls_join[c], 0));
+  }
+  BF_CUDA(e);
   return BF_OK;
 }
 
@@ -537,7 +768,10 @@ extern "C" int bf_batch_create(const bf_graph* const* graphs, int count, bf_batc
   b->graph_kernels = 0;
   b->exec_kmax = -1;
   b->exec_variant = -1;
+  b->cls_fork = nullptr;
   for (int c = 0; c < NCLS; ++c) {
+    b->cls_stream[c] = nullptr;
+    b->cls_join[c] = nullptr;
     b->has[c] = false;
     b->d_jobs[c] = nullptr;
     b->d_upd[c] = nullptr;
@@ -562,9 +796,10 @@ extern "C" int bf_batch_create(const bf_graph* const* graphs, int count, bf_batc
     }
     if (!b->has[c]) {
       b->has[c] = true;
-      b->geom[c] = g->gf;
+      b->geom[c].g = g->gf;
+      b->geom[c].rc = run_const(g->gf);
     } else {
-      const Geom<float>& r = b->geom[c];
+      const Geom<float>& r = b->geom[c].g;
       bool same = r.a_r == g->gf.a_r;
       for (int t = 0; t < BF_MAX_BOX && same; ++t) same = (r.ls[t] == g->gf.ls[t]);
       if (!same) {
@@ -619,6 +854,11 @@ extern "C" int bf_batch_free(bf_batch* b) {
   if (b->d_inst) cudaFree(b->d_inst);
   if (b->d_vec) cudaFree(b->d_vec);
   if (b->d_bar) cudaFree(b->d_bar);
+  for (int c = 0; c < NCLS; ++c) {
+    if (b->cls_stream[c]) cudaStreamDestroy(b->cls_stream[c]);
+    if (b->cls_join[c]) cudaEventDestroy(b->cls_join[c]);
+  }
+  if (b->cls_fork) cudaEventDestroy(b->cls_fork);
   for (cudaStream_t st : b->lob_streams) cudaStreamDestroy(st);
   for (cudaEvent_t ev : b->lob_events) cudaEventDestroy(ev);
   delete b;
@@ -760,7 +1000,7 @@ static int batch_run_persistent(bf_batch* b, const float* const* x0, float* cons
     pa.nupd[c] = b->nupd[c];
   }
   if (b->has[CLS_R3]) {
-    const size_t r3[3] = {bsmem<R3_32x8>(), bsmem<R3_64x4>(), bsmem<R3_16x16>()};
+    const size_t r3[3] = {bsmem<R3_64x16>(), bsmem<R3_32x32>(), bsmem<R3_128x8>()};
     smem = std::max(smem, r3[b->r3_variant]);
   }
   if (b->has[CLS_R5]) smem = std::max(smem, bsmem<ShapeR5>());
@@ -769,9 +1009,9 @@ static int batch_run_persistent(bf_batch* b, const float* const* x0, float* cons
   pa.bar = reinterpret_cast<unsigned*>(b->d_bar);
   pa.err = reinterpret_cast<int*>(b->d_bar) + 2;
   pa.skip = skip;
-  if (b->r3_variant == 1) rc = launch_persistent<R3_64x4>(b, G, pa, smem, s);
-  else if (b->r3_variant == 2) rc = launch_persistent<R3_16x16>(b, G, pa, smem, s);
-  else rc = launch_persistent<R3_32x8>(b, G, pa, smem, s);
+  if (b->r3_variant == 1) rc = launch_persistent<R3_32x32>(b, G, pa, smem, s);
+  else if (b->r3_variant == 2) rc = launch_persistent<R3_128x8>(b, G, pa, smem, s);
+  else rc = launch_persistent<R3_64x16>(b, G, pa, smem, s);
   if (rc) return rc;
   std::vector<BInst> h(b->count);
   int err = 0;

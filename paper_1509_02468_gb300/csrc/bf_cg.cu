@@ -540,6 +540,7 @@ static_assert(RUN_THREADS == BF_THREADS, "the block reductions assume BF_THREADS
 __global__ void __launch_bounds__(RUN_THREADS, 3)
 k_cgr_init(const __grid_constant__ RunConst c, int nx, int ny, const __grid_constant__ RunSrc<2> src, int vec,
            const CgArgs<float> a) {
+  bf_pdl_enter();
   __shared__ double red[4 * (RUN_THREADS / 32)];
   __shared__ int last;
   float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
@@ -573,6 +574,7 @@ template <bool FIRST>
 __global__ void __launch_bounds__(RUN_THREADS, 3)
 k_cgr_dir(const __grid_constant__ RunConst c, int nx, int ny, const __grid_constant__ RunSrc<FIRST ? 2 : 3> src, int vec,
           const CgArgs<float> a) {
+  bf_pdl_enter();
   if (a.st->status != CG_RUN) return;
   __shared__ double red[RUN_THREADS / 32];
   __shared__ int last;
@@ -629,6 +631,7 @@ __device__ __forceinline__ void cgs_upd1(float alpha, bool jac, float q, float d
 // x += alpha p, s -= alpha T q (T = D^-1: s -= alpha q / d; r = d s), sums, beta.  Four
 // pixels per vector access (all arrays 16-byte aligned), the n % 4 tail by the last block.
 __global__ void __launch_bounds__(BF_THREADS) k_cgs_update(const CgArgs<float> a) {
+  bf_pdl_enter();
   if (a.st->status != CG_RUN) return;
   __shared__ double red[4 * (BF_THREADS / 32)];
   __shared__ int last;
@@ -804,7 +807,7 @@ int cg_run_loop(const bf_graph* g, CgArgs<float>& a, int kmax, double tol, cudaS
   s2.p[1] = a.guide;
   s2.ld[0] = s2.ld[1] = 1;
   run_src_vec(s2, nx);
-  BF_LAUNCH(k_cgr_init<<<run_grid(g, k_cgr_init, 2, occ[0]), RUN_THREADS, run_smem(2), s>>>(c, nx, ny, s2, vec, a));
+  BF_LAUNCH_PDL(k_cgr_init, run_grid(g, k_cgr_init, 2, occ[0]), RUN_THREADS, run_smem(2), s, c, nx, ny, s2, vec, a);
   for (int it = 0; it < kmax; ++it) {
     a.first = (it == 0);
     a.p_old = pbuf[it & 1];
@@ -812,8 +815,8 @@ int cg_run_loop(const bf_graph* g, CgArgs<float>& a, int kmax, double tol, cudaS
     if (it == 0) {
       s2.p[0] = a.s;
       run_src_vec(s2, nx);
-      BF_LAUNCH(k_cgr_dir<true><<<run_grid(g, k_cgr_dir<true>, 2, occ[1]), RUN_THREADS, run_smem(2), s>>>(
-          c, nx, ny, s2, vec, a));
+      BF_LAUNCH_PDL(k_cgr_dir<true>, run_grid(g, k_cgr_dir<true>, 2, occ[1]), RUN_THREADS, run_smem(2), s, c, nx, ny, s2,
+                    vec, a);
     } else {
       RunSrc<3> s3;
       s3.p[0] = a.s;
@@ -821,10 +824,10 @@ int cg_run_loop(const bf_graph* g, CgArgs<float>& a, int kmax, double tol, cudaS
       s3.p[2] = a.guide;
       s3.ld[0] = s3.ld[1] = s3.ld[2] = 1;
       run_src_vec(s3, nx);
-      BF_LAUNCH(k_cgr_dir<false><<<run_grid(g, k_cgr_dir<false>, 3, occ[2]), RUN_THREADS, run_smem(3), s>>>(
-          c, nx, ny, s3, vec, a));
+      BF_LAUNCH_PDL(k_cgr_dir<false>, run_grid(g, k_cgr_dir<false>, 3, occ[2]), RUN_THREADS, run_smem(3), s, c, nx, ny, s3,
+                    vec, a);
     }
-    BF_LAUNCH(k_cgs_update<<<nb_vec, BF_THREADS, 0, s>>>(a));
+    BF_LAUNCH_PDL(k_cgs_update, nb_vec, BF_THREADS, 0, s, a);
     if (tol > 0.0 && (it + 1) % CG_POLL == 0 && it + 1 < kmax) {
       int stv = 0;
       BF_CUDA(cudaMemcpyAsync(&stv, &a.st->status, sizeof(int), cudaMemcpyDeviceToHost, s));

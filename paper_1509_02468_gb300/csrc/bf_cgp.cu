@@ -186,21 +186,6 @@ __device__ __forceinline__ auto cgp_red(CgpShared<float>& sh, CgpPair*) -> declt
 template <typename T> __device__ __forceinline__ double* cgp_part(CgpShared<T>& sh, double*) { return sh.part.d; }
 __device__ __forceinline__ CgpPair* cgp_part(CgpShared<float>& sh, CgpPair*) { return sh.part.n; }
 
-// Warp sums of four values at once, value ((lane >> 3) & 3) in a lane: 6 additions and
-// shuffles instead of 20.
-template <typename T>
-__device__ __forceinline__ T cgp_warp4(const T (&v)[4], int lane) {
-  const bool h16 = lane & 16, h8 = lane & 8;
-  T a = h16 ? v[2] : v[0], b = h16 ? v[3] : v[1];
-  a += __shfl_xor_sync(0xffffffffu, h16 ? v[0] : v[2], 16);
-  b += __shfl_xor_sync(0xffffffffu, h16 ? v[1] : v[3], 16);
-  T c = h8 ? b : a;
-  c += __shfl_xor_sync(0xffffffffu, h8 ? a : b, 8);
-#pragma unroll
-  for (int o = 4; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-  return c;
-}
-
 // Sums of v (times scale) over all threads of all CTAs, and a barrier of the grid.  Warp
 // w < NV gets the total of value w and calls tail(w, total) with all its lanes; what tail
 // writes to shared memory is visible to every thread on return.  `during` runs while the
@@ -214,7 +199,7 @@ __device__ __forceinline__ bool cgp_allreduce(const T (&v)[4], T scale, CgpShare
   auto& red = cgp_red(sh, (R*)nullptr);
   R* part = cgp_part(sh, (R*)nullptr);
   if (NV == 4) {
-    const T w = cgp_warp4<T>(v, lane);
+    const T w = warp_sum4<T>(v, lane);
     if ((lane & 7) == 0) cgp_from(w * scale, red[lane >> 3][wid]);
   } else {
     const T w = warp_sum(v[0]);

@@ -171,8 +171,6 @@ template <int CIN, int COUT, int IN, int OUT>
 __global__ void __launch_bounds__(NET_TW * NET_TH) k_net_conv(const NetArgs a) {
   static_assert(COUT == NET_CH || (COUT == 1 && CIN % 4 == 0), "layer shapes of the net");
   constexpr int COUTP = (COUT + 3) & ~3;
-  bf_pdl_enter();
-  if (a.stop && *a.stop != 0) return;
   __shared__ __align__(16) float sx[CIN * NET_HP];
   __shared__ __align__(16) float sw[CIN * 9 * COUTP];       // [c][tap][o]
   const int col = blockIdx.z;
@@ -183,6 +181,10 @@ __global__ void __launch_bounds__(NET_TW * NET_TH) k_net_conv(const NetArgs a) {
     if (o < COUT) wv = a.transpose ? a.w[(c * COUT + o) * 9 + (8 - t)] : a.w[(o * CIN + c) * 9 + t];
     sw[e] = wv;
   }
+  // the weights do not come from the kernel before this one (and the one that wrote them has
+  // finished when that one runs), so they are staged while it does
+  bf_pdl_enter();
+  if (a.stop && *a.stop != 0) return;
   const float rh = IN == IN_NET ? net_rho(a, col) : 0.0f;
   net_stage<CIN, IN>(a, a.in, col, rh, bx, by, sx);
   __syncthreads();
@@ -277,14 +279,10 @@ __global__ void __launch_bounds__(256) k_net_sums(const float* r, int64_t ldr, c
     red[8 + (threadIdx.x >> 5)] = s1;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double a0 = 0.0, a1 = 0.0;
-    for (int w = 0; w < 8; ++w) {
-      a0 += red[w];
-      a1 += red[8 + w];
-    }
-    partials[((int64_t)col * gridDim.x + blockIdx.x) * 2 + 0] = a0;
-    partials[((int64_t)col * gridDim.x + blockIdx.x) * 2 + 1] = a1;
+  if (threadIdx.x < 32) {                     // lanes 0 .. 7: the first sums, 8 .. 15: the second
+    double v = red[threadIdx.x & 15];
+    for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 23) == 0) partials[((int64_t)col * gridDim.x + blockIdx.x) * 2 + (threadIdx.x >> 3)] = v;
   }
 }
 
@@ -304,10 +302,10 @@ __global__ void __launch_bounds__(256) k_net_loss(const float* O, const float* z
   s = warp_sum(s);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int w = 0; w < 8; ++w) t += red[w];
-    partials[blockIdx.x] = t;
+  if (threadIdx.x < 32) {
+    double v = red[threadIdx.x & 7];
+    for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (threadIdx.x == 0) partials[blockIdx.x] = v;
   }
 }
 
@@ -327,11 +325,23 @@ __device__ __forceinline__ void net_wgrad(const NetArgs& a, const float* in, con
   float* sg = sh + XF;                                       // [o][px]
   const int bx = blockIdx.x * NET_TW, by = blockIdx.y * NET_TH;
   net_stage<CIN, IN>(a, in, 0, IN == IN_NET ? a.rho[0] : 0.0f, bx, by, sx);
-  for (int e = threadIdx.x; e < COUT * NET_TW * NET_TH; e += NET_TW * NET_TH) {
-    const int p = e / COUT, o = e - p * COUT;
-    const int ly = p / NET_TW, lx = p - ly * NET_TW;
-    const int x = bx + lx, y = by + ly;
-    sg[o * GS + p] = (x < a.nx && y < a.ny) ? G[((int64_t)y * a.nx + x) * COUT + o] : 0.0f;
+  {
+    const int p = threadIdx.x, x = bx + p % NET_TW, y = by + p / NET_TW;
+    const bool in = x < a.nx && y < a.ny;
+    const float* src = G + ((int64_t)y * a.nx + x) * COUT;
+    if (COUT == 1) {
+      sg[p] = in ? *src : 0.0f;
+    } else {
+#pragma unroll
+      for (int o4 = 0; o4 < COUT / 4; ++o4) {
+        float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (in) v = reinterpret_cast<const float4*>(src)[o4];
+        sg[(4 * o4) * GS + p] = v.x;
+        sg[(4 * o4 + 1) * GS + p] = v.y;
+        sg[(4 * o4 + 2) * GS + p] = v.z;
+        sg[(4 * o4 + 3) * GS + p] = v.w;
+      }
+    }
   }
   __syncthreads();
   const int grp = threadIdx.x / NP, pair = threadIdx.x - grp * NP;
