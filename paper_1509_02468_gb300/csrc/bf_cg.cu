@@ -535,17 +535,20 @@ __global__ void __launch_bounds__(STRIP_THREADS, 2) k_cgs_dir(const Geom<float> 
   if (grid_sum_last<1>(blk, a.partials, &a.st->counter, tot, &last)) cg_dir_tail(a, tot[0]);
 }
 
-// k_cgs_init and k_cgs_dir with weights on the fly, by horizontal runs (bf_run.cuh).
+// k_cgs_init and k_cgs_dir with weights on the fly, by horizontal runs (bf_run.cuh).  nx: row
+// pitch of all arrays, nxr <= nx: image width; rows of a width that is not a multiple of four
+// are padded (k_cgr_pad: guide +inf, so the padding has no weight), which keeps every access
+// a 16-byte vector (1531 x 2047: 73 us an iteration unpadded).
 static_assert(RUN_THREADS == BF_THREADS, "the block reductions assume BF_THREADS threads");
 __global__ void __launch_bounds__(RUN_THREADS, 3)
-k_cgr_init(const __grid_constant__ RunConst c, int nx, int ny, const __grid_constant__ RunSrc<2> src, int vec,
+k_cgr_init(const __grid_constant__ RunConst c, int nx, int nxr, int ny, const __grid_constant__ RunSrc<2> src, int vec,
            const CgArgs<float> a) {
   bf_pdl_enter();
   __shared__ double red[4 * (RUN_THREADS / 32)];
   __shared__ int last;
   float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
   auto epi = [&](int x0, int y, const float (&xi)[RUN_P], const float (&acc)[RUN_P], const float (&)[RUN_P]) {
-    const int cnt = run_count(x0, y, nx, ny);
+    const int cnt = run_count(x0, y, nxr, ny);
     if (!cnt) return;
     const int64_t i0 = (int64_t)y * nx + x0;
     float sj[RUN_P], d[RUN_P];
@@ -560,7 +563,7 @@ k_cgr_init(const __grid_constant__ RunConst c, int nx, int ny, const __grid_cons
       v[2] = fmaf(r, r, v[2]);
       v[3] = fmaf(xi[j], xi[j], v[3]);
     }
-    run_store(a.x, i0, cnt, vec, xi);
+    if (a.x != src.p[0]) run_store(a.x, i0, cnt, vec, xi);
     run_store(a.s, i0, cnt, vec, sj);
   };
   run_tiles<2, true, false, false>(c, nx, ny, src, [](float*) {}, epi);
@@ -572,7 +575,7 @@ k_cgr_init(const __grid_constant__ RunConst c, int nx, int ny, const __grid_cons
 // Bound by the FP32 pipe and the SFU (see bf_run.cuh) with 20 B per pixel beside them.
 template <bool FIRST>
 __global__ void __launch_bounds__(RUN_THREADS, 3)
-k_cgr_dir(const __grid_constant__ RunConst c, int nx, int ny, const __grid_constant__ RunSrc<FIRST ? 2 : 3> src, int vec,
+k_cgr_dir(const __grid_constant__ RunConst c, int nx, int nxr, int ny, const __grid_constant__ RunSrc<FIRST ? 2 : 3> src, int vec,
           const CgArgs<float> a) {
   bf_pdl_enter();
   if (a.st->status != CG_RUN) return;
@@ -592,7 +595,7 @@ k_cgr_dir(const __grid_constant__ RunConst c, int nx, int ny, const __grid_const
     }
   };
   auto epi = [&](int x0, int y, const float (&pi)[RUN_P], const float (&acc)[RUN_P], const float (&)[RUN_P]) {
-    const int cnt = run_count(x0, y, nx, ny);
+    const int cnt = run_count(x0, y, nxr, ny);
     if (!cnt) return;
     const int64_t i0 = (int64_t)y * nx + x0;
     float q[RUN_P];
@@ -608,6 +611,30 @@ k_cgr_dir(const __grid_constant__ RunConst c, int nx, int ny, const __grid_const
   double blk[1], tot[1];
   block_sum<1, float>(v, red, blk);
   if (grid_sum_last<1>(blk, a.partials, &a.st->counter, tot, &last)) cg_dir_tail(a, tot[0]);
+}
+
+// Rows padded to pitch nxp: guide (+inf), degree (1) and x0 (0); zeros in the padding of the
+// run's vectors, which nothing writes.
+__global__ void __launch_bounds__(BF_THREADS) k_cgr_pad(const float* guide, const float* d, const float* x0, int nx, int nxp,
+                                                        int ny, float* gp, float* dp, float* xp, float* s, float* q,
+                                                        float* p0, float* p1) {
+  const int64_t n = (int64_t)nxp * ny;
+  for (int64_t i = (int64_t)blockIdx.x * BF_THREADS + threadIdx.x; i < n; i += (int64_t)gridDim.x * BF_THREADS) {
+    const int64_t y = i / nxp, x = i - y * nxp, e = y * nx + x;
+    const bool in = x < nx;
+    gp[i] = in ? guide[e] : __int_as_float(0x7f800000);
+    dp[i] = in ? d[e] : 1.0f;
+    xp[i] = in ? x0[e] : 0.0f;
+    if (!in) s[i] = q[i] = p0[i] = p1[i] = 0.0f;
+  }
+}
+__global__ void __launch_bounds__(BF_THREADS) k_cgr_unpad(const float* xp, int nx, int nxp, int ny, float* x) {
+  bf_pdl_enter();
+  const int64_t n = (int64_t)nx * ny;
+  for (int64_t i = (int64_t)blockIdx.x * BF_THREADS + threadIdx.x; i < n; i += (int64_t)gridDim.x * BF_THREADS) {
+    const int64_t y = i / nx;
+    x[i] = xp[y * nxp + (i - y * nx)];
+  }
 }
 
 // One pixel of the update: x += alpha p, s -= alpha T q, and the four sums.
@@ -783,6 +810,14 @@ int cg_strip_loop_w(const bf_graph* g, CgArgs<float>& a, int kmax, double tol, c
   return BF_OK;
 }
 
+// Whether a run with weights on the fly pads its rows (it must have asked for the room), and
+// to what pitch.
+int cg_pitch(int nx) { return (nx + 3) & ~3; }
+bool cg_pads(const bf_graph* g, const bf_cg_opts& o) {
+  return g->kind == BF_KIND_BILATERAL && fast_shape(g) == FAST_R3_2D && g->p.weight_mode == BF_W_ONTHEFLY &&
+         g->nx % 4 != 0 && g->gf.a_r > 0.0f && (o.precond == BF_PRECOND_JACOBI || o.precond == BF_PRECOND_IDENTITY) && !cgp_words(g);
+}
+
 template <class F>
 int run_grid(const bf_graph* g, F fn, int na, int& per_sm) {
   if (per_sm == 0) {
@@ -795,19 +830,34 @@ int run_grid(const bf_graph* g, F fn, int na, int& per_sm) {
 }
 
 // The same loop with weights on the fly (bf_run.cuh).
-int cg_run_loop(const bf_graph* g, CgArgs<float>& a, int kmax, double tol, cudaStream_t s, float* const* pbuf) {
+// pad: NULL, or three further vectors (guide, degree, x) for padded rows.
+int cg_run_loop(const bf_graph* g, CgArgs<float>& a, int kmax, double tol, cudaStream_t s, float* const* pbuf,
+                float* const* pad) {
   static int occ[3] = {0, 0, 0};
-  const unsigned nb_vec =
-      (unsigned)std::max<int64_t>(1, std::min<int64_t>((a.n / 4 + BF_THREADS - 1) / BF_THREADS, 8 * cg_num_sms()));
   a.d = (const float*)g->d;
   const RunConst c = run_const(g->gf);
-  const int nx = g->nx, ny = g->ny, vec = nx % 4 == 0;       // x, d, s, p, q are 16-byte aligned
+  const int nxr = g->nx, ny = g->ny;
+  int nx = nxr;
+  float* x_out = a.x;
+  if (pad) {
+    nx = cg_pitch(nxr);
+    a.n = (int64_t)nx * ny;
+    const unsigned nb = (unsigned)std::min<int64_t>((a.n + BF_THREADS - 1) / BF_THREADS, 16 * cg_num_sms());
+    BF_LAUNCH(k_cgr_pad<<<nb, BF_THREADS, 0, s>>>(a.guide, a.d, a.x0, nxr, nx, ny, pad[0], pad[1], pad[2], a.s, a.q,
+                                                  pbuf[0], pbuf[1]));
+    a.guide = pad[0];
+    a.d = pad[1];
+    a.x0 = a.x = pad[2];
+  }
+  const unsigned nb_vec =
+      (unsigned)std::max<int64_t>(1, std::min<int64_t>((a.n / 4 + BF_THREADS - 1) / BF_THREADS, 8 * cg_num_sms()));
+  const int vec = nx % 4 == 0;                               // x, d, s, p, q are 16-byte aligned
   RunSrc<2> s2;
   s2.p[0] = a.x0;
   s2.p[1] = a.guide;
   s2.ld[0] = s2.ld[1] = 1;
   run_src_vec(s2, nx);
-  BF_LAUNCH_PDL(k_cgr_init, run_grid(g, k_cgr_init, 2, occ[0]), RUN_THREADS, run_smem(2), s, c, nx, ny, s2, vec, a);
+  BF_LAUNCH_PDL(k_cgr_init, run_grid(g, k_cgr_init, 2, occ[0]), RUN_THREADS, run_smem(2), s, c, nx, nxr, ny, s2, vec, a);
   for (int it = 0; it < kmax; ++it) {
     a.first = (it == 0);
     a.p_old = pbuf[it & 1];
@@ -815,7 +865,7 @@ int cg_run_loop(const bf_graph* g, CgArgs<float>& a, int kmax, double tol, cudaS
     if (it == 0) {
       s2.p[0] = a.s;
       run_src_vec(s2, nx);
-      BF_LAUNCH_PDL(k_cgr_dir<true>, run_grid(g, k_cgr_dir<true>, 2, occ[1]), RUN_THREADS, run_smem(2), s, c, nx, ny, s2,
+      BF_LAUNCH_PDL(k_cgr_dir<true>, run_grid(g, k_cgr_dir<true>, 2, occ[1]), RUN_THREADS, run_smem(2), s, c, nx, nxr, ny, s2,
                     vec, a);
     } else {
       RunSrc<3> s3;
@@ -824,7 +874,7 @@ int cg_run_loop(const bf_graph* g, CgArgs<float>& a, int kmax, double tol, cudaS
       s3.p[2] = a.guide;
       s3.ld[0] = s3.ld[1] = s3.ld[2] = 1;
       run_src_vec(s3, nx);
-      BF_LAUNCH_PDL(k_cgr_dir<false>, run_grid(g, k_cgr_dir<false>, 3, occ[2]), RUN_THREADS, run_smem(3), s, c, nx, ny, s3,
+      BF_LAUNCH_PDL(k_cgr_dir<false>, run_grid(g, k_cgr_dir<false>, 3, occ[2]), RUN_THREADS, run_smem(3), s, c, nx, nxr, ny, s3,
                     vec, a);
     }
     BF_LAUNCH_PDL(k_cgs_update, nb_vec, BF_THREADS, 0, s, a);
@@ -835,16 +885,20 @@ int cg_run_loop(const bf_graph* g, CgArgs<float>& a, int kmax, double tol, cudaS
       if (stv != CG_RUN) break;
     }
   }
+  if (pad) {
+    const unsigned nb = (unsigned)std::min<int64_t>((g->n + BF_THREADS - 1) / BF_THREADS, 16 * cg_num_sms());
+    BF_LAUNCH_PDL(k_cgr_unpad, nb, BF_THREADS, 0, s, pad[2], nxr, nx, ny, x_out);
+  }
   return BF_OK;
 }
 
 int cg_strip_loop(const bf_graph* g, CgArgs<float>& a, int kmax, double tol, cudaStream_t s,
-                  float* const* pbuf) {
+                  float* const* pbuf, float* const* pad) {
   switch (g->p.weight_mode) {
     case BF_W_STORED_F32: return cg_strip_loop_w<BF_W_STORED_F32>(g, a, kmax, tol, s, pbuf);
     case BF_W_STORED_BF16: return cg_strip_loop_w<BF_W_STORED_BF16>(g, a, kmax, tol, s, pbuf);
   }
-  return cg_run_loop(g, a, kmax, tol, s, pbuf);
+  return cg_run_loop(g, a, kmax, tol, s, pbuf, pad);
 }
 
 // Device buffers of one CG run: residual r, preconditioned residual s, q = A p, the two
@@ -857,6 +911,7 @@ struct CgBufs {
   T* p[2];
   double* partials;
   CgState* st;
+  T* pad[3];           // padded rows: guide, degree, x (NULL: none)
 };
 
 // Algorithm 2 on the buffers `b` (cg_filter: the graph's workspace; cg_filter_noalloc: the
@@ -902,9 +957,11 @@ int cg_exec(const bf_graph* g, const T* x0, int kmax, const bf_cg_opts& o, T* x_
   if (words) {                                     // the vectors fit on the chip: one launch
     rc = cgp_launch<T>(g, a, kmax, s);
     if (rc) return rc;
-  } else if (!guided && !net && sizeof(T) == 4 && fast_shape(g) == FAST_R3_2D && ((uintptr_t)x_out & 15) == 0) {
+  } else if (!guided && !net && sizeof(T) == 4 && fast_shape(g) == FAST_R3_2D &&
+             (b.pad[0] || ((uintptr_t)x_out & 15) == 0)) {
     rc = cg_strip_loop(g, reinterpret_cast<CgArgs<float>&>(a), kmax, o.tol, s,
-                       reinterpret_cast<float* const*>(b.p));
+                       reinterpret_cast<float* const*>(b.p),
+                       b.pad[0] ? reinterpret_cast<float* const*>(b.pad) : nullptr);
     if (rc) return rc;
   } else {
     rc = cg_generic_loop<T>(g, a, kmax, o, s, b.p, tg, sm, nb_elem);
@@ -940,10 +997,12 @@ template <typename T>
 int cg_run(const bf_graph* g, const T* x0, int kmax, const bf_cg_opts& o, T* x_out,
            bf_info* info, cudaStream_t s) {
   bf_graph* gm = const_cast<bf_graph*>(g);
-  const size_t vb = ((size_t)g->n * sizeof(T) + 255) & ~(size_t)255;
+  const bool pads = sizeof(T) == 4 && cg_pads(g, o);
+  const int nv = pads ? 8 : 5;
+  const size_t vb = ((size_t)(pads ? (int64_t)cg_pitch(g->nx) * g->ny : g->n) * sizeof(T) + 255) & ~(size_t)255;
   const size_t pb =
       (std::max((size_t)cg_partial_slots(g) * 4 * sizeof(double), 8 * cgp_words(g)) + 255) & ~(size_t)255;
-  int rc = bf_ws_reserve(gm, BF_WS_CG, 5 * vb + pb + 256);
+  int rc = bf_ws_reserve(gm, BF_WS_CG, nv * vb + pb + 256);
   if (rc) return rc;
   char* w = (char*)gm->ws[BF_WS_CG];
   CgBufs<T> b;
@@ -952,8 +1011,9 @@ int cg_run(const bf_graph* g, const T* x0, int kmax, const bf_cg_opts& o, T* x_o
   b.q = (T*)(w + 2 * vb);
   b.p[0] = (T*)(w + 3 * vb);
   b.p[1] = (T*)(w + 4 * vb);
-  b.partials = (double*)(w + 5 * vb);
-  b.st = (CgState*)(w + 5 * vb + pb);
+  for (int j = 0; j < 3; ++j) b.pad[j] = pads ? (T*)(w + (5 + j) * vb) : nullptr;
+  b.partials = (double*)(w + nv * vb);
+  b.st = (CgState*)(w + nv * vb + pb);
   return cg_exec<T>(g, x0, kmax, o, x_out, info, s, b, "cg_filter");
 }
 
@@ -1173,6 +1233,7 @@ int cg_run_noalloc(const bf_graph* g, const T* x0, int kmax, const bf_cg_opts& o
   b.q = (T*)(w + 2 * BF_NOALLOC_VEC_BYTES);
   b.p[0] = (T*)(w + 3 * BF_NOALLOC_VEC_BYTES);
   b.p[1] = (T*)(w + 4 * BF_NOALLOC_VEC_BYTES);
+  b.pad[0] = b.pad[1] = b.pad[2] = nullptr;      // (larger than what would need it)
   b.partials = (double*)(w + 5 * BF_NOALLOC_VEC_BYTES);
   b.st = (CgState*)(w + 5 * BF_NOALLOC_VEC_BYTES + (size_t)BF_NOALLOC_MAX_BLOCKS * 4 * sizeof(double));
   return cg_exec<T>(g, x0, kmax, o, x_out, info, s, b, "cg_filter_noalloc");

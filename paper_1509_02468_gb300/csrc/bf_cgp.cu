@@ -987,8 +987,8 @@ bool cgp_rect(int nx, int ny, CgpRect* out, int* nreg) {
   return best >= 0;
 }
 
-// Samples per CTA of a signal: at least 128 (four warps, one per scheduler; a smaller piece
-// only adds partial sums to add), 0 if it does not fit.
+// Samples per CTA of a signal: at least 128 (4096 samples in FP64, 20 steps: 157 us; 256: 185),
+// 0 if it does not fit.
 int cgp_line_width(const bf_graph* g) {
   const int maxc = cgp_max_ctas();
   if (maxc < 1) return 0;

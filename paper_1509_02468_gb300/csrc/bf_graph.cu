@@ -122,6 +122,7 @@ k_weights(const Geom<T> g, const T* __restrict__ guide, int64_t n, T* d, T* dinv
 __global__ void __launch_bounds__(RUN_THREADS, 3)
 k_weights_run(const __grid_constant__ RunConst c, int nx, int ny, const __grid_constant__ RunSrc<1> src, int vec,
               float* guide, float* d, float* dinv, float* dis, float* dls, int* flag) {
+  bf_pdl_enter();
   auto epi = [&](int x0, int y, const float (&)[RUN_P], const float (&)[RUN_P], const float (&ws)[RUN_P]) {
     const int cnt = run_count(x0, y, nx, ny);
     if (!cnt) return;
@@ -355,6 +356,7 @@ template <bool SCALED, bool STEP>
 __global__ void __launch_bounds__(RUN_THREADS, 3)
 k_apply1_run(const __grid_constant__ RunConst c, int nx, int ny, const __grid_constant__ RunSrc<SCALED ? 3 : 2> src,
              int vec_y, float* Y, int64_t ldy, double* dots) {
+  bf_pdl_enter();
   constexpr int NA = SCALED ? 3 : 2;
   float dsum = 0.0f;
   auto combine = [&](float* st) {           // operand of the scaled operators: x * scale
@@ -1032,8 +1034,8 @@ static int launch_apply1_run(const bf_graph* g, const ApplyArgs<float>& a, cudaS
   const int vec_y = g->nx % 4 == 0 && ((uintptr_t)a.Y & 15) == 0;
   const int64_t ntiles = (int64_t)run_tiles_x(g->nx) * run_tiles_y(g->ny);
   const int grid = (int)std::min<int64_t>(ntiles, (int64_t)per_sm * num_sms());
-  BF_LAUNCH(k_apply1_run<SCALED, STEP><<<grid, RUN_THREADS, run_smem(NA), s>>>(run_const(g->gf), g->nx, g->ny, src,
-                                                                             vec_y, a.Y, a.ldy, a.dots));
+  BF_LAUNCH_PDL((k_apply1_run<SCALED, STEP>), grid, RUN_THREADS, run_smem(NA), s, run_const(g->gf), g->nx, g->ny, src,
+                vec_y, a.Y, a.ldy, a.dots);
   BF_CUDA(cudaGetLastError());
   return BF_OK;
 }
@@ -1287,6 +1289,7 @@ extern "C" int bf_weights(const bf_params* p, const void* guide, bf_graph** out,
     if ((e = cudaMalloc(&g->wf, wb)) != cudaSuccess) return cleanup(bf_cuda_fail(e, "cudaMalloc(weights)"));
   }
   if ((e = cudaMalloc(&g->flag, sizeof(int))) != cudaSuccess) return cleanup(bf_cuda_fail(e, "cudaMalloc(flag)"));
+  if ((e = cudaMemsetAsync(g->flag, 0, sizeof(int), s)) != cudaSuccess) return cleanup(bf_cuda_fail(e, "memset(flag)"));
   const int rc = compute_weights(g, guide, s);
   if (rc) return cleanup(rc);
   *out = g;
@@ -1315,9 +1318,9 @@ static int launch_weights(bf_graph* g, const void* guide, cudaStream_t s) {
     run_src_vec(src, g->nx);
     const int64_t ntiles = (int64_t)run_tiles_x(g->nx) * run_tiles_y(g->ny);
     const int grid = (int)std::min<int64_t>(ntiles, (int64_t)per_sm * num_sms());
-    BF_LAUNCH(k_weights_run<<<grid, RUN_THREADS, run_smem(1), s>>>(
-        run_const(g->gf), g->nx, g->ny, src, g->nx % 4 == 0, (float*)g->guide, (float*)g->d, (float*)g->dinv,
-        (float*)g->dis, (float*)g->dls, g->flag));
+    BF_LAUNCH_PDL(k_weights_run, grid, RUN_THREADS, run_smem(1), s, run_const(g->gf), g->nx, g->ny, src,
+                  (int)(g->nx % 4 == 0), (float*)g->guide, (float*)g->d, (float*)g->dinv, (float*)g->dis,
+                  (float*)g->dls, g->flag);
     if ((e = cudaGetLastError()) != cudaSuccess) return bf_cuda_fail(e, "k_weights_run launch");
     return BF_OK;
   }
@@ -1337,19 +1340,40 @@ static int launch_weights(bf_graph* g, const void* guide, cudaStream_t s) {
   return BF_OK;
 }
 
+// A pinned int per host thread for the flag's copy (a copy to pageable memory goes through a
+// staging buffer and waits twice); NULL if it cannot be had.
+static int* pinned_flag() {
+  struct Pinned {
+    int* p = nullptr;
+    ~Pinned() {
+      if (p) cudaFreeHost(p);
+    }
+  };
+  static thread_local Pinned h;
+  if (!h.p && cudaHostAlloc(&h.p, sizeof(int), cudaHostAllocPortable) != cudaSuccess) {
+    h.p = nullptr;
+    (void)cudaGetLastError();
+  }
+  return h.p;
+}
+
+// Wait for s and report a flagged guide.  The flag is 0 between calls (cleared when the graph
+// is made and whenever it was found set), so a call does not clear it first.
 static int read_flag(bf_graph* g, cudaStream_t s, const char* what) {
   cudaError_t e;
-  int hflag = 0;
-  if ((e = cudaMemcpyAsync(&hflag, g->flag, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess)
+  int local = 0, *pin = pinned_flag();
+  volatile int& hflag = pin ? *pin : local;
+  if ((e = cudaMemcpyAsync((void*)&hflag, g->flag, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess)
     return bf_cuda_fail(e, "cudaMemcpyAsync(flag)");
   if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return bf_cuda_fail(e, "weights sync");
-  if (hflag) return bf_fail(BF_ENONFINITE, what);
+  if (hflag) {
+    if ((e = cudaMemsetAsync(g->flag, 0, sizeof(int), s)) != cudaSuccess) return bf_cuda_fail(e, "memset(flag)");
+    return bf_fail(BF_ENONFINITE, what);
+  }
   return BF_OK;
 }
 
 static int compute_weights(bf_graph* g, const void* guide, cudaStream_t s) {
-  cudaError_t e;
-  if ((e = cudaMemsetAsync(g->flag, 0, sizeof(int), s)) != cudaSuccess) return bf_cuda_fail(e, "memset(flag)");
   const int rc = launch_weights(g, guide, s);
   if (rc) return rc;
   return read_flag(g, s, "bf_weights: guide holds NaN or Inf");
@@ -1437,7 +1461,6 @@ extern "C" int bf_reguided_filter(bf_graph* g, const void* x0, int iters, void* 
   int rc = bf_ws_reserve(g, BF_WS_SIMPLE, 2 * nba);
   if (rc) return rc;
   void* tmp[2] = {g->ws[BF_WS_SIMPLE], (char*)g->ws[BF_WS_SIMPLE] + nba};
-  BF_CUDA(cudaMemsetAsync(g->flag, 0, sizeof(int), s));
   // on-the-fly weights: one kernel per step, the iterate staged as its own guide; the graph
   // is rebuilt once, for the last guide.  Stored weights: rebuilt every step.
   const bool otf = g->p.weight_mode == BF_W_ONTHEFLY && g->kind == BF_KIND_BILATERAL;

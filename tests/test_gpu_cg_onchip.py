@@ -119,3 +119,26 @@ def test_guided_images(shape, radius):
         ref = solvers.cg(O, host(g).reshape(-1), iters, **kw)
         assert info.iters == ref["iters"]
         assert rel_l2(host(x), ref["x"]) < TOL_F32
+
+
+@pytest.mark.parametrize("shape", [(1103, 1201), (1290, 1002), (1030, 1280), (601, 2203)])
+def test_images_beyond_the_chip(shape):
+    """Images too large for the one-launch form, with rows that are padded to whole vectors and
+    rows that are not, against the FP64 path on the same guide (itself held to the oracle)."""
+    rng = np.random.default_rng(shape[1])
+    img = np.cumsum(rng.uniform(-0.03, 0.03, shape), axis=1).astype(np.float32)
+    g = torch.as_tensor(img, device="cuda")
+    G, G64 = bf().bf_weights(g, 3, 2.0, 0.08), bf().bf_weights(g.double(), 3, 2.0, 0.08)
+    x0 = g.reshape(-1)
+    for kw in ({}, {"shift": 0.05, "precond": "identity"}):
+        ref = bf().cg_filter(G64, x0.double(), 6, **kw)[0]
+        x, info, _ = bf().cg_filter(G, x0, 6, **kw)
+        assert info.iters == 6 and rel_l2(host(x), host(ref)) < TOL_F32
+        y = x0.clone()
+        bf().cg_filter(G, y, 6, out=y, **kw)
+        assert torch.equal(x, y)
+    wide = torch.zeros(x0.numel() + 1, device="cuda")        # vectors off the 16-byte grid
+    wide[1:] = x0
+    out = torch.empty_like(wide)[1:]
+    bf().cg_filter(G, wide[1:], 6, out=out)
+    assert rel_l2(host(out), host(bf().cg_filter(G64, x0.double(), 6)[0])) < TOL_F32
