@@ -376,11 +376,14 @@ __global__ void __launch_bounds__(RR_T) k_rr_reduce(const RRParams a) {
   auto reflector = [&](int j) {
     const int n1 = m - j - 1;
     float* col = J + (j + 1) * RR_LDF + j;
-    float s = 0.0f;
-    for (int i = lane; i < n1; i += 32) s = fmaf(col[i * RR_LDF], col[i * RR_LDF], s);
+    float s = 0.0f, cv[RR_MMAX / 32];
+#pragma unroll
+    for (int u = 0; u < RR_MMAX / 32; ++u) cv[u] = lane + 32 * u < n1 ? col[(lane + 32 * u) * RR_LDF] : 0.0f;
+#pragma unroll
+    for (int u = 0; u < RR_MMAX / 32; ++u) s = fmaf(cv[u], cv[u], s);
     s = warp_sum(s);
     if (lane == 0) {
-      const float x0 = col[0];
+      const float x0 = cv[0];
       const float tail = s - x0 * x0;
       float al = x0, be = 0.0f;
       if (tail > 0.0f) {
@@ -403,6 +406,12 @@ __global__ void __launch_bounds__(RR_T) k_rr_reduce(const RRParams a) {
     const float beta = bet32[j];
     float* col = J + (j + 1) * RR_LDF + j;          // v_i = col[i * RR_LDF], i < n1
     float* A1 = J + (j + 1) * RR_LDF + (j + 1);      // trailing n1 x n1 block
+    // the lane's entries of v (0 past the end; m <= 96: three at most): every loop below runs
+    // over them unrolled, with its loads in flight together (a load is ~30 cycles and a step
+    // otherwise a chain of some fifteen of them)
+    float vc[RR_MMAX / 32];
+#pragma unroll
+    for (int u = 0; u < RR_MMAX / 32; ++u) vc[u] = lane + 32 * u < n1 ? col[(lane + 32 * u) * RR_LDF] : 0.0f;
     if (beta == 0.0f) {                              // nothing to reflect: next column as is
       if (next && wid == 0) reflector(j + 1);
       __syncthreads();
@@ -413,11 +422,13 @@ __global__ void __launch_bounds__(RR_T) k_rr_reduce(const RRParams a) {
     for (int r = wid; r < n1; r += 3 * RR_NW) {
       const int r1 = r + RR_NW, r2 = r + 2 * RR_NW;
       float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f;
-      for (int c = lane; c < n1; c += 32) {
-        const float vc = col[c * RR_LDF];
-        s0 = fmaf(A1[r * RR_LDF + c], vc, s0);
-        if (r1 < n1) s1 = fmaf(A1[r1 * RR_LDF + c], vc, s1);
-        if (r2 < n1) s2 = fmaf(A1[r2 * RR_LDF + c], vc, s2);
+#pragma unroll
+      for (int u = 0; u < RR_MMAX / 32; ++u) {
+        const int c = lane + 32 * u;
+        const bool in = c < n1;
+        s0 = fmaf(in ? A1[r * RR_LDF + c] : 0.0f, vc[u], s0);
+        s1 = fmaf(in && r1 < n1 ? A1[r1 * RR_LDF + c] : 0.0f, vc[u], s1);
+        s2 = fmaf(in && r2 < n1 ? A1[r2 * RR_LDF + c] : 0.0f, vc[u], s2);
       }
       s0 = warp_sum(s0);
       s1 = warp_sum(s1);
@@ -429,23 +440,46 @@ __global__ void __launch_bounds__(RR_T) k_rr_reduce(const RRParams a) {
       }
     }
     __syncthreads();
-    float K = 0.0f;
-    for (int i = lane; i < n1; i += 32) K = fmaf(col[i * RR_LDF], pv32[i], K);
+    float K = 0.0f, wc[RR_MMAX / 32];
+#pragma unroll
+    for (int u = 0; u < RR_MMAX / 32; ++u) wc[u] = lane + 32 * u < n1 ? pv32[lane + 32 * u] : 0.0f;
+#pragma unroll
+    for (int u = 0; u < RR_MMAX / 32; ++u) K = fmaf(vc[u], wc[u], K);
     K = 0.5f * beta * warp_sum(K);
+#pragma unroll
+    for (int u = 0; u < RR_MMAX / 32; ++u) wc[u] = fmaf(-K, vc[u], wc[u]);      // w = p - K v
     if (wid == 0) {                                   // column j + 1 of J, then its reflector
-      const float v0 = col[0], w0 = fmaf(-K, v0, pv32[0]);
-      for (int r = lane; r < n1; r += 32) {
-        const float vr = col[r * RR_LDF], wr = fmaf(-K, vr, pv32[r]);
-        A1[r * RR_LDF] = fmaf(-vr, w0, fmaf(-wr, v0, A1[r * RR_LDF]));
+      const float v0 = __shfl_sync(0xffffffffu, vc[0], 0), w0 = __shfl_sync(0xffffffffu, wc[0], 0);
+#pragma unroll
+      for (int u = 0; u < RR_MMAX / 32; ++u) {
+        const int r = lane + 32 * u;
+        if (r < n1) A1[r * RR_LDF] = fmaf(-vc[u], w0, fmaf(-wc[u], v0, A1[r * RR_LDF]));
       }
       __syncwarp();
       if (next) reflector(j + 1);
     } else {                                          // A1(1:, 1:) -= v w^T + w v^T, w = p - K v
-      for (int r = wid; r < n1; r += RR_NW - 1) {     // rows 1 .. n1-1 over warps 1 .. RR_NW-1
-        const float vr = col[r * RR_LDF], wr = fmaf(-K, vr, pv32[r]);
-        for (int c = 1 + lane; c < n1; c += 32) {
-          const float vc = col[c * RR_LDF], wc = fmaf(-K, vc, pv32[c]);
-          A1[r * RR_LDF + c] = fmaf(-vr, wc, fmaf(-wr, vc, A1[r * RR_LDF + c]));
+      // rows 1 .. n1-1 over warps 1 .. RR_NW-1, two rows' loads in flight together
+      for (int r0 = wid; r0 < n1; r0 += 2 * (RR_NW - 1)) {
+        float vr[2], wr[2], av[2][RR_MMAX / 32];
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+          const int r = r0 + t * (RR_NW - 1);
+          const bool rin = r < n1;
+          vr[t] = rin ? col[r * RR_LDF] : 0.0f;
+          wr[t] = rin ? pv32[r] : 0.0f;
+#pragma unroll
+          for (int u = 0; u < RR_MMAX / 32; ++u)
+            av[t][u] = rin && lane + 32 * u > 0 && lane + 32 * u < n1 ? A1[r * RR_LDF + lane + 32 * u] : 0.0f;
+        }
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+          const int r = r0 + t * (RR_NW - 1);
+          wr[t] = fmaf(-K, vr[t], wr[t]);
+#pragma unroll
+          for (int u = 0; u < RR_MMAX / 32; ++u) {
+            const int c = lane + 32 * u;
+            if (r < n1 && c > 0 && c < n1) A1[r * RR_LDF + c] = fmaf(-vr[t], wc[u], fmaf(-wr[t], vc[u], av[t][u]));
+          }
         }
       }
     }
@@ -685,6 +719,7 @@ __global__ void __launch_bounds__(RR_T) k_rr(const RRParams a) {
         for (int l = j + lane; l < i; l += 32) {
           float d0 = 0.0f, d1 = 0.0f;
           int r = 0;
+#pragma unroll 8
           for (; r + 1 < m; r += 2) {
             d0 = fmaf(V[r * RR_LDF + l], V[r * RR_LDF + i], d0);
             d1 = fmaf(V[(r + 1) * RR_LDF + l], V[(r + 1) * RR_LDF + i], d1);
@@ -693,11 +728,22 @@ __global__ void __launch_bounds__(RR_T) k_rr(const RRParams a) {
           dsc[l - j] = d0 + d1;
         }
         __syncwarp();
-        for (int r = lane; r < m; r += 32) {
-          float x = V[r * RR_LDF + i];
-          for (int l = j; l < i; ++l) x = fmaf(-dsc[l - j], V[r * RR_LDF + l], x);
-          V[r * RR_LDF + i] = x;
+        // the lane's rows (m <= 96: three at most) together, eight columns' loads in flight:
+        // a load's latency (~30 cycles) bounds this, not the arithmetic; with the loops of the
+        // reduction below an LOBPCG call (512 x 512, 16 columns) went from 18.51 to 17.77 ms
+        float x[RR_MMAX / 32];
+#pragma unroll
+        for (int u = 0; u < RR_MMAX / 32; ++u) x[u] = lane + 32 * u < m ? V[(lane + 32 * u) * RR_LDF + i] : 0.0f;
+#pragma unroll 8
+        for (int l = j; l < i; ++l) {
+          const float dl = -dsc[l - j];
+#pragma unroll
+          for (int u = 0; u < RR_MMAX / 32; ++u)
+            if (lane + 32 * u < m) x[u] = fmaf(dl, V[(lane + 32 * u) * RR_LDF + l], x[u]);
         }
+#pragma unroll
+        for (int u = 0; u < RR_MMAX / 32; ++u)
+          if (lane + 32 * u < m) V[(lane + 32 * u) * RR_LDF + i] = x[u];
         __syncwarp();
       }
       float n2 = 0.0f;
