@@ -134,3 +134,14 @@ def test_cg_and_lobpcg_concurrently_on_one_graph():
     assert torch.equal(xc, xs)
     assert torch.equal(lc["theta"], ls["theta"])
     assert torch.equal(lc["y"], ls["y"])
+
+
+@pytest.mark.parametrize("k", [5, 12, 20, 32])
+@pytest.mark.parametrize("pencil", ["D", "I"])
+def test_lobpcg_block_widths_and_pencils(k, pencil):
+    """The Gram kernel's copies and pixel groups at widths that are whole quads and that are
+    not, with and without a B diagonal, on an image that ends inside a chunk of pixels."""
+    _, g = image_case(41, 47, 16)
+    out, ref, O = run_pair(g, 3, 2.0, 0.08, k, 6, pencil=pencil)
+    assert ritz_ok(host(out["theta"]), ref["theta"]) < TOL_RITZ_SMALL_F32
+    assert rel_l2(host(out["y"]), ref["y"]) < TOL_F32
