@@ -462,7 +462,7 @@ def run_gpu(args):
 # capture of `bench.py --case apply` (512 x 512: the 16.8 MB of Y stay in L2 during the
 # launch) and of `bench.py --case apply --case-side 2048`
 TRAFFIC_APPLY_512 = 17909760
-TRAFFIC_APPLY_2048 = 499885824
+TRAFFIC_APPLY_2048 = 502832384
 FP32_LANES_PER_SM = 128
 # FP64 FMAs of one Rayleigh-Ritz call at m = 48, k = 16 (Cholesky with the forward solve
 # 2m^3/3, standard form m^3/6, M X twice 2 m^2 k, Gram/Löwdin/H 3 m k^2, back-substitution
@@ -470,7 +470,7 @@ FP32_LANES_PER_SM = 128
 # an ncu launch list of the timed step
 RR_FP64_FMA = (2 * 48 ** 3 / 3 + 48 ** 3 / 6 + 2 * 48 * 48 * 16 + 3 * 48 * 16 * 16
                + 48 * 48 * 16 / 2 + 48 * 48 * 16 + 2 * 48 * 16 * 16)
-RR_SHARE = 0.495
+RR_SHARE = 0.518
 
 
 def _sm_max_ghz():

@@ -232,6 +232,10 @@ int bf_reguided_filter(bf_graph* g, const void* x0, int iters, void* x_out, void
  * scalar state is initialised by a kernel, not copied from the host), so it can be
  * captured in a CUDA graph once an uncaptured call on the same graph has sized the
  * workspace (the first call, or one with a larger problem, may allocate it).
+ * Signals, 7 x 7 FP32 images with weights on the fly and guided FP32 images of radius <= 3
+ * whose vectors fit on the chip run, with T = Jacobi or identity, in one cooperative launch
+ * that tests the tolerance itself (no polling); its waits are bounded by a second, after
+ * which the run ends with BF_ETIMEOUT (reported through info; x_out is then undefined).
  * BF_PRECOND_NET takes T from opts->net, BF_PRECOND_SPD from opts->spd (both run s = T r
  * by kernels of their own after each update of x and r). */
 int cg_filter(const bf_graph* g, const void* x0, int kmax, const bf_cg_opts* opts,

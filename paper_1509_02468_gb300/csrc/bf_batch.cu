@@ -186,8 +186,9 @@ __device__ __forceinline__ void bdir_state(BState& st, double pq) {
 }
 
 // bcg_init_job and bcg_dir_job (below) of the image class, by runs: a tile of 1024 pixels per
-// pass instead of 256 with one pixel per thread (64 instances of 64 .. 512 pixels a side:
-// the class's direction kernel 88 us before).
+// pass instead of 256 with one pixel per thread.  20 iterations of 48 images of 64 .. 512 pixels
+// a side and 16 signals: 1432 us (3189 with one pixel per thread and the classes' launches one
+// behind the other); bound by the FP32 pipe at the larger images, by launches below.
 template <class SH>
 __device__ __forceinline__ void bcg_init_run(const RunConst& c, const BArgs& a, int job, unsigned char* smem) {
   __shared__ double red[4 * (BF_THREADS / 32)];

@@ -538,7 +538,8 @@ __global__ void __launch_bounds__(STRIP_THREADS, 2) k_cgs_dir(const Geom<float> 
 // k_cgs_init and k_cgs_dir with weights on the fly, by horizontal runs (bf_run.cuh).  nx: row
 // pitch of all arrays, nxr <= nx: image width; rows of a width that is not a multiple of four
 // are padded (k_cgr_pad: guide +inf, so the padding has no weight), which keeps every access
-// a 16-byte vector (1531 x 2047: 73 us an iteration unpadded).
+// a 16-byte vector.  An iteration of 1531 x 2047 pixels takes 57 us (direction 35, bound by the
+// FP32 pipe; update 18, by memory), 67 unpadded, 86 by vertical strips in scalar arithmetic.
 static_assert(RUN_THREADS == BF_THREADS, "the block reductions assume BF_THREADS threads");
 __global__ void __launch_bounds__(RUN_THREADS, 3)
 k_cgr_init(const __grid_constant__ RunConst c, int nx, int nxr, int ny, const __grid_constant__ RunSrc<2> src, int vec,
@@ -954,7 +955,10 @@ int cg_exec(const bf_graph* g, const T* x0, int kmax, const bf_cg_opts& o, T* x_
   const size_t sm = hp * 2 * sizeof(T);
   const bool guided = (g->kind == BF_KIND_GUIDED);
   int rc = BF_OK;
-  if (words) {                                     // the vectors fit on the chip: one launch
+  // The vectors fit on the chip: one launch.  50 iterations of 512 x 512 pixels take 436 us so
+  // and 1143 us by the run loop, whose launches and cold staging are 20 of its 23 us; near the
+  // largest image that fits an iteration takes 18 us (1040 x 1040), beyond it 33 (1100 x 1100).
+  if (words) {
     rc = cgp_launch<T>(g, a, kmax, s);
     if (rc) return rc;
   } else if (!guided && !net && sizeof(T) == 4 && fast_shape(g) == FAST_R3_2D &&

@@ -118,7 +118,9 @@ k_weights(const Geom<T> g, const T* __restrict__ guide, int64_t n, T* d, T* dinv
 // The degree and scalings of a float graph with the 7 x 7 window and weights on the fly, by
 // horizontal runs (bf_run.cuh); also copies the guide into the graph.  Bound by the SFU and
 // the FP32 pipe (48 exponentials and 4 x 48 lane operations per pixel) with 4 B read and
-// 20 B written per pixel beside them.
+// 20 B written per pixel beside them.  A graph update of 1080 x 1920 pixels with its degree
+// read back takes 59 us (139 with one pixel per thread and 49 global loads each); other
+// windows, types and stored weights stay on k_weights.
 __global__ void __launch_bounds__(RUN_THREADS, 3)
 k_weights_run(const __grid_constant__ RunConst c, int nx, int ny, const __grid_constant__ RunSrc<1> src, int vec,
               float* guide, float* d, float* dinv, float* dis, float* dls, int* flag) {
@@ -351,7 +353,9 @@ __global__ void __launch_bounds__(BF_THREADS) k_apply_fast(const Geom<float> g, 
 // One column (k = 1) through the 7 x 7 window with weights on the fly, by horizontal runs
 // (bf_run.cuh), persistent over 64 x 16 tiles: the L-type operators (SCALED: D^-1/2 L D^-1/2
 // and (diag L)^-1/2 L (diag L)^-1/2), or STEP: the BF step D^-1 W in difference form,
-// y_i = x_i - sum_j w_ij (x_i - x_j) / d_i; optional fused dot x^T y.
+// y_i = x_i - sum_j w_ij (x_i - x_j) / d_i; optional fused dot x^T y.  Bound by the FP32 pipe
+// as bf_run.cuh says.  Ten re-guided steps of 767 x 1021 pixels took 346 us with one pixel per
+// thread and 16 x 16 tiles, 205 us so.
 template <bool SCALED, bool STEP>
 __global__ void __launch_bounds__(RUN_THREADS, 3)
 k_apply1_run(const __grid_constant__ RunConst c, int nx, int ny, const __grid_constant__ RunSrc<SCALED ? 3 : 2> src,
@@ -740,7 +744,7 @@ __global__ void __launch_bounds__(PipeTile<K>::threads + PIPE_STAGERS, 1) k_appl
 // where they are issued.
 // Its tile: 12 computing warps (128 registers a thread with the two that copy), strips of two
 // pixels where a thread carries 16 columns: with four, the loads could only be issued two
-// steps ahead, 0.1 us before use, and the kernel waited for them (216 us).
+// steps ahead, 0.1 us before use, and the kernel waited for them (216 us; 140 us so).
 template <int K>
 struct PipeTileW {
   static constexpr int threads = 384;

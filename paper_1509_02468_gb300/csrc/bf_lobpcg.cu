@@ -187,9 +187,10 @@ __global__ void k_project(T* V, int k, int64_t n, const LobState* st) {
 // one pixel group of the staged chunk.  Float path: FP32 products summed over runs of 16
 // pixels, then folded by TwoSum into (hi, lo) pairs; groups are combined by a tree of
 // TwoSums, and the block partial hi + lo is written in FP64.
-// Issue slots bound it (60 % of them were address arithmetic, staging and folds): copies step
-// by a constant, folds are taken out of the pixel loop, arithmetic is on column pairs.  An
-// LOBPCG call (512 x 512, 16 columns) went from 17.77 to 17.45 ms with it.
+// Copies step by a constant, folds are out of the pixel loop and the arithmetic is on column
+// pairs, since 60 % of the issue slots went into addresses, staging and folds; what bounds it
+// now is latency at one CTA per SM (the accumulators take all registers).  An LOBPCG call (512
+// x 512, 16 columns) went from 17.77 to 17.45 ms with it.
 #define GRAM_T 512
 // pixels per shared-memory chunk (two buffers of S and A S chunks, m4 <= 96 columns each):
 // 128 in FP32 (193 KB), 64 in FP64; longer chunks mean fewer CTA barriers per pixel
