@@ -16,11 +16,11 @@
 // all-reduce is one write and one polled read of L2, and the halo words, written before it,
 // are there when it is done.  (With plain stores, a fence on either side and FP64 additions
 // the two all-reduces of an iteration took 17 of its 27 thousand cycles at 512 x 512.)
-// All CTAs add the partials alike and take the same decisions; the scalar recurrences are
-// in FP64.  50 iterations of 512 x 512 pixels: 436 us (two launches per iteration: 1347, and
-// 1143 with this file's window sums); the exchange is 2300 cycles per all-reduce of 144 CTAs
-// with a line of L2 per slot, 3100 with half a line, 7200 with slots packed, 2790 with an
-// atomic counter.
+// All CTAs add the partials alike and take the same decisions; sums and scalars are pairs of
+// floats in FP32 runs and FP64 in FP64 runs (see below).  50 iterations of 512 x 512 pixels:
+// 436 us (two launches per iteration: 1347, and 1143 with this file's window sums); the
+// exchange is 2300 cycles per all-reduce of 144 CTAs with a line of L2 per slot, 3100 with half
+// a line, 7200 with slots packed, 2790 with an atomic counter.
 //
 // Every wait is bounded (1 s by %globaltimer): a CTA that gives up sets the status to
 // CG_TIMEOUT; the others see it and leave too.
@@ -89,9 +89,14 @@ __device__ bool cgp_wait2(const u64* p, u64& a, u64& b, unsigned epoch, CgState*
 // ---- sums and scalars
 // A dependent FP64 addition takes about 115 cycles here and holds its scheduler's pipe for
 // 64, so FP32 runs carry their sums and scalars as unevaluated pairs of floats h + l (48 bits;
-// the terms are FP32 warp sums): an addition is a chain of six 4-cycle operations.  The pairs
-// are scaled by a power of two taken from the start's sums (which are FP64), so they do not
-// leave the FP32 range where the FP64 sums would not.  FP64 runs use FP64.
+// the terms are FP32 warp sums): an addition (Knuth's two-sum) is a chain of six 4-cycle
+// operations.  FP64 runs use FP64.
+// Sums are kept times a power of two (exact).  It is taken from the start's sums and again
+// from s^T r whenever that has left the range 2^+-CgpRange::BAND (cgp_prepare_beta): the sums
+// fall with the square of the residual, far past the range of a float (and, in FP64 runs, to
+// where alpha / s^T r overflows), while a run may go on for as long as the FP32 (FP64) terms
+// themselves have not vanished.  Scale and beta's factor are made while the update's words are
+// on their way: made before it, they cost 512 x 512 pixels 10 to 20 of its 436 us.
 struct CgpPair {
   float h, l;
 };
@@ -124,20 +129,6 @@ __device__ __forceinline__ void cgp_join(unsigned w0, unsigned w1, CgpPair& r) {
 __device__ __forceinline__ void cgp_join(unsigned w0, unsigned w1, double& r) {
   r = __longlong_as_double((long long)(((u64)w1 << 32) | w0));
 }
-__device__ __forceinline__ CgpPair cgp_div(CgpPair a, CgpPair b) {
-  const float r = __frcp_rn(b.h), q = a.h * r;
-  const float rem = fmaf(-q, b.h, a.h) + fmaf(-q, b.l, a.l);
-  return cgp_norm({q, rem * r});
-}
-// FP32 seed (error below 2^-22), one cubic step in FP64; a divisor outside the seed's range
-// takes the divide.
-__device__ __forceinline__ double cgp_div(double a, double b) {
-  const int e = (int)((__double_as_longlong(b) >> 52) & 0x7ff);
-  if (e < 1023 - 100 || e > 1023 + 100) return a / b;
-  const double r = (double)__frcp_rn((float)b);
-  const double d = fma(-b, r, 1.0);
-  return a * fma(r, fma(d, d, d), r);
-}
 __device__ __forceinline__ CgpPair cgp_mul(CgpPair a, CgpPair b) {
   const float p = a.h * b.h;
   return cgp_norm({p, fmaf(a.h, b.h, -p) + fmaf(a.h, b.l, a.l * b.h)});
@@ -161,19 +152,44 @@ __device__ __forceinline__ void cgp_set(double x, double& r) { r = x; }
 __device__ __forceinline__ float cgp_value(CgpPair a) { return a.h; }
 __device__ __forceinline__ double cgp_value(double a) { return a; }
 
+__device__ __forceinline__ CgpPair cgp_times(CgpPair a, float f) { return {a.h * f, a.l * f}; }
+__device__ __forceinline__ double cgp_times(double a, double f) { return a * f; }
+// exponent of a normal number (below every one of them for 0 and subnormal numbers)
+__device__ __forceinline__ int cgp_exponent(float a) { return (int)((__float_as_uint(a) >> 23) & 0xff) - 127; }
+__device__ __forceinline__ int cgp_exponent(double a) { return (int)((__double_as_longlong(a) >> 52) & 0x7ff) - 1023; }
+__device__ __forceinline__ void cgp_pow2(int k, float& r) { r = __uint_as_float((unsigned)(127 + k) << 23); }
+__device__ __forceinline__ void cgp_pow2(int k, double& r) { r = __longlong_as_double((long long)(1023 + k) << 52); }
+// Quotient by a reciprocal of the divisor's high part and one residual correction (a Newton
+// step); a divisor near the ends of the range, where the reciprocal or the residual would
+// leave it, is brought near 1 by a power of two first.
+__device__ __forceinline__ CgpPair cgp_div(CgpPair a, CgpPair b) {
+  float f = 1.0f;
+  const int e = cgp_exponent(b.h);
+  if (e < -100 || e > 100) {
+    cgp_pow2(max(-126, min(126, -e)), f);
+    b = cgp_times(b, f);
+  }
+  const float r = __frcp_rn(b.h), q = a.h * r;
+  const float rem = fmaf(-q, b.h, a.h) + fmaf(-q, b.l, a.l);
+  return cgp_times(cgp_norm({q, rem * r}), f);
+}
+__device__ __forceinline__ double cgp_div(double a, double b) { return a / b; }
+
 template <typename T> struct CgpNum;
 template <> struct CgpNum<float> { typedef CgpPair type; };
 template <> struct CgpNum<double> { typedef double type; };
+
+// Exponents: s^T r (scaled) stays within 2^+-BAND, the scale within 2^+-LIM.
+template <typename T> struct CgpRange;
+template <> struct CgpRange<float> { static constexpr int BAND = 20, LIM = 120; };
+template <> struct CgpRange<double> { static constexpr int BAND = 200, LIM = 900; };
 
 // What a CTA's threads share: the sums in flight (N) and the scalars of the run, which one
 // warp each computes (64 cycles of a scheduler per FP64 instruction and warp) for the others.
 template <typename T>
 struct CgpShared {
   typedef typename CgpNum<T>::type N;
-  union {
-    double d[4][CGP_T / 32];
-    N n[4][CGP_T / 32];
-  } red;
+  T red[4][CGP_T / 32];                    // the warps' sums, unscaled
   union {                                  // the CTAs' partial sums, [CTA][value]
     double d[CGP_MAXC * 4];
     N n[CGP_MAXC * 4];
@@ -181,36 +197,34 @@ struct CgpShared {
   double tot[4];                           // start: the four sums
   N sr, ss, rr, alpha, beta, cb;           // scaled by `scale`, except the quotients
   double ref2, thr;                        // thr: scaled tol^2 ref^2
-  float scale;                             // FP32 runs: of the sums (a power of two)
+  T scale, factor;                         // of the sums (a power of two); its next change
   int fin[4], conv, status;
 };
-template <typename T> __device__ __forceinline__ auto cgp_red(CgpShared<T>& sh, double*) -> decltype((sh.red.d)) { return sh.red.d; }
-__device__ __forceinline__ auto cgp_red(CgpShared<float>& sh, CgpPair*) -> decltype((sh.red.n)) { return sh.red.n; }
 template <typename T> __device__ __forceinline__ double* cgp_part(CgpShared<T>& sh, double*) { return sh.part.d; }
 __device__ __forceinline__ CgpPair* cgp_part(CgpShared<float>& sh, CgpPair*) { return sh.part.n; }
 
-// Sums of v (times scale) over all threads of all CTAs, and a barrier of the grid.  Warp
+// Sums of v (times sh.scale) over all threads of all CTAs, and a barrier of the grid.  Warp
 // w < NV gets the total of value w and calls tail(w, total) with all its lanes; what tail
 // writes to shared memory is visible to every thread on return.  `during` runs while the
 // words of the other CTAs are on their way.  R: representation of the sums.  Returns false
 // (in every thread) when a wait gave up.
 template <int NV, int NT, typename R, typename T, class During, class Tail>
-__device__ __forceinline__ bool cgp_allreduce(const T (&v)[4], T scale, CgpShared<T>& sh, u64* slots, unsigned epoch,
+__device__ __forceinline__ bool cgp_allreduce(const T (&v)[4], CgpShared<T>& sh, u64* slots, unsigned epoch,
                                               CgState* st, During during, Tail tail) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nc = gridDim.x;
   u64* base = slots + (size_t)(epoch & 1) * CGP_MAXC * CGP_SLOT;
-  auto& red = cgp_red(sh, (R*)nullptr);
   R* part = cgp_part(sh, (R*)nullptr);
   if (NV == 4) {
     const T w = warp_sum4<T>(v, lane);
-    if ((lane & 7) == 0) cgp_from(w * scale, red[lane >> 3][wid]);
+    if ((lane & 7) == 0) sh.red[lane >> 3][wid] = w;
   } else {
     const T w = warp_sum(v[0]);
-    if (lane == 0) cgp_from(w * scale, red[0][wid]);
+    if (lane == 0) sh.red[0][wid] = w;
   }
   __syncthreads();
   if (wid < NV) {
-    R t = red[wid][lane & (NT / 32 - 1)];
+    R t;
+    cgp_from(sh.red[wid][lane & (NT / 32 - 1)] * sh.scale, t);
 #pragma unroll
     for (int o = NT / 64; o > 0; o >>= 1) t = cgp_add(t, cgp_shfl(t, o));
     t = cgp_norm(t);
@@ -267,16 +281,10 @@ __device__ void cgp_start(CgpShared<T>& sh, double shift, double tol2) {
     sh.status = (cgp_finite(sr) && cgp_finite(ss) && cgp_finite(rr)) ? CG_RUN : CG_NONFINITE;
     const double b2 = shift * shift * sh.tot[3];
     sh.ref2 = b2 > 0.0 ? b2 : rr;
-    double sc = 1.0;
-    if (sizeof(T) == 4) {                      // 2^-exponent of the largest sum, within 2^+-120
-      const double m = fmax(fmax(fabs(sr), ss), rr);
-      const int e = (int)((__double_as_longlong(m) >> 52) & 0x7ff) - 1023;
-      const int k = max(-120, min(120, -e));
-      sh.scale = __uint_as_float((unsigned)(127 + k) << 23);
-      sc = (double)sh.scale;
-    } else {
-      sh.scale = 1.0f;
-    }
+    // 2^-exponent of the largest sum, within the scale's range
+    const int k = max(-CgpRange<T>::LIM, min(CgpRange<T>::LIM, -cgp_exponent(fmax(fmax(fabs(sr), ss), rr))));
+    cgp_pow2(k, sh.scale);
+    const double sc = (double)sh.scale;
     cgp_set(sr * sc, sh.sr);
     cgp_set(ss * sc, sh.ss);
     cgp_set(rr * sc, sh.rr);
@@ -286,7 +294,8 @@ __device__ void cgp_start(CgpShared<T>& sh, double shift, double tol2) {
   }
   __syncthreads();
 }
-// Direction (warp 0): p^T q -> the breakdown tests and alpha.
+// Direction (warp 0): p^T q -> the breakdown tests and alpha (not finite: the run stops
+// before x is touched).
 template <typename T>
 __device__ __forceinline__ void cgp_direction(CgpShared<T>& sh, typename CgpNum<T>::type pq, int lane) {
   int status = CG_RUN;
@@ -295,30 +304,44 @@ __device__ __forceinline__ void cgp_direction(CgpShared<T>& sh, typename CgpNum<
   else if (!cgp_finite(pq)) status = CG_NONFINITE;
   else if (cgp_zero(pq) || cgp_negative(pq)) status = CG_BREAK;
   const typename CgpNum<T>::type alpha = cgp_div(sr, pq);
+  if (status == CG_RUN && !cgp_finite(alpha)) status = CG_NONFINITE;
   if (lane == 0) {
     sh.status = status;
     if (status == CG_RUN) sh.alpha = alpha;
   }
 }
-// beta's factor -alpha / (s^T r or s^T s), by the last warp beside the update.
+// By the last thread, while the update's words are on their way: beta's factor -alpha / (s^T r or
+// s^T s), and the factor of the scale's change (1 until s^T r has left its band).
 template <typename T>
 __device__ __forceinline__ void cgp_prepare_beta(CgpShared<T>& sh, int beta_mode) {
-  if (threadIdx.x == blockDim.x - 1)
-    sh.cb = cgp_neg(cgp_div(sh.alpha, beta_mode == BF_BETA_PRINTED ? sh.ss : sh.sr));
+  if (threadIdx.x != blockDim.x - 1) return;
+  constexpr int BAND = CgpRange<T>::BAND, LIM = CgpRange<T>::LIM;
+  const int e = cgp_exponent(cgp_value(sh.sr));
+  T f = T(1);
+  if (e < -BAND || e > BAND) {
+    const int cur = cgp_exponent(sh.scale);
+    cgp_pow2(max(-LIM, min(LIM, max(-LIM, min(LIM, cur - e)) - cur)), f);
+  }
+  sh.factor = f;
+  sh.cb = cgp_neg(cgp_div(sh.alpha, beta_mode == BF_BETA_PRINTED ? sh.ss : sh.sr));
 }
-// Update (warps 0 .. 3): s^T r, s^T q, s^T s, r^T r -> beta and the stopping tests.
+// Update (warps 0 .. 3): s^T r, s^T q, s^T s, r^T r -> beta and the stopping tests, the sums in
+// the new scale.
 template <typename T>
 __device__ __forceinline__ void cgp_update_tail(CgpShared<T>& sh, int w, typename CgpNum<T>::type t, int lane) {
   typename CgpNum<T>::type b = t;
   if (w == 1) b = cgp_mul(sh.cb, t);
   if (lane != 0) return;
+  const T f = sh.factor;
   sh.fin[w] = cgp_finite(t);
-  if (w == 0) sh.sr = t;
+  if (w == 0) sh.sr = cgp_times(t, f);
   else if (w == 1) sh.beta = b;
-  else if (w == 2) sh.ss = t;
+  else if (w == 2) sh.ss = cgp_times(t, f);
   else {
-    sh.rr = t;
+    sh.rr = cgp_times(t, f);
     sh.conv = sh.thr >= 0.0 && cgp_double(t) <= sh.thr;
+    sh.thr *= (double)f;
+    sh.scale *= f;
   }
 }
 // After the update's all-reduce, by every thread: the status.
@@ -594,6 +617,7 @@ __global__ void __launch_bounds__(CGP_T, 1) k_cgp_image(const __grid_constant__ 
   const bool jac = a.cg.dinv != nullptr;
   const int beta_mode = a.cg.st->beta_mode;
   const double tol2 = a.cg.st->tol2;
+  if (threadIdx.x == 0) sh.scale = 1.0f;
   // ---- x0 on the rectangle and its halo, the operator's tiles, the degree
   for (int q = threadIdx.x; q < xs * (H + 2 * HALO); q += CGP_T) {
     const int hy = q / xs, hx = q - hy * xs;
@@ -672,14 +696,13 @@ __global__ void __launch_bounds__(CGP_T, 1) k_cgp_image(const __grid_constant__ 
       *reinterpret_cast<float4*>(X + y * W + x) = make_float4(xi[0], xi[1], xi[2], xi[3]);
       if (cnt) frame(x, y, cnt, s, 1u);
     }
-    if (!cgp_allreduce<4, CGP_T, double>(v, 1.0f, sh, a.slots, epoch, a.cg.st, halo_get, [&](int w, double t) {
+    if (!cgp_allreduce<4, CGP_T, double>(v, sh, a.slots, epoch, a.cg.st, halo_get, [&](int w, double t) {
           if (lane == 0) sh.tot[w] = t;
         }))
       return;
     cgp_start(sh, (double)a.cg.shift, tol2);
   }
   int it = 0, status = sh.status;
-  const float scale = sh.scale;
   for (; it < a.kmax && status == CG_RUN; ++it) {
     const float beta = cgp_value(sh.beta);     // 0 before the first step
     // ---- p = s + beta p
@@ -723,15 +746,13 @@ __global__ void __launch_bounds__(CGP_T, 1) k_cgp_image(const __grid_constant__ 
       }
       *reinterpret_cast<float4*>(Q + y * W + x) = make_float4(q[0], q[1], q[2], q[3]);
     }
-    if (!cgp_allreduce<1, CGP_T, N>(v, scale, sh, a.slots, ++epoch, a.cg.st, [] {},
+    if (!cgp_allreduce<1, CGP_T, N>(v, sh, a.slots, ++epoch, a.cg.st, [] {},
                                     [&](int, N t) { cgp_direction(sh, t, lane); }))
       return;
     status = sh.status;
     if (status != CG_RUN) break;
     // ---- x += alpha p, s -= alpha T q, the sums
     const float alpha = cgp_value(sh.alpha);
-    cgp_prepare_beta(sh, beta_mode);
-    cgp_history(sh, a.cg.hist, it);
     v[0] = 0.0f;
     for (int u = wid; u < nunits; u += CGP_T / 32) {
       const int x = (u % ux_n) * 32 + rx, y = (u / ux_n) * 4 + ry;
@@ -758,7 +779,12 @@ __global__ void __launch_bounds__(CGP_T, 1) k_cgp_image(const __grid_constant__ 
       *reinterpret_cast<float4*>(S + y * W + x) = make_float4(s[0], s[1], s[2], s[3]);
       if (cnt) frame(x, y, cnt, s, (unsigned)it + 2u);
     }
-    if (!cgp_allreduce<4, CGP_T, N>(v, scale, sh, a.slots, ++epoch, a.cg.st, halo_get,
+    auto during = [&] {
+      halo_get();
+      cgp_prepare_beta(sh, beta_mode);
+      cgp_history(sh, a.cg.hist, it);
+    };
+    if (!cgp_allreduce<4, CGP_T, N>(v, sh, a.slots, ++epoch, a.cg.st, during,
                                     [&](int w, N t) { cgp_update_tail(sh, w, t, lane); }))
       return;
     status = cgp_status(sh);
@@ -810,6 +836,7 @@ __global__ void __launch_bounds__(CGP_TL, 1) k_cgp_line(const __grid_constant__ 
   T* DI = Q + W;
   T* WF = DI + W;                              // [R][W + R], origin b - R
   const int b = blockIdx.x * W, len = min(W, n - b);
+  if (threadIdx.x == 0) sh.scale = T(1);
   // ---- x0 with halo, 1 / d, the weights
   for (int q = threadIdx.x; q < W + 2 * R; q += CGP_TL) {
     const int i = b - R + q;
@@ -891,14 +918,13 @@ __global__ void __launch_bounds__(CGP_TL, 1) k_cgp_line(const __grid_constant__ 
       v[2] = fma(r, r, v[2]);
       v[3] = fma(xi, xi, v[3]);
     }
-    if (!cgp_allreduce<4, CGP_TL, double>(v, T(1), sh, a.slots, epoch, a.cg.st, halo_get, [&](int w, double t) {
+    if (!cgp_allreduce<4, CGP_TL, double>(v, sh, a.slots, epoch, a.cg.st, halo_get, [&](int w, double t) {
           if (lane == 0) sh.tot[w] = t;
         }))
       return;
     cgp_start(sh, (double)a.cg.shift, tol2);
   }
   int it = 0, status = sh.status;
-  const T scale = (T)sh.scale;
   for (; it < a.kmax && status == CG_RUN; ++it) {
     const T beta = (T)cgp_value(sh.beta);      // 0 before the first step
     for (int q = threadIdx.x; q < W; q += CGP_TL) {
@@ -919,14 +945,12 @@ __global__ void __launch_bounds__(CGP_TL, 1) k_cgp_line(const __grid_constant__ 
       Q[q] = qq;
       v[0] = fma(p, qq, v[0]);
     }
-    if (!cgp_allreduce<1, CGP_TL, N>(v, scale, sh, a.slots, ++epoch, a.cg.st, [] {},
+    if (!cgp_allreduce<1, CGP_TL, N>(v, sh, a.slots, ++epoch, a.cg.st, [] {},
                                     [&](int, N t) { cgp_direction(sh, t, lane); }))
       return;
     status = sh.status;
     if (status != CG_RUN) break;
     const T alpha = (T)cgp_value(sh.alpha);
-    cgp_prepare_beta(sh, beta_mode);
-    cgp_history(sh, a.cg.hist, it);
     v[0] = T(0);
     for (int q = threadIdx.x; q < len; q += CGP_TL) {
       const T qq = Q[q];
@@ -940,7 +964,12 @@ __global__ void __launch_bounds__(CGP_TL, 1) k_cgp_line(const __grid_constant__ 
       v[2] = fma(s, s, v[2]);
       v[3] = fma(r, r, v[3]);
     }
-    if (!cgp_allreduce<4, CGP_TL, N>(v, scale, sh, a.slots, ++epoch, a.cg.st, halo_get,
+    auto during = [&] {
+      halo_get();
+      cgp_prepare_beta(sh, beta_mode);
+      cgp_history(sh, a.cg.hist, it);
+    };
+    if (!cgp_allreduce<4, CGP_TL, N>(v, sh, a.slots, ++epoch, a.cg.st, during,
                                     [&](int w, N t) { cgp_update_tail(sh, w, t, lane); }))
       return;
     status = cgp_status(sh);
