@@ -1300,10 +1300,8 @@ extern "C" int bf_weights(const bf_params* p, const void* guide, bf_graph** out,
   return BF_OK;
 }
 
-// Copy the guide into the graph and compute the degree, the scalings and (stored modes)
-// the weights; synchronises s to report a non-finite guide.
-// Eq. 2 weights, degree and scalings of g for a new guide, enqueued on s; a non-finite
-// guide value sets g->flag (which the caller clears and reads).
+// The guide, Eq. 2 weights (stored modes), degree and scalings of g for a new guide, enqueued on
+// s; a non-finite guide value sets g->flag, which read_flag reads and drop_flag clears.
 static int launch_weights(bf_graph* g, const void* guide, cudaStream_t s) {
   if (g->kind == BF_KIND_GUIDED) return bf_guided_prep(g, guide, s);
   cudaError_t e;
@@ -1361,25 +1359,30 @@ static int* pinned_flag() {
   return h.p;
 }
 
-// Wait for s and report a flagged guide.  The flag is 0 between calls (cleared when the graph
-// is made and whenever it was found set), so a call does not clear it first.
+// The flag is 0 between calls, on any stream: cleared when the graph is made, and here, with a
+// wait, by every call that found it set or that fails after it may have been set (`rc`: what
+// that call returns).  So a call that succeeds does not clear it first.
+static int drop_flag(bf_graph* g, cudaStream_t s, int rc) {
+  if (cudaMemsetAsync(g->flag, 0, sizeof(int), s) != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess)
+    (void)cudaGetLastError();
+  return rc;
+}
+
+// Wait for s and report a flagged guide.
 static int read_flag(bf_graph* g, cudaStream_t s, const char* what) {
   cudaError_t e;
   int local = 0, *pin = pinned_flag();
   volatile int& hflag = pin ? *pin : local;
   if ((e = cudaMemcpyAsync((void*)&hflag, g->flag, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess)
-    return bf_cuda_fail(e, "cudaMemcpyAsync(flag)");
-  if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return bf_cuda_fail(e, "weights sync");
-  if (hflag) {
-    if ((e = cudaMemsetAsync(g->flag, 0, sizeof(int), s)) != cudaSuccess) return bf_cuda_fail(e, "memset(flag)");
-    return bf_fail(BF_ENONFINITE, what);
-  }
+    return drop_flag(g, s, bf_cuda_fail(e, "cudaMemcpyAsync(flag)"));
+  if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return drop_flag(g, s, bf_cuda_fail(e, "weights sync"));
+  if (hflag) return drop_flag(g, s, bf_fail(BF_ENONFINITE, what));
   return BF_OK;
 }
 
 static int compute_weights(bf_graph* g, const void* guide, cudaStream_t s) {
   const int rc = launch_weights(g, guide, s);
-  if (rc) return rc;
+  if (rc) return drop_flag(g, s, rc);
   return read_flag(g, s, "bf_weights: guide holds NaN or Inf");
 }
 
@@ -1474,7 +1477,7 @@ extern "C" int bf_reguided_filter(bf_graph* g, const void* x0, int iters, void* 
     void* dst = (last && x_out != src) ? x_out : tmp[it & 1];
     if (!otf) {
       rc = launch_weights(g, src, s);
-      if (rc) return rc;
+      if (rc) return drop_flag(g, s, rc);
     }
     if (g->kind == BF_KIND_GUIDED)                   // the window statistics of src are in g
       rc = (g->esize == 4)
@@ -1484,12 +1487,12 @@ extern "C" int bf_reguided_filter(bf_graph* g, const void* x0, int iters, void* 
       rc = (g->esize == 4)
                ? apply_bf_step_with_guide<float>(g, (const float*)src, (const float*)src, (float*)dst, s)
                : apply_bf_step_with_guide<double>(g, (const double*)src, (const double*)src, (double*)dst, s);
-    if (rc) return rc;
-    if (last && otf) {
-      rc = launch_weights(g, src, s);              // src is intact: dst differs from it
-      if (rc) return rc;
+    if (!rc && last && otf) rc = launch_weights(g, src, s);   // src is intact: dst differs from it
+    if (!rc && last && dst != x_out) {
+      const cudaError_t e = cudaMemcpyAsync(x_out, dst, nb, cudaMemcpyDeviceToDevice, s);
+      if (e != cudaSuccess) rc = bf_cuda_fail(e, "cudaMemcpyAsync(x_out)");
     }
-    if (last && dst != x_out) BF_CUDA(cudaMemcpyAsync(x_out, dst, nb, cudaMemcpyDeviceToDevice, s));
+    if (rc) return drop_flag(g, s, rc);
     src = dst;
   }
   return read_flag(g, s, "bf_reguided_filter: an iterate holds NaN or Inf");
