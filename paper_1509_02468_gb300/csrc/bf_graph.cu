@@ -18,6 +18,7 @@
 #include "bf_strip.cuh"
 #include "bf_hrun.cuh"
 #include "bf_run.cuh"
+#include "bf_index.h"
 
 // ================================================================== errors
 static thread_local std::string g_last_error;
@@ -793,7 +794,7 @@ __device__ __forceinline__ void pipe_step_w(const void* wf, int n, int nx, int n
     bool in = true;
     if (MASK)
       in = x < nx && y0 + p < ny && (unsigned)(x + dx) < (unsigned)nx && (unsigned)(y0 + p + dy) < (unsigned)ny;
-    w[p] = in ? pipe_ld_w<WM>((const char*)wf, off + (unsigned)(e * ES)) : 0.0f;
+    w[p] = in ? pipe_ld_w<WM>((const char*)wf, off + bf_byte_offset(e, ES)) : 0.0f;
   }
 }
 
@@ -951,8 +952,8 @@ static int launch_apply_rb_w(const bf_graph* g, const ApplyArgs<float>& a, cudaS
   if (a.op == BF_OP_L && !a.scale && ((uintptr_t)a.X & 15) == 0 && ((uintptr_t)a.Y & 15) == 0 && a.ldx % 4 == 0 &&
       a.ldy % 4 == 0) {
     // (the stored kernel's byte offsets are 32-bit)
-    if (g->p.weight_mode == BF_W_STORED_F32 && g->n < 44000000) return launch_apply_pipe_w<K, BF_W_STORED_F32>(g, a, s);
-    if (g->p.weight_mode == BF_W_STORED_BF16 && g->n < 44000000) return launch_apply_pipe_w<K, BF_W_STORED_BF16>(g, a, s);
+    if (g->p.weight_mode == BF_W_STORED_F32 && g->n < BF_PIPE_W_MAX_N) return launch_apply_pipe_w<K, BF_W_STORED_F32>(g, a, s);
+    if (g->p.weight_mode == BF_W_STORED_BF16 && g->n < BF_PIPE_W_MAX_N) return launch_apply_pipe_w<K, BF_W_STORED_BF16>(g, a, s);
     if (g->p.weight_mode == BF_W_ONTHEFLY && g->gf.a_r > 0.0f) return launch_apply_pipe<K>(g, a, s);
   }
   if (g->p.weight_mode == BF_W_ONTHEFLY) return launch_apply_rb<K, false>(g, a, s);
