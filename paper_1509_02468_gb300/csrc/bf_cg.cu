@@ -811,12 +811,14 @@ int cg_strip_loop_w(const bf_graph* g, CgArgs<float>& a, int kmax, double tol, c
   return BF_OK;
 }
 
-// Whether a run with weights on the fly pads its rows (it must have asked for the room), and
-// to what pitch.
+// Whether runs on a graph with weights on the fly pad their rows when T = Jacobi or identity, and
+// to what pitch.  A workspace that grew would leave runs captured in a CUDA graph with the old
+// one, so its size is a matter of the graph alone: the room is there for any T, and a graph whose
+// larger workspace could not be had (no_pad) stays with the smaller one.
 int cg_pitch(int nx) { return (nx + 3) & ~3; }
-bool cg_pads(const bf_graph* g, const bf_cg_opts& o) {
+bool cg_pad_room(const bf_graph* g) {
   return g->kind == BF_KIND_BILATERAL && fast_shape(g) == FAST_R3_2D && g->p.weight_mode == BF_W_ONTHEFLY &&
-         g->nx % 4 != 0 && g->gf.a_r > 0.0f && (o.precond == BF_PRECOND_JACOBI || o.precond == BF_PRECOND_IDENTITY) && !cgp_words(g);
+         g->nx % 4 != 0 && g->gf.a_r > 0.0f && !g->no_pad && !cgp_words(g);
 }
 
 template <class F>
@@ -1001,13 +1003,25 @@ template <typename T>
 int cg_run(const bf_graph* g, const T* x0, int kmax, const bf_cg_opts& o, T* x_out,
            bf_info* info, cudaStream_t s) {
   bf_graph* gm = const_cast<bf_graph*>(g);
-  const bool pads = sizeof(T) == 4 && cg_pads(g, o);
-  const int nv = pads ? 8 : 5;
-  const size_t vb = ((size_t)(pads ? (int64_t)cg_pitch(g->nx) * g->ny : g->n) * sizeof(T) + 255) & ~(size_t)255;
+  bool room = sizeof(T) == 4 && cg_pad_room(g);
   const size_t pb =
       (std::max((size_t)cg_partial_slots(g) * 4 * sizeof(double), 8 * cgp_words(g)) + 255) & ~(size_t)255;
-  int rc = bf_ws_reserve(gm, BF_WS_CG, nv * vb + pb + 256);
+  int nv = 0;
+  size_t vb = 0;
+  auto reserve = [&] {
+    nv = room ? 8 : 5;
+    vb = ((size_t)(room ? (int64_t)cg_pitch(g->nx) * g->ny : g->n) * sizeof(T) + 255) & ~(size_t)255;
+    return bf_ws_reserve(gm, BF_WS_CG, nv * vb + pb + 256);
+  };
+  int rc = reserve();
+  if (rc == BF_ENOMEM && room) {
+    (void)cudaGetLastError();
+    gm->no_pad = 1;
+    room = false;
+    rc = reserve();
+  }
   if (rc) return rc;
+  const bool pads = room && (o.precond == BF_PRECOND_JACOBI || o.precond == BF_PRECOND_IDENTITY);
   char* w = (char*)gm->ws[BF_WS_CG];
   CgBufs<T> b;
   b.r = (T*)(w);
@@ -1237,7 +1251,7 @@ int cg_run_noalloc(const bf_graph* g, const T* x0, int kmax, const bf_cg_opts& o
   b.q = (T*)(w + 2 * BF_NOALLOC_VEC_BYTES);
   b.p[0] = (T*)(w + 3 * BF_NOALLOC_VEC_BYTES);
   b.p[1] = (T*)(w + 4 * BF_NOALLOC_VEC_BYTES);
-  b.pad[0] = b.pad[1] = b.pad[2] = nullptr;      // (larger than what would need it)
+  b.pad[0] = b.pad[1] = b.pad[2] = nullptr;      // no room: rows that are not whole vectors go unpadded
   b.partials = (double*)(w + 5 * BF_NOALLOC_VEC_BYTES);
   b.st = (CgState*)(w + 5 * BF_NOALLOC_VEC_BYTES + (size_t)BF_NOALLOC_MAX_BLOCKS * 4 * sizeof(double));
   return cg_exec<T>(g, x0, kmax, o, x_out, info, s, b, "cg_filter_noalloc");

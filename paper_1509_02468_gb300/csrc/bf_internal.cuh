@@ -114,6 +114,7 @@ struct bf_graph {
   Geom<double> gd;
   void* ws[3];           // grow-only workspaces, one per filter family (BF_WS_*)
   size_t ws_bytes[3];
+  int no_pad;            // the CG workspace has no room for padded rows (it could not be had)
   int* flag;             // [1] non-finite guide flag of the weights kernel
   int kind;              // BF_KIND_*
   double eps;            // guided: epsilon of Algorithm 1
