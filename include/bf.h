@@ -235,7 +235,10 @@ int bf_reguided_filter(bf_graph* g, const void* x0, int iters, void* x_out, void
  * Signals, 7 x 7 FP32 images with weights on the fly and guided FP32 images of radius <= 3
  * whose vectors fit on the chip run, with T = Jacobi or identity, in one cooperative launch
  * that tests the tolerance itself (no polling); its waits are bounded by a second, after
- * which the run ends with BF_ETIMEOUT (reported through info; x_out is then undefined).
+ * which the run ends with BF_ETIMEOUT (reported through info; each part of x_out then holds
+ * the iterate that it had reached).  The launch needs up to all SMs but four at one moment: it
+ * starts when blocks of other streams have left it that many, where the two kernels per
+ * iteration of the other form fill in between them.
  * BF_PRECOND_NET takes T from opts->net, BF_PRECOND_SPD from opts->spd (both run s = T r
  * by kernels of their own after each update of x and r). */
 int cg_filter(const bf_graph* g, const void* x0, int kmax, const bf_cg_opts* opts,

@@ -49,6 +49,15 @@ int bf_gram_tc_test(const float* S0, const float* S1, const float* S2, const flo
  * intact.  Synchronises the stream. */
 int bf_wait_test(int iters, int arrive, void* stream);
 
+/* cg_filter (Jacobi, flexible beta, no shift) on a graph that runs in one cooperative launch of
+ * more than one CTA, with CTA `absent` leaving before it sends anything, so that every other
+ * CTA's bounded wait runs out (1 s): returns BF_ETIMEOUT and leaves the context and the graph
+ * usable; x_out holds x0 except for the absent CTA's part, which is not written.  BF_EINVAL
+ * for a graph that takes another form.  Needs the graph type from bf.h. */
+struct bf_graph;
+int bf_cg_wait_test(const struct bf_graph* g, const void* x0, int kmax, int absent, void* x_out,
+                    void* stream);
+
 /* bf_batch_cg_persistent (Jacobi, flexible beta, no shift) with CTA 0 leaving before its
  * first grid barrier, so that every other CTA's bounded wait runs out: returns
  * BF_ETIMEOUT and leaves the context usable.  Needs the batch type from bf.h. */

@@ -113,6 +113,7 @@ def _load():
         "bf_spd_adam": [vp, ctypes.c_float, ctypes.c_float, vp],
         "bf_gram_tc_test": [vp, vp, vp, vp, vp, vp, vp, i32, i32, i64, i32, vp, vp],
         "bf_wait_test": [i32, i32, vp],
+        "bf_cg_wait_test": [vp, vp, i32, i32, vp, vp],
         "bf_batch_create": [vp, i32, ctypes.POINTER(vp)],
         "bf_batch_free": [vp],
         "bf_batch_cg": [vp, vp, vp, i32, ctypes.POINTER(bf_cg_opts), vp, vp],
@@ -620,6 +621,14 @@ def wait_test(iters: int, arrive: bool, stream=None):
     """The library's bounded device wait on a barrier of its own (include/bf_testing.h):
     returns normally when thread 0 arrives, raises BFError(BF_ETIMEOUT) when nothing does."""
     _check(_lib.bf_wait_test(int(iters), int(bool(arrive)), _stream(stream)))
+
+
+def cg_wait_test(g: Graph, x0: torch.Tensor, kmax: int = 2, absent: int = 0, out=None, stream=None):
+    """One-launch CG run with one CTA that never sends anything (include/bf_testing.h): raises
+    BFError(BF_ETIMEOUT)."""
+    out = torch.empty_like(x0) if out is None else out
+    _check(_lib.bf_cg_wait_test(g.handle, _ptr(x0), kmax, absent, _ptr(out), _stream(stream)))
+    return out
 
 
 def gram_tc(S_blocks, AS_blocks, b=None, split: bool = False, stream=None, mode: str | None = None):

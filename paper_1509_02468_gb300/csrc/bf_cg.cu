@@ -921,7 +921,7 @@ struct CgBufs {
 // library's static array).  `who` names the entry point in error messages.
 template <typename T>
 int cg_exec(const bf_graph* g, const T* x0, int kmax, const bf_cg_opts& o, T* x_out,
-            bf_info* info, cudaStream_t s, const CgBufs<T>& b, const char* who) {
+            bf_info* info, cudaStream_t s, const CgBufs<T>& b, const char* who, int absent = -1) {
   const int64_t n = g->n;
   const dim3 tg = tile_grid(g);
   const unsigned nb_elem = (unsigned)std::min<int64_t>((n + BF_THREADS - 1) / BF_THREADS, 8 * cg_num_sms());
@@ -942,6 +942,7 @@ int cg_exec(const bf_graph* g, const T* x0, int kmax, const bf_cg_opts& o, T* x_
   a.shift = (T)o.shift;
   a.hist = o.hist;
   a.first = 1;
+  a.absent = absent;
   a.p_old = b.p[0];
   a.p_new = b.p[1];
   const bool net = (o.precond == BF_PRECOND_NET || o.precond == BF_PRECOND_SPD);
@@ -1001,7 +1002,7 @@ inline unsigned cg_partial_slots(const bf_graph* g) {
 
 template <typename T>
 int cg_run(const bf_graph* g, const T* x0, int kmax, const bf_cg_opts& o, T* x_out,
-           bf_info* info, cudaStream_t s) {
+           bf_info* info, cudaStream_t s, int absent = -1) {
   bf_graph* gm = const_cast<bf_graph*>(g);
   bool room = sizeof(T) == 4 && cg_pad_room(g);
   const size_t pb =
@@ -1032,7 +1033,7 @@ int cg_run(const bf_graph* g, const T* x0, int kmax, const bf_cg_opts& o, T* x_o
   for (int j = 0; j < 3; ++j) b.pad[j] = pads ? (T*)(w + (5 + j) * vb) : nullptr;
   b.partials = (double*)(w + nv * vb);
   b.st = (CgState*)(w + nv * vb + pb);
-  return cg_exec<T>(g, x0, kmax, o, x_out, info, s, b, "cg_filter");
+  return cg_exec<T>(g, x0, kmax, o, x_out, info, s, b, "cg_filter", absent);
 }
 
 }  // namespace
@@ -1059,6 +1060,17 @@ extern "C" int cg_filter(const bf_graph* g, const void* x0, int kmax, const bf_c
   cudaStream_t s = (cudaStream_t)stream;
   if (g->esize == 4) return cg_run<float>(g, (const float*)x0, kmax, o, (float*)x_out, info, s);
   return cg_run<double>(g, (const double*)x0, kmax, o, (double*)x_out, info, s);
+}
+
+extern "C" int bf_cg_wait_test(const bf_graph* g, const void* x0, int kmax, int absent, void* x_out, void* stream) {
+  if (!g || !x0 || !x_out || kmax < 0 || absent < 0) return bf_fail(BF_EINVAL, "bf_cg_wait_test: bad argument");
+  if (!cgp_words(g)) return bf_fail(BF_EINVAL, "bf_cg_wait_test: the graph does not run in one launch");
+  bf_cg_opts o;
+  memset(&o, 0, sizeof(o));
+  bf_info info;
+  cudaStream_t s = (cudaStream_t)stream;
+  if (g->esize == 4) return cg_run<float>(g, (const float*)x0, kmax, o, (float*)x_out, &info, s, absent);
+  return cg_run<double>(g, (const double*)x0, kmax, o, (double*)x_out, &info, s, absent);
 }
 
 // ==================================================================== refinement

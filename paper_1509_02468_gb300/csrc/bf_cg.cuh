@@ -43,6 +43,7 @@ struct CgArgs {
   double* partials;
   CgState* st;
   double* hist;        // [2 kmax] or NULL
+  int absent;          // testing: the CTA of a one-launch run that leaves before it sends anything (-1: none)
 };
 
 // The whole run in one cooperative launch with its vectors on the chip (bf_cgp.cu).

@@ -23,7 +23,7 @@
 // a line, 7200 with slots packed, 2790 with an atomic counter.
 //
 // Every wait is bounded (1 s by %globaltimer): a CTA that gives up sets the status to
-// CG_TIMEOUT; the others see it and leave too.
+// CG_TIMEOUT; the others see it and leave too, each with its part of x as far as it has come.
 #include <math.h>
 
 #include <algorithm>
@@ -596,12 +596,30 @@ __device__ __forceinline__ void cgp_halo_pos(int h, int W, int H, int& tx, int& 
   }
 }
 
+// x of the rectangle to the image, at the end and when a wait gives up (as far as the run has
+// come).  Not inlined: with the store in place and breaks out of the loop to it, 512 x 512 pixels
+// take 30 us more (the window sums are the same code; where it lies is not).
+__device__ __noinline__ void cgp_store_x(const CgpImage& a, const float* X) {
+  const int W = a.rc.W, H = a.rc.H;
+  const int bx = (blockIdx.x % a.rc.ncx) * W, by = (blockIdx.x / a.rc.ncx) * H;
+  const bool vec = a.vec && ((uintptr_t)a.cg.x & 15) == 0;
+  __syncthreads();
+  for (int q = threadIdx.x; q < W * H / 4; q += CGP_T) {
+    const int y = 4 * q / W, x = 4 * q - y * W;
+    const int cnt = run_count(bx + x, by + y, a.nx, a.ny);
+    const float4 x4 = *reinterpret_cast<const float4*>(X + 4 * q);
+    const float xv[4] = {x4.x, x4.y, x4.z, x4.w};
+    if (cnt) run_store(a.cg.x, (int64_t)(by + y) * a.nx + bx + x, cnt, vec, xv);
+  }
+}
+
 template <class OP>
 __global__ void __launch_bounds__(CGP_T, 1) k_cgp_image(const __grid_constant__ OP op, const __grid_constant__ CgpImage a) {
   constexpr int HALO = OP::HALO, LP = OP::LP;
   extern __shared__ __align__(16) float cgp_smem[];
   typedef CgpPair N;
   __shared__ CgpShared<float> sh;
+  if ((int)blockIdx.x == a.cg.absent) return;
   const int W = a.rc.W, H = a.rc.H, xs = W + 2 * LP;
   const int nx = a.nx, ny = a.ny;
   float* P = cgp_smem;
@@ -699,7 +717,7 @@ __global__ void __launch_bounds__(CGP_T, 1) k_cgp_image(const __grid_constant__ 
     if (!cgp_allreduce<4, CGP_T, double>(v, sh, a.slots, epoch, a.cg.st, halo_get, [&](int w, double t) {
           if (lane == 0) sh.tot[w] = t;
         }))
-      return;
+      return cgp_store_x(a, X);
     cgp_start(sh, (double)a.cg.shift, tol2);
   }
   int it = 0, status = sh.status;
@@ -727,7 +745,7 @@ __global__ void __launch_bounds__(CGP_T, 1) k_cgp_image(const __grid_constant__ 
         const float s = himg[k] >= 0 ? __uint_as_float((unsigned)hw[k]) : 0.0f;
         P[htile[k]] = it ? fmaf(beta, P[htile[k]], s) : s;
       }
-    if (__syncthreads_or(!ok)) return;
+    if (__syncthreads_or(!ok)) return cgp_store_x(a, X);
     // ---- q = (L + sigma I) p, p^T q
     float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     op.prepare(P, EX, W, H, bx, by, nx, ny);
@@ -748,7 +766,7 @@ __global__ void __launch_bounds__(CGP_T, 1) k_cgp_image(const __grid_constant__ 
     }
     if (!cgp_allreduce<1, CGP_T, N>(v, sh, a.slots, ++epoch, a.cg.st, [] {},
                                     [&](int, N t) { cgp_direction(sh, t, lane); }))
-      return;
+      return cgp_store_x(a, X);
     status = sh.status;
     if (status != CG_RUN) break;
     // ---- x += alpha p, s -= alpha T q, the sums
@@ -786,16 +804,10 @@ __global__ void __launch_bounds__(CGP_T, 1) k_cgp_image(const __grid_constant__ 
     };
     if (!cgp_allreduce<4, CGP_T, N>(v, sh, a.slots, ++epoch, a.cg.st, during,
                                     [&](int w, N t) { cgp_update_tail(sh, w, t, lane); }))
-      return;
+      return cgp_store_x(a, X);
     status = cgp_status(sh);
   }
-  for (int u = wid; u < nunits; u += CGP_T / 32) {
-    const int x = (u % ux_n) * 32 + rx, y = (u / ux_n) * 4 + ry;
-    const int cnt = run_count(bx + x, by + y, nx, ny);
-    const float4 x4 = *reinterpret_cast<const float4*>(X + y * W + x);
-    const float xv[4] = {x4.x, x4.y, x4.z, x4.w};
-    if (cnt) run_store(a.cg.x, (int64_t)(by + y) * nx + bx + x, cnt, a.vec && (((uintptr_t)a.cg.x & 15) == 0), xv);
-  }
+  cgp_store_x(a, X);
   cgp_write_state(sh, a.cg.st, it, status);
 }
 
@@ -819,11 +831,20 @@ __host__ __device__ inline size_t cgp_line_elems(int W, int R) {
   return (size_t)(W + 2 * R) + 5 * (size_t)W + (size_t)R * (W + R);
 }
 
+// x of the piece to the signal.
+template <typename T>
+__device__ __noinline__ void cgp_store_x(const CgpLine<T>& a, const T* X) {
+  const int b = blockIdx.x * a.W, len = min(a.W, a.n - b);
+  __syncthreads();
+  for (int q = threadIdx.x; q < len; q += CGP_TL) a.cg.x[b + q] = X[q];
+}
+
 template <typename T>
 __global__ void __launch_bounds__(CGP_TL, 1) k_cgp_line(const __grid_constant__ CgpLine<T> a) {
   extern __shared__ __align__(16) float cgp_smem[];
   typedef typename CgpNum<T>::type N;
   __shared__ CgpShared<T> sh;
+  if ((int)blockIdx.x == a.cg.absent) return;
   const int lane = threadIdx.x & 31;
   const int W = a.W, R = a.R, n = a.n;
   const int beta_mode = a.cg.st->beta_mode;
@@ -921,7 +942,7 @@ __global__ void __launch_bounds__(CGP_TL, 1) k_cgp_line(const __grid_constant__ 
     if (!cgp_allreduce<4, CGP_TL, double>(v, sh, a.slots, epoch, a.cg.st, halo_get, [&](int w, double t) {
           if (lane == 0) sh.tot[w] = t;
         }))
-      return;
+      return cgp_store_x(a, X);
     cgp_start(sh, (double)a.cg.shift, tol2);
   }
   int it = 0, status = sh.status;
@@ -938,7 +959,7 @@ __global__ void __launch_bounds__(CGP_TL, 1) k_cgp_line(const __grid_constant__ 
                                          : (T)__longlong_as_double((long long)((hw[1] << 32) | (hw[0] & 0xffffffffull))));
       *hp = it ? fma(beta, *hp, s) : s;
     }
-    if (__syncthreads_or(!ok)) return;
+    if (__syncthreads_or(!ok)) return cgp_store_x(a, X);
     T v[4] = {T(0), T(0), T(0), T(0)};
     for (int q = threadIdx.x; q < len; q += CGP_TL) {
       const T p = P[q + R], qq = fma(a.cg.shift, p, lap(q));
@@ -947,7 +968,7 @@ __global__ void __launch_bounds__(CGP_TL, 1) k_cgp_line(const __grid_constant__ 
     }
     if (!cgp_allreduce<1, CGP_TL, N>(v, sh, a.slots, ++epoch, a.cg.st, [] {},
                                     [&](int, N t) { cgp_direction(sh, t, lane); }))
-      return;
+      return cgp_store_x(a, X);
     status = sh.status;
     if (status != CG_RUN) break;
     const T alpha = (T)cgp_value(sh.alpha);
@@ -971,10 +992,10 @@ __global__ void __launch_bounds__(CGP_TL, 1) k_cgp_line(const __grid_constant__ 
     };
     if (!cgp_allreduce<4, CGP_TL, N>(v, sh, a.slots, ++epoch, a.cg.st, during,
                                     [&](int w, N t) { cgp_update_tail(sh, w, t, lane); }))
-      return;
+      return cgp_store_x(a, X);
     status = cgp_status(sh);
   }
-  for (int q = threadIdx.x; q < len; q += CGP_TL) a.cg.x[b + q] = X[q];
+  cgp_store_x(a, X);
   cgp_write_state(sh, a.cg.st, it, status);
 }
 
