@@ -1022,7 +1022,8 @@ int cg_run(const bf_graph* g, const T* x0, int kmax, const bf_cg_opts& o, T* x_o
     rc = reserve();
   }
   if (rc) return rc;
-  const bool pads = room && (o.precond == BF_PRECOND_JACOBI || o.precond == BF_PRECOND_IDENTITY);
+  // (no step: copying into padded rows took 25 of 124 us at 2048 x 2047)
+  const bool pads = room && kmax > 0 && (o.precond == BF_PRECOND_JACOBI || o.precond == BF_PRECOND_IDENTITY);
   char* w = (char*)gm->ws[BF_WS_CG];
   CgBufs<T> b;
   b.r = (T*)(w);

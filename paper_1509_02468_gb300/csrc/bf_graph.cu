@@ -121,7 +121,10 @@ k_weights(const Geom<T> g, const T* __restrict__ guide, int64_t n, T* d, T* dinv
 // the FP32 pipe (48 exponentials and 4 x 48 lane operations per pixel) with 4 B read and
 // 20 B written per pixel beside them.  A graph update of 1080 x 1920 pixels with its degree
 // read back takes 59 us (139 with one pixel per thread and 49 global loads each); other
-// windows, types and stored weights stay on k_weights.
+// windows, types and stored weights stay on k_weights, and so do images of fewer than 12 columns
+// or 4 rows, of which a 64 x 16 tile holds too little (2.4 million pixels, runs against k_weights:
+// 1 column 1668 and 104 us, 6: 323 and 143, 12: 150 and 146; 1 row 364 and 104, 3: 139 and 115,
+// 4: 115 and 123).
 __global__ void __launch_bounds__(RUN_THREADS, 3)
 k_weights_run(const __grid_constant__ RunConst c, int nx, int ny, const __grid_constant__ RunSrc<1> src, int vec,
               float* guide, float* d, float* dinv, float* dis, float* dls, int* flag) {
@@ -947,13 +950,34 @@ static int launch_apply_rb(const bf_graph* g, const ApplyArgs<float>& a, cudaStr
   return BF_OK;
 }
 
+// Whether the stored-weight walk is taken rather than k_apply_rb, whose tiles are lower.  The walk
+// reads and sums rows that do not exist: below three or four rows it is the slower one (2.4
+// million pixels in one row, FP32 weights: 8 columns 5276 us against 3677, 16: 4505 against 3694;
+// in four rows 1450 against 2147 and 1208 against 2192).  Where it is little faster per pixel (four
+// columns of FP32 weights, eight of BF16: 0.85 of the time), its rows in the image's last tiles
+// must not cost more than that, unless every tile has an SM to itself (64 rows of 37500 pixels: 4
+// columns, FP32 164 us against 142; 8 columns, BF16 812 against 616).
+template <int K>
+static bool pipe_w_pays(const bf_graph* g) {
+  const bool bf16 = g->p.weight_mode == BF_W_STORED_BF16;
+  if (K == 4 && bf16) return true;
+  if (g->ny < (K >= 16 && !bf16 ? 3 : 4)) return false;
+  if (!(K == 4 || (K == 8 && bf16))) return true;
+  typedef PipeTileW<K> TW;
+  typedef RBTile<K> TR;
+  const int64_t tw = (g->ny + TW::th - 1) / TW::th, tr = (g->ny + TR::th - 1) / TR::th;
+  return tw * ((g->nx + TW::tw - 1) / TW::tw) <= num_sms() || 0.85 * (double)(tw * TW::th) <= (double)(tr * TR::th);
+}
+
 template <int K>
 static int launch_apply_rb_w(const bf_graph* g, const ApplyArgs<float>& a, cudaStream_t s) {
   if (a.op == BF_OP_L && !a.scale && ((uintptr_t)a.X & 15) == 0 && ((uintptr_t)a.Y & 15) == 0 && a.ldx % 4 == 0 &&
       a.ldy % 4 == 0) {
     // (the stored kernel's byte offsets are 32-bit)
-    if (g->p.weight_mode == BF_W_STORED_F32 && g->n < BF_PIPE_W_MAX_N) return launch_apply_pipe_w<K, BF_W_STORED_F32>(g, a, s);
-    if (g->p.weight_mode == BF_W_STORED_BF16 && g->n < BF_PIPE_W_MAX_N) return launch_apply_pipe_w<K, BF_W_STORED_BF16>(g, a, s);
+    if (g->p.weight_mode != BF_W_ONTHEFLY && g->n < BF_PIPE_W_MAX_N && pipe_w_pays<K>(g)) {
+      if (g->p.weight_mode == BF_W_STORED_F32) return launch_apply_pipe_w<K, BF_W_STORED_F32>(g, a, s);
+      return launch_apply_pipe_w<K, BF_W_STORED_BF16>(g, a, s);
+    }
     if (g->p.weight_mode == BF_W_ONTHEFLY && g->gf.a_r > 0.0f) return launch_apply_pipe<K>(g, a, s);
   }
   if (g->p.weight_mode == BF_W_ONTHEFLY) return launch_apply_rb<K, false>(g, a, s);
@@ -1071,13 +1095,24 @@ static int apply_fast_shape(const bf_graph* g, int K, const ApplyArgs<float>& a,
   return 0;
 }
 
+// Whether one column with weights on the fly goes by runs (tiles of 64 x 16) rather than with one
+// pixel per thread (32 x 8, rows outside the image cost nothing).  2.4 million pixels, runs
+// against pixels: L one row 386 and 145 us, five 95 and 84, six 83 and 82, eight 68 and 78; D^-1 W
+// six rows 94 and 82, eight 76 and 80; D^-1 W of 6 columns (rows that are not whole vectors) 364
+// and 343.  The limit of the other kernel's grid stays on the runs' side.
+static bool run_pays(const bf_graph* g, int op) {
+  if ((g->ny + BF_TH2 - 1) / BF_TH2 > 65535) return true;
+  return g->ny > 6 && !(op == BF_OP_DINV_W && g->nx < 12 && g->nx % 4 != 0);
+}
+
 static int try_apply_fast(const bf_graph* g, int K, const ApplyArgs<float>& a, cudaStream_t s, int* rc) {
   if (!(a.op == BF_OP_L || a.op == BF_OP_NSYM || a.op == BF_OP_NDIAGL || a.op == BF_OP_DINV_W)) return 0;
-  if (fast_shape(g) == FAST_R3_2D && K == 1 && a.op != BF_OP_DINV_W) {
+  const bool otf = g->p.weight_mode == BF_W_ONTHEFLY;
+  if (fast_shape(g) == FAST_R3_2D && K == 1 && a.op != BF_OP_DINV_W && (!otf || run_pays(g, a.op))) {
     *rc = launch_apply1_w(g, a, s);
     return 1;
   }
-  if (fast_shape(g) == FAST_R3_2D && K == 1 && g->p.weight_mode == BF_W_ONTHEFLY) {
+  if (fast_shape(g) == FAST_R3_2D && K == 1 && otf && run_pays(g, a.op)) {
     *rc = launch_apply1_run<false, true>(g, a, s);
     return 1;
   }
@@ -1306,7 +1341,7 @@ extern "C" int bf_weights(const bf_params* p, const void* guide, bf_graph** out,
 static int launch_weights(bf_graph* g, const void* guide, cudaStream_t s) {
   if (g->kind == BF_KIND_GUIDED) return bf_guided_prep(g, guide, s);
   cudaError_t e;
-  if (fast_shape(g) == FAST_R3_2D && g->p.weight_mode == BF_W_ONTHEFLY) {
+  if (fast_shape(g) == FAST_R3_2D && g->p.weight_mode == BF_W_ONTHEFLY && g->nx >= 12 && g->ny >= 4) {
     static int per_sm = 0;
     if (per_sm == 0) {
       int v = 0;
