@@ -816,7 +816,7 @@ __global__ void __launch_bounds__(CGP_T, 1) k_cgp_image(const __grid_constant__ 
 // pairs (i, i + t), t = 1 .. R, i from R samples before its piece to its end, so that an
 // iteration has no exponentials (in FP64 they were 9/10 of the arithmetic at 2 FMA per clock
 // and SM).  Generic recurrences: r and s = T r are both kept.  4096 samples, FP64, 11 taps, 20
-// iterations: 157 us (two launches per iteration on 16 CTAs: 725).
+// iterations: 160 us (two launches per iteration on 16 CTAs: 725).
 template <typename T>
 struct CgpLine {
   CgArgs<T> cg;
@@ -1018,36 +1018,48 @@ int cgp_max_ctas() {
 }
 
 // The rectangle split of an image with the fewest units of 32 x 4 pixels per scheduler, then
-// the smallest halo; false: the image does not fit.
+// the smallest halo; false: the image does not fit.  Where one unit per scheduler is enough,
+// rectangles of four units (32 x 16) do the same on a quarter of the CTAs: they leave the others
+// to runs on other streams and have shorter all-reduces.  30 steps of 128 x 128 pixels: 172 us
+// (192 with 128 CTAs of one unit); on 8 streams 44 us a run (186; 111 to 147 with two launches
+// per iteration, which overlap).  Fewer than 17 CTAs stay as they are (32 x 32, guided, radius 3:
+// 251 us against 257), and larger rectangles have no such choice: 256 x 256 pixels take 128 CTAs
+// and run one after the other (189 us each; 122 to 147 on 8 streams with two launches).
 template <class OP>
 bool cgp_rect(int nx, int ny, CgpRect* out, int* nreg) {
   const int maxc = cgp_max_ctas();
   long best = -1;
+  auto take = [&](int W, int H, long cost) {
+    best = cost;
+    out->W = W;
+    out->H = H;
+    out->ncx = (nx + W - 1) / W;
+    *nreg = out->ncx * ((ny + H - 1) / H);
+  };
   for (int W = 32; W <= 256; W += 32) {
     const int ncx = (nx + W - 1) / W;
     if (ncx > maxc) continue;
     const int want = std::min(maxc / ncx, (ny + 3) / 4);
-    const int H = 4 * ((ny + 4 * want - 1) / (4 * want)), ncy = (ny + H - 1) / H;
+    const int H = 4 * ((ny + 4 * want - 1) / (4 * want));
     const int nhalo = 2 * OP::HALO * (W + 2 * OP::HALO) + 2 * OP::HALO * H;
     if (cgp_image_floats<OP>(W, H) * 4 > CGP_SMEM_MAX || nhalo > CGP_HALO_REGS * CGP_T) continue;
     const long cost = (long)((W / 32 * (H / 4) + 3) / 4) * 100000 + nhalo;
-    if (best < 0 || cost < best) {
-      best = cost;
-      out->W = W;
-      out->H = H;
-      out->ncx = ncx;
-      *nreg = ncx * ncy;
-    }
+    if (best < 0 || cost < best) take(W, H, cost);
   }
+  const int four = ((nx + 31) / 32) * ((ny + 15) / 16);
+  if (best >= 0 && best < 200000 && *nreg > 16 && 2 * four <= *nreg) take(32, 16, best);
   return best >= 0;
 }
 
-// Samples per CTA of a signal: at least 128 (4096 samples in FP64, 20 steps: 157 us; 256: 185),
-// 0 if it does not fit.
+// Samples per CTA of a signal: at least 128 (4096 samples in FP64, 20 steps: 160 us; 256: 185),
+// 0 if it does not fit.  FP32 runs that would take more than half of the SMs so and not with 256
+// samples leave them to runs on other streams where it costs nothing (30 steps of 15000, radius 5:
+// 133 us either way, on 8 streams 31 us a run against 75; radius 20: 146 us against 139).
 int cgp_line_width(const bf_graph* g) {
   const int maxc = cgp_max_ctas();
   if (maxc < 1) return 0;
-  int64_t W = std::max<int64_t>(128, (g->n + maxc - 1) / maxc);
+  const bool half = g->esize == 4 && g->rx <= 8 && g->n > 64 * (int64_t)maxc && g->n <= 128 * (int64_t)maxc;
+  int64_t W = std::max<int64_t>(half ? 256 : 128, (g->n + maxc - 1) / maxc);
   W = std::max<int64_t>((W + 31) / 32 * 32, 2 * g->rx);
   return cgp_line_elems((int)std::min<int64_t>(W, 1 << 20), g->rx) * g->esize > CGP_SMEM_MAX ? 0 : (int)W;
 }

@@ -142,3 +142,56 @@ def test_images_beyond_the_chip(shape):
     out = torch.empty_like(wide)[1:]
     bf().cg_filter(G, wide[1:], 6, out=out)
     assert rel_l2(host(out), host(bf().cg_filter(G64, x0.double(), 6)[0])) < TOL_F32
+
+
+@pytest.mark.parametrize("kind,shape", [("image", (64, 64)), ("image", (63, 97)), ("image", (128, 128)), ("image", (130, 161)),
+                                        ("guided", (128, 128)), ("signal", (9472,)), ("signal", (9473,)), ("signal", (18944,)),
+                                        ("signal", (18945,))])
+def test_splits_that_leave_room_for_other_streams(kind, shape):
+    """Small images by rectangles of four units and mid-length signals by pieces of 256 samples:
+    either side of the lines where those splits are taken, alone and four at a time."""
+    n = int(np.prod(shape))
+    if kind == "signal":
+        x0 = _signal(n, torch.float32)
+        G = [bf().bf_weights(x0, 5, 3.0, 0.1) for _ in range(4)]
+        O = Graph(host(x0), (1, n), 5, 3.0, 0.1)
+    else:
+        from oracle.guided import GuidedGraph
+        g = torch.as_tensor(synth.polygon_image(*shape, seed=7, polygons=6)[1].astype(np.float32), device="cuda")
+        x0 = g.reshape(-1).clone()
+        G = [bf().guided_graph(g, 2, 0.01) if kind == "guided" else bf().bf_weights(g, 3, 2.0, 0.08) for _ in range(4)]
+        O = (GuidedGraph(host(g), shape, 2, 0.01) if kind == "guided" else Graph(host(g), shape, 3, 2.0, 0.08))
+    ref = solvers.cg(O, host(x0).reshape(-1), 12, shift=0.2)["x"]
+    x, info, _ = bf().cg_filter(G[0], x0, 12, shift=0.2)
+    assert info.iters == 12 and rel_l2(host(x), ref) < TOL_F32
+    streams = [torch.cuda.Stream() for _ in G]
+    outs = [torch.empty_like(x0) for _ in G]
+    torch.cuda.synchronize()
+    for _ in range(3):
+        for H, o, s in zip(G, outs, streams):
+            bf().cg_filter(H, x0, 12, shift=0.2, out=o, sync=False, stream=s)
+    torch.cuda.synchronize()
+    for o in outs:
+        assert torch.equal(o, x)
+
+
+def test_small_runs_on_eight_streams_overlap():
+    """Eight runs on eight streams take far less than eight runs (they would one after the other)."""
+    import time
+    g = torch.as_tensor(synth.polygon_image(128, 128, seed=8, polygons=6)[1].astype(np.float32), device="cuda")
+    x0 = g.reshape(-1)
+    G = [bf().bf_weights(g, 3, 2.0, 0.08) for _ in range(8)]
+    streams, outs = [torch.cuda.Stream() for _ in G], [torch.empty_like(x0) for _ in G]
+
+    def run(k):
+        times = []
+        for _ in range(7):
+            torch.cuda.synchronize()
+            t = time.perf_counter()
+            for i in range(k):
+                bf().cg_filter(G[i], x0, 300, shift=0.01, out=outs[i], sync=False, stream=streams[i])
+            torch.cuda.synchronize()
+            times.append(time.perf_counter() - t)
+        return sorted(times)[3]
+
+    assert run(8) < 5.0 * run(1)
