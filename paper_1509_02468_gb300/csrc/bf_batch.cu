@@ -1107,7 +1107,7 @@ extern "C" int bf_batch_lobpcg(bf_batch* b, const float* const* X0, int k, int k
 }
 
 // Autotune the image class's tile shape: time `iters` CG iterations of the batch with each
-// candidate (32 x 8, 64 x 4, 16 x 16) on the given vectors and keep the fastest.
+// candidate (64 x 16, 32 x 32, 128 x 8) on the given vectors and keep the fastest.
 extern "C" int bf_batch_tune(bf_batch* b, const float* const* x0, float* const* x_out, int iters,
                              float* ms_out, void* stream) {
   if (!b || !x0 || !x_out) return bf_fail(BF_EINVAL, "bf_batch_tune: NULL argument");

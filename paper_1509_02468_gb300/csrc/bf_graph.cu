@@ -738,15 +738,13 @@ __global__ void __launch_bounds__(PipeTile<K>::threads + PIPE_STAGERS, 1) k_appl
 }
 
 // ---- the same walk with STORED weights (modes FP32 and BF16): the weights between a strip's
-// four pixels and a halo pixel are loaded from the planes of wf a few halo pixels ahead of
-// their use.  A warp's load of one tap is 32 consecutive weights; a forward weight plane is
+// pixels and a halo pixel are loaded from the planes of wf a few halo pixels ahead of their
+// use (eight with 16 columns a thread, five with fewer, two in tiles at the border).  A warp's load of one tap is 32 consecutive weights; a forward weight plane is
 // read once by the pixel and once, as the backward tap, by the neighbour (an L1 or L2 hit).
 // Bound by the FP32 pipe (2 K lane operations per pixel and neighbour) and the weights'
 // bytes.  (k_apply_rb, which loads each weight where it is used, stood on their latency:
 // 1024 x 1024, K = 16, BF16: 470 us.)
-// The weight at byte offset `off` of the planes; volatile, so that the loads of a row stay
-// where they are issued.
-// Its tile: 12 computing warps (128 registers a thread with the two that copy), strips of two
+// The tile: 12 computing warps (128 registers a thread with the two that copy), strips of two
 // pixels where a thread carries 16 columns: with four, the loads could only be issued two
 // steps ahead, 0.1 us before use, and the kernel waited for them (216 us; 140 us so).
 template <int K>
@@ -766,6 +764,8 @@ struct PipeTileW {
   static constexpr size_t smem = 2 * stage;
 };
 
+// The weight at byte offset `off` of the planes; volatile, so that the loads of a row stay
+// where they are issued.
 template <int WM>
 __device__ __forceinline__ float pipe_ld_w(const char* wf, unsigned off) {
   if (WM == BF_W_STORED_BF16) {
@@ -779,10 +779,10 @@ __device__ __forceinline__ float pipe_ld_w(const char* wf, unsigned off) {
 }
 
 // Weights between the halo pixel (row r of the strip's rows, column x + dx) and the strip's
-// pixels (column x, rows y0 ..; off: byte offset of pixel (x, y0) in a plane).  MASK: 0 unless
+// pixels (column x, rows y0 ..; base: byte offset of pixel (x, y0) in plane F0, see bf_index.h).  MASK: 0 unless
 // pixel and neighbour lie in the image (nothing else is read then).
-template <int WM, bool MASK, int P>
-__device__ __forceinline__ void pipe_step_w(const void* wf, int n, int nx, int ny, int x, int y0, unsigned off, int r,
+template <int WM, bool MASK, int P, int F0>
+__device__ __forceinline__ void pipe_step_w(const void* wf, int n, int nx, int ny, int x, int y0, unsigned base, int r,
                                             int dx, float (&w)[P]) {
   constexpr int ES = WM == BF_W_STORED_BF16 ? 2 : 4;
   // opaque: the offsets of a strip's 192 loads would be kept for all its steps, and spilled
@@ -793,28 +793,28 @@ __device__ __forceinline__ void pipe_step_w(const void* wf, int n, int nx, int n
     if (dy < -3 || dy > 3 || (dy == 0 && dx == 0)) continue;
     const bool fwd = dy > 0 || (dy == 0 && dx > 0);
     const int f = fwd ? ShapeR3::fwd_index(dy, dx) : ShapeR3::fwd_index(-dy, -dx);
-    const int e = f * n + p * nx + (fwd ? 0 : dy * nx + dx);
+    const int e = (f - F0) * n + p * nx + (fwd ? 0 : dy * nx + dx);
     bool in = true;
     if (MASK)
       in = x < nx && y0 + p < ny && (unsigned)(x + dx) < (unsigned)nx && (unsigned)(y0 + p + dy) < (unsigned)ny;
-    w[p] = in ? pipe_ld_w<WM>((const char*)wf, off + bf_byte_offset(e, ES)) : 0.0f;
+    w[p] = in ? pipe_ld_w<WM>((const char*)wf, bf_tap_offset(base, e, ES)) : 0.0f;
   }
 }
 
-template <int K, int WM, bool MASK>
+template <int K, int WM, bool MASK, int F0>
 __device__ __forceinline__ void pipe_tile_w(const Geom<float>& g, const ApplyArgs<float>& a, const float4* sx, int bx,
                                             int by, int lx, int grp, int row0) {
   typedef PipeTileW<K> TT;
   constexpr int CS = TT::cs, CS4 = CS / 4, P = TT::P;
   const int x = bx + lx, y0 = by + row0;
   const int n = (int)a.n, nx = g.nx;
-  const unsigned off = (unsigned)(y0 * nx + x) * (WM == BF_W_STORED_BF16 ? 2u : 4u);
+  const unsigned base = bf_base_offset((unsigned)(y0 * nx + x), F0, (unsigned)n, WM == BF_W_STORED_BF16 ? 2u : 4u);
   unsigned long long acc2[P][CS / 2], xi2[P][CS / 2];
   // steps (row, dx) in order, the weights loaded AHEAD steps before they are used
   constexpr int AHEAD = MASK ? 2 : TT::AHEAD, RING = AHEAD + 1, STEPS = 7 * (P + 6);
   float w[RING][P];
 #pragma unroll
-  for (int q = 0; q < AHEAD; ++q) pipe_step_w<WM, MASK, P>(a.wf, n, nx, g.ny, x, y0, off, q / 7, q % 7 - 3, w[q]);
+  for (int q = 0; q < AHEAD; ++q) pipe_step_w<WM, MASK, P, F0>(a.wf, n, nx, g.ny, x, y0, base, q / 7, q % 7 - 3, w[q]);
 #pragma unroll
   for (int p = 0; p < P; ++p) {
     const int hp = (row0 + p + 3) * TT::hw + lx + 3;
@@ -833,7 +833,7 @@ __device__ __forceinline__ void pipe_tile_w(const Geom<float>& g, const ApplyArg
   for (int dx = -3; dx <= 3; ++dx) {
     const int q = 7 * r + dx + 3;
     if (q + AHEAD < STEPS)
-      pipe_step_w<WM, MASK, P>(a.wf, n, nx, g.ny, x, y0, off, (q + AHEAD) / 7, (q + AHEAD) % 7 - 3, w[(q + AHEAD) % RING]);
+      pipe_step_w<WM, MASK, P, F0>(a.wf, n, nx, g.ny, x, y0, base, (q + AHEAD) / 7, (q + AHEAD) % 7 - 3, w[(q + AHEAD) % RING]);
     const int hp = (row0 + r) * TT::hw + lx + 3 + dx;
     unsigned long long xj2[CS / 2];
 #pragma unroll
@@ -862,7 +862,7 @@ __device__ __forceinline__ void pipe_tile_w(const Geom<float>& g, const ApplyArg
   }
 }
 
-template <int K, int WM>
+template <int K, int WM, int F0>
 __global__ void __launch_bounds__(PipeTileW<K>::threads + PIPE_STAGERS, 1)
 k_apply_pipe_w(const __grid_constant__ Geom<float> g, const ApplyArgs<float> a) {
   bf_pdl_enter();
@@ -890,9 +890,9 @@ k_apply_pipe_w(const __grid_constant__ Geom<float> g, const ApplyArgs<float> a) 
     const float4* sx = reinterpret_cast<const float4*>(smem + b * TT::stage);
     const int bx = (t % ntx) * TT::tw, by = (t / ntx) * TT::th;
     if (bx >= 3 && bx + TT::tw + 3 <= g.nx && by >= 3 && by + TT::th + 3 <= g.ny)
-      pipe_tile_w<K, WM, false>(g, a, sx, bx, by, lx, grp, row0);
+      pipe_tile_w<K, WM, false, F0>(g, a, sx, bx, by, lx, grp, row0);
     else
-      pipe_tile_w<K, WM, true>(g, a, sx, bx, by, lx, grp, row0);
+      pipe_tile_w<K, WM, true, F0>(g, a, sx, bx, by, lx, grp, row0);
   }
 }
 
@@ -921,17 +921,17 @@ static int launch_apply_pipe(const bf_graph* g, const ApplyArgs<float>& a, cudaS
   return BF_OK;
 }
 
-template <int K, int WM>
+template <int K, int WM, int F0>
 static int launch_apply_pipe_w(const bf_graph* g, const ApplyArgs<float>& a, cudaStream_t s) {
   typedef PipeTileW<K> TT;
   static_assert(TT::smem <= 227 * 1024, "stored-weight apply tile does not fit in shared memory");
   {
-    const int rc_ = bf_smem_attr((const void*)k_apply_pipe_w<K, WM>, (int)TT::smem, "cudaFuncSetAttribute(k_apply_pipe_w)");
+    const int rc_ = bf_smem_attr((const void*)k_apply_pipe_w<K, WM, F0>, (int)TT::smem, "cudaFuncSetAttribute(k_apply_pipe_w)");
     if (rc_) return rc_;
   }
   const int64_t ntiles = ((g->nx + TT::tw - 1) / TT::tw) * (int64_t)((g->ny + TT::th - 1) / TT::th);
   const int grid = (int)std::min<int64_t>(ntiles, num_sms());
-  BF_LAUNCH_PDL((k_apply_pipe_w<K, WM>), grid, TT::threads + PIPE_STAGERS, TT::smem, s, g->gf, a);
+  BF_LAUNCH_PDL((k_apply_pipe_w<K, WM, F0>), grid, TT::threads + PIPE_STAGERS, TT::smem, s, g->gf, a);
   BF_CUDA(cudaGetLastError());
   return BF_OK;
 }
@@ -973,10 +973,14 @@ template <int K>
 static int launch_apply_rb_w(const bf_graph* g, const ApplyArgs<float>& a, cudaStream_t s) {
   if (a.op == BF_OP_L && !a.scale && ((uintptr_t)a.X & 15) == 0 && ((uintptr_t)a.Y & 15) == 0 && a.ldx % 4 == 0 &&
       a.ldy % 4 == 0) {
-    // (the stored kernel's byte offsets are 32-bit)
-    if (g->p.weight_mode != BF_W_ONTHEFLY && g->n < BF_PIPE_W_MAX_N && pipe_w_pays<K>(g)) {
-      if (g->p.weight_mode == BF_W_STORED_F32) return launch_apply_pipe_w<K, BF_W_STORED_F32>(g, a, s);
-      return launch_apply_pipe_w<K, BF_W_STORED_BF16>(g, a, s);
+    if (g->p.weight_mode == BF_W_STORED_BF16 && pipe_w_pays<K>(g) && bf_tap_offset_fits(g->n, g->nx, 0, 2))
+      return launch_apply_pipe_w<K, BF_W_STORED_BF16, 0>(g, a, s);
+    if (g->p.weight_mode == BF_W_STORED_F32 && pipe_w_pays<K>(g)) {
+      // counted from the first plane, 8 and 16 columns are faster (2048 x 2048: 214 us against 220, 369
+      // against 380), 4 and 32 are not (153 against 150, 786 against 748)
+      if constexpr (K == 8 || K == 16)
+        if (bf_tap_offset_fits(g->n, g->nx, 0, 4)) return launch_apply_pipe_w<K, BF_W_STORED_F32, 0>(g, a, s);
+      if (bf_tap_offset_fits(g->n, g->nx, 12, 4)) return launch_apply_pipe_w<K, BF_W_STORED_F32, 12>(g, a, s);
     }
     if (g->p.weight_mode == BF_W_ONTHEFLY && g->gf.a_r > 0.0f) return launch_apply_pipe<K>(g, a, s);
   }

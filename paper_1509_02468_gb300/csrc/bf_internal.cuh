@@ -39,8 +39,9 @@ void bf_count_launches(int n);
     bf_count_launches(1);       \
   } while (0)
 
-// Programmatic dependent launch for the kernels of the block-LOBPCG iteration chain: a
-// kernel launched by BF_LAUNCH_PDL may be scheduled while its predecessor in the stream
+// Programmatic dependent launch for kernels that follow one another in a stream (the iteration
+// chains of block LOBPCG and of CG on images beyond the chip, the operator, graph updates, the
+// layers of the net): a kernel launched by BF_LAUNCH_PDL may be scheduled while its predecessor in the stream
 // still runs, once every CTA of the predecessor has called bf_pdl_enter (or exited); it
 // must itself call bf_pdl_enter before touching anything the predecessor writes, since
 // the wait in it returns only when the predecessor grid has completed and its memory

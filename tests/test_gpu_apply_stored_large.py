@@ -10,14 +10,15 @@ from tests.gpu_helpers import bf
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("mode,shape", [("stored_f32", (4801, 5003)), ("stored_f32", (6631, 6635)),
+@pytest.mark.parametrize("mode,shape", [("stored_f32", (4701, 4703)), ("stored_f32", (4801, 5003)), ("stored_f32", (6631, 6635)),
                                         ("stored_bf16", (6631, 6635)), ("stored_f32", (6636, 6632))])
-def test_against_one_column(mode, shape):
+@pytest.mark.parametrize("k", [4, 8, 16])
+def test_against_one_column(mode, shape, k):
     gen = torch.Generator(device="cuda").manual_seed(1)
     g = torch.rand(shape, device="cuda", generator=gen)
     G = bf().bf_weights(g, 3, 2.0, 0.5, weight_mode=mode)
-    X = torch.rand((G.n, 4), device="cuda", generator=gen)
+    X = torch.rand((G.n, k), device="cuda", generator=gen)
     Y = bf().bf_apply(G, "L", X)
-    for c in range(4):
+    for c in (0, k // 2, k - 1):
         y = bf().bf_apply(G, "L", X[:, c].contiguous())
         assert (Y[:, c] - y).abs().max().item() <= 2.7e-4

@@ -10,17 +10,31 @@ CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
 
 SOURCE = """
 #include "bf_index.h"
-// first byte of the weight of tap plane f, `shift` samples from pixel i, by both routes
-constexpr bool right(long long n, long long i, int f, int shift, int es) {
-  const int e = f * (int)n + shift;
-  return (unsigned)i * (unsigned)es + bf_byte_offset(e, es) == (unsigned long long)((f * n + i + shift) * es);
+// weight of plane f, `shift` samples from pixel i: both routes
+constexpr bool right(long long n, long long i, int f0, int f, long long shift, int es) {
+  return bf_tap_offset(bf_base_offset((unsigned)i, (unsigned)f0, (unsigned)n, (unsigned)es),
+                       (f - f0) * (int)n + (int)shift, es) ==
+         (unsigned long long)((f * n + i + shift) * es);
 }
-constexpr long long N = BF_PIPE_W_MAX_N - 1;
-static_assert(24 * N * 4 <= 0xffffffffll && 24 * N <= 0x7fffffff, "range of the arithmetic");
-static_assert(right(N, N - 1, 23, 0, 4) && right(N, N - 1, 23, -30001, 4) && right(N, N - 1, 0, -30001, 4), "last pixel");
-static_assert(right(N, 30001, 0, -30001, 4) && right(N, 0, 23, 0, 4) && right(N, 0, 0, 0, 4), "first pixels");
-static_assert(right(N, N / 2, 12, -7, 4) && right(N, N / 2, 13, -7, 2) && right(N, N - 1, 23, -3, 2), "between");
-static_assert(right(23400000, 23399999, 23, 0, 4) && right(23300000, 23299999, 23, 0, 4), "either side of 2^31 bytes");
+// every plane, from the first and the last pixel: 3 rows and columns back where that lies in the
+// planes; and the strip's pixels past the image, which are not read
+constexpr bool ends(long long n, long long nx, int f0, int es) {
+  if (!bf_tap_offset_fits(n, nx, f0, es)) return false;
+  for (int f = 0; f < 24; ++f) {
+    if (!right(n, n - 1, f0, f, 0, es) || !right(n, 0, f0, f, 0, es)) return false;
+    if (3 * nx + 3 < n && (!right(n, n - 1, f0, f, -3 * nx - 3, es) || !right(n, 3 * nx + 3, f0, f, -3 * nx - 3, es)))
+      return false;
+    if (bf_tap_offset(0, (f - f0) * (int)n + (int)(6 * nx + 3), es) == 1) return false;
+  }
+  return true;
+}
+static_assert(ends(43999999, 1000, 12, 4) && ends(43999999, 1400000, 12, 4) && ends(43997000, 6635, 12, 4), "largest FP32");
+static_assert(ends(22300000, 5000, 0, 4) && ends(22300000, 5000, 12, 4) && ends(23400000, 5000, 12, 4), "around 2^31 bytes");
+static_assert(ends(43999999, 9000, 0, 2) && ends(43999999, 2900000, 0, 2) && ends(43999999, 43000000, 12, 2), "largest BF16");
+static_assert(ends(49, 7, 0, 4) && ends(400, 100, 12, 2), "small");
+static_assert(!bf_tap_offset_fits(44000000, 1000, 12, 4) && !bf_tap_offset_fits(43999999, 1500000, 12, 4), "refused");
+static_assert(!bf_tap_offset_fits(44000000, 1000, 12, 2) && !bf_tap_offset_fits(1ll << 33, 1 << 16, 12, 2), "refused");
+static_assert(!bf_tap_offset_fits(22400000, 5000, 0, 4), "refused from the first plane");
 int main() { return 0; }
 """
 
