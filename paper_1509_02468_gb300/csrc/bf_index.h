@@ -7,6 +7,13 @@
 #define BF_HD
 #endif
 
+// Integer that orders doubles (by their bits) as their values do, NaNs before all others: ranks by
+// it, ties by place, are a permutation whatever the values are.
+BF_HD constexpr long long bf_order_key(long long bits) {
+  const long long mag = bits & 0x7fffffffffffffffll;
+  return mag > 0x7ff0000000000000ll ? -0x7fffffffffffffffll : (bits < 0 ? -mag : mag);
+}
+
 // Byte offsets of the stored-weight walk: 24 planes of n weights of es bytes, rows of nx.  A
 // weight is addressed from its pixel's place in plane f0 (unsigned bytes from the first plane on)
 // by a signed number of weights, whose product with es stays within an int; the sum is taken

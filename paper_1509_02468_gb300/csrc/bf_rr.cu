@@ -30,6 +30,7 @@
 #include <math.h>
 
 #include "bf_internal.cuh"
+#include "bf_index.h"
 #include "bf_rr.cuh"
 
 #define RR_T 512
@@ -1016,12 +1017,13 @@ __global__ void __launch_bounds__(RR_T) k_rr(const RRParams a) {
       if (nrot == 0) break;
     }
   }
-  for (int i = tid; i < kk; i += RR_T) {             // ascending order of the kk values
-    const double li = H[i * RR_KLD + i];
+  // ascending order of the kk values (a NaN comes first, and is reported below)
+  for (int i = tid; i < kk; i += RR_T) {
+    const long long li = bf_order_key(__double_as_longlong(H[i * RR_KLD + i]));
     int rank = 0;
     for (int j = 0; j < kk; ++j) {
-      const double lj = H[j * RR_KLD + j];
-      rank += (lj < li) || (lj == li && j < i);
+      const long long lj = bf_order_key(__double_as_longlong(H[j * RR_KLD + j]));
+      rank += lj < li || (lj == li && j < i);
     }
     perm[rank] = i;
   }

@@ -45,3 +45,44 @@ def test_stored_weight_offsets(tmp_path):
     src.write_text(SOURCE)
     r = subprocess.run(["g++", "-std=c++17", "-fsyntax-only", "-I", CSRC, str(src)], capture_output=True, text=True)
     assert r.returncode == 0, r.stderr
+
+
+ORDER = """
+#include <cmath>
+#include <cstring>
+#include "bf_index.h"
+long long key(double v) {
+  long long b;
+  std::memcpy(&b, &v, 8);
+  return bf_order_key(b);
+}
+bool before(double a, int i, double b, int j) { return key(a) < key(b) || (key(a) == key(b) && i < j); }
+bool permutation(const double* v, int n) {       // ranks 0 .. n - 1, each taken once
+  unsigned seen = 0;
+  for (int i = 0; i < n; ++i) {
+    int rank = 0;
+    for (int j = 0; j < n; ++j) rank += before(v[j], j, v[i], i);
+    seen |= 1u << rank;
+  }
+  return seen == (1u << n) - 1;
+}
+int main() {
+  const double x = std::nan(""), inf = INFINITY;
+  const double a[8] = {3, 1, 2, 1, -inf, inf, 0, -0.0}, b[8] = {x, 1, x, 0, 2, x, inf, 1}, c[3] = {x, x, x}, d[2] = {1, x};
+  if (!permutation(a, 8) || !permutation(b, 8) || !permutation(c, 3) || !permutation(d, 2)) return 1;
+  const double up[] = {-x, -inf, -2, -1, -1e-310, 0, 1e-320, 1, 1.5, 1e300, inf};      // by value
+  for (int i = 0; i + 1 < 11; ++i)
+    if (!before(up[i], 9, up[i + 1], 1) || before(up[i + 1], 1, up[i], 9)) return 2;
+  return key(0.0) == key(-0.0) ? 0 : 3;
+}
+"""
+
+
+@pytest.mark.skipif(shutil.which("g++") is None, reason="no host compiler")
+def test_ritz_value_order_is_a_permutation(tmp_path):
+    """The Ritz values' ranks index the vectors: they must be a permutation with NaNs among them
+    too (places that no rank names would be read uninitialised)."""
+    src, exe = tmp_path / "order.cpp", tmp_path / "order"
+    src.write_text(ORDER)
+    subprocess.run(["g++", "-std=c++17", "-I", CSRC, "-o", str(exe), str(src)], check=True, capture_output=True)
+    assert subprocess.run([str(exe)]).returncode == 0
